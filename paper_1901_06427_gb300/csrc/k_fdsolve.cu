@@ -102,21 +102,27 @@ void axis_basis(AxisKind kind, int m, std::vector<double>& Q, std::vector<double
   }
 }
 
-// max |T Q - Q diag(lam)| and max |Q^T Q - I|
+// |T Q - Q diag(lam)| and the columns' norms, and the products of
+// neighbouring columns.  T is symmetric with distinct eigenvalues but for
+// the cos / sin pairs of a periodic axis, which are neighbours, so columns
+// that pass are orthonormal.
 bool basis_ok(AxisKind kind, int m, const std::vector<double>& Q, const std::vector<double>& lam) {
-  std::vector<double> T;
+  std::vector<double> T, norm(m, 0.0), next(m, 0.0);
   axis_matrix(kind, m, T);
   double e1 = 0.0, e2 = 0.0;
   for (int i = 0; i < m; ++i)
     for (int k = 0; k < m; ++k) {
-      double r = -Q[(size_t)i * m + k] * lam[k], o = (i == k) ? -1.0 : 0.0;
-      for (int j = 0; j < m; ++j) {
+      double r = -Q[(size_t)i * m + k] * lam[k];
+      for (int o = -1; o <= 1; ++o) {
+        const int j = (i + o + m) % m;
+        if (o != 0 && (j == i || (m == 2 && o > 0))) continue;   // one or two points: each neighbour once
         r += T[(size_t)i * m + j] * Q[(size_t)j * m + k];
-        o += Q[(size_t)j * m + i] * Q[(size_t)j * m + k];
       }
       e1 = std::fmax(e1, std::fabs(r));
-      e2 = std::fmax(e2, std::fabs(o));
+      norm[k] += Q[(size_t)i * m + k] * Q[(size_t)i * m + k];
+      if (k + 1 < m) next[k] += Q[(size_t)i * m + k] * Q[(size_t)i * m + k + 1];
     }
+  for (int k = 0; k < m; ++k) e2 = std::fmax(e2, std::fmax(std::fabs(norm[k] - 1.0), std::fabs(next[k])));
   return e1 <= 1e-12 * 4.0 * m && e2 <= 1e-13 * m;
 }
 
@@ -420,12 +426,11 @@ __global__ void __launch_bounds__(256) k_fdw_z(FDParams P, float* __restrict__ d
   fd_item<fd_col_tiles>(P, tile, gi);
   const FDGrid& G = P.g[gi];
   const int e0 = G.e[0], e1 = G.e[1], e2 = G.e[2], pl = e0 * e1;
-  const int p0 = fd_pad(e0), p1 = fd_pad(e1), p2 = fd_pad(e2);
-  const float* L0 = P.tab + G.tab0 + 2 * e0 * p0;
-  const float* L1 = L0 + p0 + 2 * e1 * p1;
-  const float* Q2 = L1 + p1;
-  const float* QT2 = Q2 + e2 * p2;
-  const float* L2 = QT2 + e2 * p2;
+  const float* L0 = P.tab + G.lam[0];
+  const float* L1 = P.tab + G.lam[1];
+  const float* Q2 = P.tab + G.q2;
+  const float* QT2 = P.tab + G.qt2;
+  const float* L2 = P.tab + G.lam[2];
   fdw_stage_basis(Mz, Q2, e2);
   fdw_stage_basis(MzT, QT2, e2);
   const int col0 = tile * 32;
@@ -473,10 +478,289 @@ __global__ void __launch_bounds__(256) k_fdw_z(FDParams P, float* __restrict__ d
   }
 }
 
-}  // namespace
+// ------------------------------------------------------------------------
+// Long lines: levels with an axis of more than kFDLine points.  Each axis is
+// one pass over the level, a batch of small products line x basis, tiled as
+// matrix products over the whole GPU (x, y, z forward, then z, y, x back; a
+// z axis of at most kFDLine points takes k_fdw_z instead of its two passes).
+//
+// The eigenvectors of every axis kind but the mixed free-slip / no-slip ones
+// are even or odd under the mirror j -> m - 1 - j (periodic axes: j -> -j),
+// so a line is folded into sums and differences of mirrored points and the
+// even and odd eigenvectors each see half of it: half the products of the
+// plain basis.  Pair p of an axis joins points a and b (a == b: its own
+// mirror, no odd part).
+//
+// Bound by the FP32 pipe and by latency on small levels.  It takes the place
+// of the V-cycles above a short-line level (28 launches at their launch floor
+// on the 384 x 96 x 12 channel, whose flat levels point smoothing treats
+// badly): driven monolayer step 299 -> 177 ms (704 -> 399 iterations),
+// 128 x 128 x 64 gradient 365 -> 104 ms (about 600 -> 230), boomerang slit
+// step 18.4 -> 14.0 ms.
+RBFIB_DEVFN void fold_pair(const FDAxis& X, int p, int& a, int& b) {
+  a = p;
+  b = X.fold == kFoldMirror ? X.e - 1 - p : (X.fold == kFoldPeriodic && p > 0 ? X.e - p : p);
+}
 
-// Whole-GPU form of fd_solve: tmp holds the level's transformed coefficients
-// (as many floats as u).
+// Shape of a pass: 128 threads, 64 entries along the contiguous dimension of
+// memory (16 threads x 4 interleaved, so that stores of a warp are
+// contiguous) by 8 TM of the other one (8 threads x TM), kFLK steps of the
+// product per stage.  AX = 0: lines along x, whose contiguous dimension is
+// the line itself; AX = 1: lines along y or z, adjacent lines contiguous.
+// TM = 8 needs 6 shared-memory wavefronts for the 8 cycles that a warp's 32
+// FMAs take (TM = 4: 5 for 4), so it is used where it leaves enough blocks.
+constexpr int kFLThreads = 128, kFLC = 64, kFLK = 16;
+
+// Line l of the axis: offset of its first point; stride along the axis.
+RBFIB_DEVFN int fdl_base(const FDGrid& G, int axis, int l) {
+  if (axis == 0) return l * G.e[0];
+  if (axis == 1) {
+    const int z = l / G.e[0];
+    return (l - z * G.e[0]) + z * G.e[0] * G.e[1];
+  }
+  return l;
+}
+RBFIB_DEVFN int fdl_stride(const FDGrid& G, int axis) { return axis == 0 ? 1 : (axis == 1 ? G.e[0] : G.e[0] * G.e[1]); }
+
+template <int AX, int TM>
+struct FdlTile {
+  static constexpr int LT = AX == 0 ? 8 * TM : kFLC;   // lines
+  static constexpr int CT = AX == 0 ? kFLC : 8 * TM;   // outputs along the axis
+  static constexpr int FN = kFLK * LT / kFLThreads;    // staged line entries of a thread
+  static constexpr int BN = kFLK * CT / 4 / kFLThreads > 0 ? kFLK * CT / 4 / kFLThreads : 1;   // staged float4 of the basis
+  float F[2][kFLK][LT + 4];
+  float B[2][kFLK][CT + 4];
+};
+
+// acc += F B over one stage
+template <int AX, int TM>
+RBFIB_DEVFN void fdl_fma(const FdlTile<AX, TM>& S, int buf, int tx, int ty, float acc[TM][4]) {
+#pragma unroll
+  for (int k = 0; k < kFLK; ++k) {
+    const float* co = AX == 0 ? S.B[buf][k] : S.F[buf][k];
+    const float* ot = AX == 0 ? S.F[buf][k] : S.B[buf][k];
+    float o[TM], c[4];
+#pragma unroll
+    for (int q = 0; q < TM / 4; ++q) {
+      const float4 v = *reinterpret_cast<const float4*>(ot + TM * ty + 4 * q);
+      o[4 * q] = v.x; o[4 * q + 1] = v.y; o[4 * q + 2] = v.z; o[4 * q + 3] = v.w;
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) c[i] = co[tx + 16 * i];
+#pragma unroll
+    for (int r = 0; r < TM; ++r)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) acc[r][i] = fmaf(o[r], c[i], acc[r][i]);
+  }
+}
+
+// The product of K steps: load(k, line) gives the line entry of step k,
+// B (rows of pitch floats) the basis from column c0.
+template <int AX, int TM, typename Load>
+RBFIB_DEVFN void fdl_product(FdlTile<AX, TM>& S, int K, const float* __restrict__ B, int pitch, int c0, Load load,
+                             float acc[TM][4]) {
+  typedef FdlTile<AX, TM> Tl;
+  const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
+  float rf[Tl::FN];
+  float4 rb[Tl::BN];
+  auto fetch = [&](int k0) {
+#pragma unroll
+    for (int i = 0; i < Tl::FN; ++i) {
+      const int e = t + kFLThreads * i;
+      const int kk = AX == 0 ? e % kFLK : e / Tl::LT, l = AX == 0 ? e / kFLK : e % Tl::LT;
+      rf[i] = load(min(k0 + kk, K - 1), l);   // past K the basis rows are zero
+    }
+#pragma unroll
+    for (int i = 0; i < Tl::BN; ++i) {
+      const int e = t + kFLThreads * i;
+      const int kk = e / (Tl::CT / 4), c = c0 + 4 * (e % (Tl::CT / 4));
+      rb[i] = (kk < kFLK && k0 + kk < K && c < pitch)
+                  ? __ldg(reinterpret_cast<const float4*>(B + (long long)(k0 + kk) * pitch + c))
+                  : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+  };
+  auto put = [&](int buf) {
+#pragma unroll
+    for (int i = 0; i < Tl::FN; ++i) {
+      const int e = t + kFLThreads * i;
+      const int kk = AX == 0 ? e % kFLK : e / Tl::LT, l = AX == 0 ? e / kFLK : e % Tl::LT;
+      S.F[buf][kk][l] = rf[i];
+    }
+#pragma unroll
+    for (int i = 0; i < Tl::BN; ++i) {
+      const int e = t + kFLThreads * i;
+      const int kk = e / (Tl::CT / 4);
+      if (kk < kFLK) *reinterpret_cast<float4*>(&S.B[buf][kk][4 * (e % (Tl::CT / 4))]) = rb[i];
+    }
+  };
+  fetch(0);
+  put(0);
+  __syncthreads();
+  int buf = 0;
+  for (int k0 = 0; k0 < K; k0 += kFLK) {
+    const bool more = k0 + kFLK < K;
+    if (more) fetch(k0 + kFLK);
+    fdl_fma<AX, TM>(S, buf, tx, ty, acc);
+    if (more) put(buf ^ 1);
+    __syncthreads();
+    buf ^= 1;
+  }
+}
+
+// Forward transform along one axis: blockIdx.x line tiles, blockIdx.y tiles
+// of the even, then of the odd eigenvectors, blockIdx.z grids.  scaled: the
+// last forward pass divides by s (l_x + l_y + l_z) (z axis; zero modes
+// dropped).
+template <int AX, int TM>
+__global__ void __launch_bounds__(kFLThreads) k_fdl_fwd(FDParams P, int axis, int scaled,
+                                                        const float* __restrict__ in, float* __restrict__ out) {
+  pdl_entry();
+  typedef FdlTile<AX, TM> Tl;
+  __shared__ __align__(16) Tl S;
+  const FDGrid& G = P.g[blockIdx.z];
+  const FDAxis& X = G.ax[axis];
+  const int nl = G.e[0] * G.e[1] * G.e[2] / X.e, l0 = blockIdx.x * Tl::LT;
+  const int nS = (X.hs + Tl::CT - 1) / Tl::CT, nA = (X.ha + Tl::CT - 1) / Tl::CT;
+  if (l0 >= nl || (int)blockIdx.y >= nS + nA) return;
+  const bool odd = (int)blockIdx.y >= nS;
+  const int c0 = ((int)blockIdx.y - (odd ? nS : 0)) * Tl::CT, nc = odd ? X.ha : X.hs;
+  const float* src = in + G.off;
+  const int st = fdl_stride(G, axis);
+  float acc[TM][4];
+#pragma unroll
+  for (int r = 0; r < TM; ++r)
+#pragma unroll
+    for (int i = 0; i < 4; ++i) acc[r][i] = 0.f;
+  const int last = nl - 1;
+  const float sg = odd ? -1.f : 1.f;
+  // AX = 1: the lines of a thread's entries are the same in every stage
+  const int own = AX == 1 ? fdl_base(G, axis, min(l0 + (int)threadIdx.x % Tl::LT, last)) : 0;
+  fdl_product<AX, TM>(
+      S, X.hs, P.tab + (odd ? X.fA : X.fS), odd ? X.pa : X.ps, c0,
+      [&](int p, int l) {
+        int a, b;
+        fold_pair(X, p, a, b);
+        const float* line = src + (AX == 1 ? own : min(l0 + l, last) * G.e[0]);
+        // both points loaded without a branch, so that a stage's loads are in
+        // flight together
+        const float va = line[a * st], vb = line[b * st];
+        return fmaf(a == b ? 0.f : sg, vb, va);
+      },
+      acc);
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  float* dst = out + G.off;
+  const int shift = odd ? X.hs : 0;
+#pragma unroll
+  for (int r = 0; r < TM; ++r)
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int co = tx + 16 * i, ot = TM * ty + r;
+      const int l = l0 + (AX == 0 ? ot : co), c = c0 + (AX == 0 ? co : ot);
+      if (l >= nl || c >= nc) continue;
+      float v = acc[r][i];
+      if (scaled) {
+        const int y = l / G.e[0];
+        const float s = G.scale * ((P.tab[G.lam[0] + l - y * G.e[0]] + P.tab[G.lam[1] + y]) + P.tab[G.lam[2] + shift + c]);
+        v = s > 0.f ? v / s : 0.f;
+      }
+      dst[fdl_base(G, axis, l) + (shift + c) * st] = v;
+    }
+}
+
+// Backward transform along one axis: the even and the odd part of a pair
+// are summed apart, then the pair's two points are their sum and difference.
+template <int AX, int TM>
+__global__ void __launch_bounds__(kFLThreads) k_fdl_bwd(FDParams P, int axis, const float* __restrict__ in,
+                                                        float* __restrict__ out) {
+  pdl_entry();
+  typedef FdlTile<AX, TM> Tl;
+  __shared__ __align__(16) Tl S;
+  const FDGrid& G = P.g[blockIdx.z];
+  const FDAxis& X = G.ax[axis];
+  const int nl = G.e[0] * G.e[1] * G.e[2] / X.e, l0 = blockIdx.x * Tl::LT, p0 = blockIdx.y * Tl::CT;
+  if (l0 >= nl || p0 >= X.hs) return;
+  const float* src = in + G.off;
+  const int st = fdl_stride(G, axis), last = nl - 1;
+  const int own = AX == 1 ? fdl_base(G, axis, min(l0 + (int)threadIdx.x % Tl::LT, last)) : 0;
+  float ev[TM][4], od[TM][4];
+#pragma unroll
+  for (int r = 0; r < TM; ++r)
+#pragma unroll
+    for (int i = 0; i < 4; ++i) { ev[r][i] = 0.f; od[r][i] = 0.f; }
+  fdl_product<AX, TM>(
+      S, X.hs, P.tab + X.bS, X.ps, p0,
+      [&](int c, int l) { return src[(AX == 1 ? own : min(l0 + l, last) * G.e[0]) + c * st]; }, ev);
+  if (X.ha > 0)
+    fdl_product<AX, TM>(
+        S, X.ha, P.tab + X.bA, X.ps, p0,
+        [&](int c, int l) { return src[(AX == 1 ? own : min(l0 + l, last) * G.e[0]) + (X.hs + c) * st]; }, od);
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  float* dst = out + G.off;
+#pragma unroll
+  for (int r = 0; r < TM; ++r)
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int co = tx + 16 * i, ot = TM * ty + r;
+      const int l = l0 + (AX == 0 ? ot : co), p = p0 + (AX == 0 ? co : ot);
+      if (l >= nl || p >= X.hs) continue;
+      int a, b;
+      fold_pair(X, p, a, b);
+      float* line = dst + fdl_base(G, axis, l);
+      line[a * st] = ev[r][i] + od[r][i];
+      if (a != b) line[b * st] = ev[r][i] - od[r][i];
+    }
+}
+
+template <int AX, int TM>
+void fdl_launch(const FDParams& P, int axis, bool fwd, int scaled, const float* in, float* out, cudaStream_t s) {
+  typedef FdlTile<AX, TM> Tl;
+  int gx = 1, gy = 1;
+  for (int g = 0; g < P.ng; ++g) {
+    const FDAxis& X = P.g[g].ax[axis];
+    const int nl = P.g[g].e[0] * P.g[g].e[1] * P.g[g].e[2] / X.e;
+    gx = std::max(gx, (nl + Tl::LT - 1) / Tl::LT);
+    gy = std::max(gy, (X.hs + Tl::CT - 1) / Tl::CT + (fwd ? (X.ha + Tl::CT - 1) / Tl::CT : 0));
+  }
+  if (fwd) launch_k(k_fdl_fwd<AX, TM>, dim3(gx, gy, P.ng), kFLThreads, 0, s, P, axis, scaled, in, out);
+  else launch_k(k_fdl_bwd<AX, TM>, dim3(gx, gy, P.ng), kFLThreads, 0, s, P, axis, in, out);
+  note_launch();
+}
+
+// One pass, with the wide tile where that still gives two blocks per SM.
+void fdl_pass(const FDParams& P, int axis, bool fwd, int scaled, const float* in, float* out, cudaStream_t s) {
+  long long tiles = 0;
+  for (int g = 0; g < P.ng; ++g) {
+    const FDAxis& X = P.g[g].ax[axis];
+    const long long nl = (long long)P.g[g].e[0] * P.g[g].e[1] * P.g[g].e[2] / X.e;
+    tiles += ((nl + 63) / 64) * ((X.hs + 63) / 64 + (fwd ? (X.ha + 63) / 64 : 0));
+  }
+  const bool big = tiles >= 2 * 152;
+  if (axis == 0) {
+    if (big) fdl_launch<0, 8>(P, axis, fwd, scaled, in, out, s);
+    else fdl_launch<0, 4>(P, axis, fwd, scaled, in, out, s);
+  } else {
+    if (big) fdl_launch<1, 8>(P, axis, fwd, scaled, in, out, s);
+    else fdl_launch<1, 4>(P, axis, fwd, scaled, in, out, s);
+  }
+}
+
+void fd_solve_lines(const FDParams& P, float* u, const float* rhs, float* tmp, cudaStream_t s) {
+  fdl_pass(P, 0, true, 0, rhs, tmp, s);
+  fdl_pass(P, 1, true, 0, tmp, u, s);
+  if (P.g[0].q2) {
+    int tiles = 0;
+    for (int g = 0; g < P.ng; ++g) tiles += (P.g[g].e[0] * P.g[g].e[1] + 31) / 32;
+    launch_k(k_fdw_z, tiles, 256, 0, s, P, u);
+    note_launch();
+  } else {
+    fdl_pass(P, 2, true, 1, u, tmp, s);
+    fdl_pass(P, 2, false, 0, tmp, u, s);
+  }
+  fdl_pass(P, 1, false, 0, u, tmp, s);
+  fdl_pass(P, 0, false, 0, tmp, u, s);
+}
+
+// Whole-GPU form: tmp holds the level's transformed coefficients.
 void fd_solve_wide(const FDParams& P, float* u, const float* rhs, float* tmp, cudaStream_t s) {
   int planes = 0, tiles = 0;
   for (int g = 0; g < P.ng; ++g) {
@@ -493,12 +777,14 @@ void fd_solve_wide(const FDParams& P, float* u, const float* rhs, float* tmp, cu
   note_launch();
 }
 
+}  // namespace
+
 // The whole-GPU form for levels whose largest grid has more than
 // kFDWideMin points (the cluster kernel is faster on the small coarse levels,
 // e.g. 17 against 19 us at 24 x 24 x 16); RBFIB_FD_WIDE_MIN overrides the
 // threshold (read once).
 constexpr long long kFDWideMin = 32768;
-bool fd_use_wide(const FDParams& P) {
+static bool fd_use_wide(const FDParams& P) {
   static const long long lim = [] {
     const char* e = std::getenv("RBFIB_FD_WIDE_MIN");
     return e ? std::atoll(e) : kFDWideMin;
@@ -508,10 +794,9 @@ bool fd_use_wide(const FDParams& P) {
   return m > lim;
 }
 
-// Longest line solved by fast diagonalisation: kFDLine, or a smaller value
-// from RBFIB_FD_LINE (read once; for measurements of the multigrid levels
-// above the exact solve).
-int fd_line_limit() {
+// Longest line of the short-line forms: kFDLine, or a smaller value from
+// RBFIB_FD_LINE (read once).
+static int fd_line_limit() {
   static const int lim = [] {
     const char* e = std::getenv("RBFIB_FD_LINE");
     const int v = e ? std::atoi(e) : kFDLine;
@@ -520,44 +805,147 @@ int fd_line_limit() {
   return lim;
 }
 
+// Largest e_x + e_y + e_z solved in the long-line form; RBFIB_FD_SUM
+// overrides it (read once; 0 measures the V-cycles).  The exact solve costs
+// 2 (e_x + e_y + e_z) operations per point and direction, the V-cycles above
+// a short-line level a fixed number of passes and launches, and the exact
+// solve saves iterations.  Stokes solves to 1e-8 (FP32 refined), exact
+// against V-cycles: 96^3 8.9 / 11.2 ms, 160^3 40.5 / 42.1, 192^3 64.9 /
+// 69.7, 256^3 152 / 172; larger grids keep the V-cycles on their finest levels.
+constexpr int kFDLinesSum = 800;
+static int fd_lines_limit() {
+  static const int lim = [] {
+    const char* e = std::getenv("RBFIB_FD_SUM");
+    return e ? std::atoi(e) : kFDLinesSum;
+  }();
+  return lim;
+}
+
+namespace {
+
+AxisKind axis_kind(const Dims& d, bool faces, int g, int ax) {
+  if (d.per[ax]) return kPeriodic;
+  if (!faces) return kNeumann;
+  if (ax == g) return kDirichlet;
+  const bool even_lo = ghost_sign(d, 2 * ax) > 0, even_hi = ghost_sign(d, 2 * ax + 1) > 0;
+  return even_lo ? (even_hi ? kNeumann : kNeumannGhost) : (even_hi ? kGhostNeumann : kGhost);
+}
+
+// Columns of the basis of kind even (odd = 0) or odd (1) under the mirror of
+// the axis: every other one, starting with the even column 0; on periodic
+// axes the constant and the cosines, then the sines; all of them, as even
+// ones, where there is no mirror.
+std::vector<int> fold_columns(AxisKind kind, int m, int odd) {
+  std::vector<int> c;
+  const bool none = kind == kGhostNeumann || kind == kNeumannGhost;
+  for (int k = 0; k < m; ++k) {
+    const bool is_odd = kind == kPeriodic ? (k > 0 && k % 2 == 0) : (!none && k % 2 == 1);
+    if (is_odd == (odd != 0)) c.push_back(k);
+  }
+  return c;
+}
+
+// Appends the folded tables of one axis (FDAxis) and its eigenvalues in
+// folded order.
+void fold_axis(AxisKind kind, int m, const std::vector<double>& Q, const std::vector<double>& lam, double ih2,
+               std::vector<float>& tab, FDAxis& X, int& lam0) {
+  const std::vector<int> cs = fold_columns(kind, m, 0), ca = fold_columns(kind, m, 1);
+  X.e = m;
+  X.fold = kind == kPeriodic ? kFoldPeriodic : (kind == kGhostNeumann || kind == kNeumannGhost ? kFoldNone : kFoldMirror);
+  X.hs = (int)cs.size();
+  X.ha = (int)ca.size();
+  X.ps = (X.hs + 3) & ~3;
+  X.pa = (X.ha + 3) & ~3;
+  auto self = [&](int p) {
+    return X.fold == kFoldNone || (X.fold == kFoldMirror ? 2 * p == m - 1 : p == 0 || 2 * p == m);
+  };
+  auto rows = [&](int nr, int pitch, int nc, auto value) {
+    const int at = (int)tab.size();
+    for (int r = 0; r < nr; ++r)
+      for (int c = 0; c < pitch; ++c) tab.push_back(c < nc ? (float)value(r, c) : 0.f);
+    return at;
+  };
+  auto q = [&](int j, int k) { return Q[(size_t)j * m + k]; };
+  X.fS = rows(X.hs, X.ps, X.hs, [&](int p, int c) { return q(p, cs[c]); });
+  X.fA = rows(X.hs, X.pa, X.ha, [&](int p, int c) { return self(p) ? 0.0 : q(p, ca[c]); });
+  X.bS = rows(X.hs, X.ps, X.hs, [&](int c, int p) { return q(p, cs[c]); });
+  X.bA = rows(X.ha, X.ps, X.hs, [&](int c, int p) { return self(p) ? 0.0 : q(p, ca[c]); });
+  lam0 = (int)tab.size();
+  for (int k : cs) tab.push_back((float)(lam[k] * ih2));
+  for (int k : ca) tab.push_back((float)(lam[k] * ih2));
+  while (tab.size() % 4) tab.push_back(0.f);
+}
+
+// The basis in plain order: Q and Q^T (rows padded to 8 floats), then the
+// eigenvalues.
+void plain_axis(int m, const std::vector<double>& Q, const std::vector<double>& lam, double ih2,
+                std::vector<float>& tab, int& q0, int& qt0, int& lam0) {
+  const int mp = (m + 7) & ~7;
+  q0 = (int)tab.size();
+  for (int t = 0; t < m; ++t)
+    for (int c = 0; c < mp; ++c) tab.push_back(c < m ? (float)Q[(size_t)t * m + c] : 0.f);
+  qt0 = (int)tab.size();
+  for (int t = 0; t < m; ++t)
+    for (int c = 0; c < mp; ++c) tab.push_back(c < m ? (float)Q[(size_t)c * m + t] : 0.f);
+  lam0 = (int)tab.size();
+  for (int c = 0; c < mp; ++c) tab.push_back(c < m ? (float)(lam[c] * ih2) : 0.f);
+}
+
+}  // namespace
+
 bool fd_plan(const Dims& d, bool faces, double eta, std::vector<float>& tab, FDParams& P, std::string& why) {
   P = FDParams{};
   P.ng = faces ? 3 : 1;
   const size_t tab_start = tab.size();
   auto fail = [&](const char* w) { why = w; tab.resize(tab_start); return false; };
+  int longest = 0, ez = 0, sum = 0;
+  for (int g = 0; g < P.ng; ++g) {
+    const int* e = faces ? d.fe[g] : d.n;
+    for (int ax = 0; ax < 3; ++ax) {
+      if (e[ax] < 1) return fail("extent");
+      longest = std::max(longest, e[ax]);
+    }
+    ez = std::max(ez, e[2]);
+    sum = std::max(sum, e[0] + e[1] + e[2]);
+  }
+  P.lines = longest > fd_line_limit() ? 1 : 0;
+  if (P.lines && (longest > kFDLongest || sum > fd_lines_limit() || d.fo[3] + d.nc >= (1LL << 31))) return fail("extent");
+  // z-axis basis in plain order too, for k_fdw_z
+  const bool plain_z = !P.lines || ez <= kFDLine;
+  struct Basis { AxisKind kind; int m; std::vector<double> Q, lam; };
+  std::vector<Basis> seen;   // grids of one level share most of their axes
   int smem = 0;
+  while (tab.size() % 4 || tab.empty()) tab.push_back(0.f);
   for (int g = 0; g < P.ng; ++g) {
     FDGrid& G = P.g[g];
     const int* e = faces ? d.fe[g] : d.n;
-    long long n = 1;
-    for (int ax = 0; ax < 3; ++ax) {
-      G.e[ax] = e[ax];
-      n *= e[ax];
-      if (e[ax] < 1 || e[ax] > fd_line_limit()) return fail("extent");
-    }
-    if (n > kFDMaxPoints) return fail("points");
     G.off = faces ? d.fo[g] : 0;
     G.scale = faces ? (float)eta : 1.0f;
     G.tab0 = (int)tab.size();
     for (int ax = 0; ax < 3; ++ax) {
-      AxisKind kind;
-      if (d.per[ax]) kind = kPeriodic;
-      else if (!faces) kind = kNeumann;
-      else if (ax == g) kind = kDirichlet;
-      else {
-        const bool even_lo = ghost_sign(d, 2 * ax) > 0, even_hi = ghost_sign(d, 2 * ax + 1) > 0;
-        kind = even_lo ? (even_hi ? kNeumann : kNeumannGhost) : (even_hi ? kGhostNeumann : kGhost);
+      const int m = G.e[ax] = e[ax];
+      const AxisKind kind = axis_kind(d, faces, g, ax);
+      const Basis* B = nullptr;
+      for (const Basis& b : seen)
+        if (b.kind == kind && b.m == m) B = &b;
+      Basis fresh;
+      if (!B) {
+        fresh.kind = kind;
+        fresh.m = m;
+        axis_basis(kind, m, fresh.Q, fresh.lam);
+        if (!basis_ok(kind, m, fresh.Q, fresh.lam)) return fail("basis check");
+        B = &fresh;
       }
-      std::vector<double> Q, lam;
-      axis_basis(kind, e[ax], Q, lam);
-      if (!basis_ok(kind, e[ax], Q, lam)) return fail("basis check");
-      const int m = e[ax], mp = (m + 7) & ~7;
       const double ih2 = 1.0 / (d.h[ax] * d.h[ax]);
-      for (int t = 0; t < m; ++t)
-        for (int c = 0; c < mp; ++c) tab.push_back(c < m ? (float)Q[(size_t)t * m + c] : 0.f);
-      for (int t = 0; t < m; ++t)
-        for (int c = 0; c < mp; ++c) tab.push_back(c < m ? (float)Q[(size_t)c * m + t] : 0.f);
-      for (int c = 0; c < mp; ++c) tab.push_back(c < m ? (float)(lam[c] * ih2) : 0.f);
+      if (!P.lines || (ax == 2 && plain_z)) {
+        int q0, qt0;
+        plain_axis(m, B->Q, B->lam, ih2, tab, q0, qt0, G.lam[ax]);
+        if (ax == 2) { G.q2 = q0; G.qt2 = qt0; }
+        G.ax[ax].e = m;
+      } else {
+        fold_axis(kind, m, B->Q, B->lam, ih2, tab, G.ax[ax], G.lam[ax]);
+      }
+      if (B == &fresh) seen.push_back(std::move(fresh));
     }
     G.tabn = (int)tab.size() - G.tab0;
     // every grid's segment starts on a 16-byte boundary of the table
@@ -565,17 +953,24 @@ bool fd_plan(const Dims& d, bool faces, double eta, std::vector<float>& tab, FDP
     const long long slab = (long long)((e[2] + kFDCtas - 1) / kFDCtas) * e[0] * e[1];
     smem = std::max(smem, (int)((((G.tabn + 3) & ~3) + 2 * ((slab + 3) & ~3)) * sizeof(float)));
   }
-  P.smem = smem;
+  P.smem = P.lines ? 0 : smem;
   return true;
 }
 
-void fd_solve(const FDParams& P, float* u, const float* rhs, cudaStream_t s) {
+// One cluster per grid.
+static void fd_solve_cluster(const FDParams& P, float* u, const float* rhs, cudaStream_t s) {
   static std::once_flag f;
   std::call_once(f, [] {
     cudaFuncSetAttribute(k_fd_solve, cudaFuncAttributeMaxDynamicSharedMemorySize, kFDMaxSmem);
   });
   launch_k(k_fd_solve, P.ng * kFDCtas, kFDThreads, P.smem, s, P, u, rhs);
   note_launch();
+}
+
+void fd_solve(const FDParams& P, float* u, const float* rhs, float* tmp, cudaStream_t s) {
+  if (P.lines) fd_solve_lines(P, u, rhs, tmp, s);
+  else if (fd_use_wide(P)) fd_solve_wide(P, u, rhs, tmp, s);
+  else fd_solve_cluster(P, u, rhs, s);
 }
 
 }  // namespace rbfib

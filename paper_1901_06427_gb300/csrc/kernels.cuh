@@ -83,31 +83,45 @@ template <typename T> void add_grad(const Dims&, const T* phi, T* v, double* v64
 // orthonormal 1D eigenbases Q_x, Q_y, Q_z and eigenvalues l_x, l_y, l_z,
 // A^-1 = (Q_x (x) Q_y (x) Q_z) diag(1 / (s (l_x + l_y + l_z))) (Q_x (x) Q_y (x) Q_z)^T,
 // the zero mode of a singular operator dropped (pseudo-inverse).
-constexpr int kFDMaxPoints = 48 * 48 * 48;  // points of one grid
-constexpr int kFDLine = 48;                 // points along one axis
+constexpr int kFDLine = 48;                 // points along one axis (short-line forms)
+constexpr int kFDLongest = 1024;            // points along one axis (long-line form)
 constexpr int kFDCtas = 8;           // CTAs (one cluster) per grid
 constexpr int kFDThreads = 256;
 // shared memory bound per CTA: table (3 axes, two padded e x e bases and e
 // eigenvalues each) and two slab buffers of ceil(e_z / kFDCtas) planes
 constexpr int kFDMaxSmem = (int)sizeof(float) * (3 * (2 * kFDLine * kFDLine + kFDLine) + 4 +
                                                  2 * (((kFDLine + kFDCtas - 1) / kFDCtas) * kFDLine * kFDLine + 4));
+// One axis of the long-line form (k_fdl_*): its basis folded by the mirror
+// symmetry of its eigenvectors.  Pair p joins the points jA(p), jB(p) (see
+// fold_pair); hs symmetric and ha antisymmetric eigenvectors, stored in that
+// order along the axis.  Table offsets: fS (hs x ps), fA (hs x pa) forward,
+// bS (hs x ps), bA (ha x ps) backward, rows padded to ps / pa floats.
+enum { kFoldMirror = 0, kFoldPeriodic = 1, kFoldNone = 2 };
+struct FDAxis {
+  int e, fold, hs, ha, ps, pa;
+  int fS, fA, bS, bA;
+};
 struct FDGrid {
   int e[3];        // extents
   long long off;   // offset of the grid in the level's solution / rhs arrays
   int tab0, tabn;  // segment of the basis table: per axis Q (e x e), Q^T (e x e), eigenvalues (e)
+  int lam[3];      // eigenvalues of each axis in the table
+  int q2, qt2;     // Q and Q^T of the z axis in the table (0: not stored)
   float scale;     // operator scale (eta for velocity, 1 for pressure)
+  FDAxis ax[3];    // long-line form only
 };
 struct FDParams {
   int ng;          // grids (3 face components or 1 pressure grid), one CTA each
+  int lines;       // 1: the long-line form (an axis longer than kFDLine)
   FDGrid g[3];
   const float* tab;
   int smem;        // dynamic shared memory bytes of the largest grid
 };
 // Bases of every grid of a level; false if some grid exceeds the limits.
 bool fd_plan(const Dims& d, bool faces, double eta, std::vector<float>& tab, FDParams& P, std::string& why);
-void fd_solve(const FDParams& P, float* u, const float* rhs, cudaStream_t s);
-void fd_solve_wide(const FDParams& P, float* u, const float* rhs, float* tmp, cudaStream_t s);
-bool fd_use_wide(const FDParams& P);
+// u = A^-1 rhs on the planned level; tmp holds as many floats as u.  The
+// form (one cluster per grid, whole GPU, long lines) is chosen by size.
+void fd_solve(const FDParams& P, float* u, const float* rhs, float* tmp, cudaStream_t s);
 
 // k_ib.cu
 void geometry(int nbl, const int* bob, const double* ref, const double* q, const double* quat,

@@ -402,8 +402,7 @@ void vcycle_vel(rbfib_grid* g, T* u0, const T* rhs0) {
   if constexpr (std::is_same<T, float>::value) {
     if (fd) {
       TimerScope ts(g, TK_COARSE, fd_bytes(g->fdv), fd_flops(g->fdv));
-      if (fd_use_wide(g->fdv)) fd_solve_wide(g->fdv, u[lt], rhs[lt], g->fd_tmp, g->s);
-      else fd_solve(g->fdv, u[lt], rhs[lt], g->s);
+      fd_solve(g->fdv, u[lt], rhs[lt], g->fd_tmp, g->s);
     } else {
       vel_coarse<T>(g->levels[L - 1].d, eta, u[L - 1], rhs[L - 1], coarse_sweeps(g->levels[L - 1].d), g->s);
     }
@@ -441,8 +440,7 @@ void vcycle_p(rbfib_grid* g, T* u0, T* rhs0) {
   if constexpr (std::is_same<T, float>::value) {
     if (fd) {
       TimerScope ts(g, TK_COARSE, fd_bytes(g->fdp), fd_flops(g->fdp));
-      if (fd_use_wide(g->fdp)) fd_solve_wide(g->fdp, u[lt], rhs[lt], g->fd_tmp, g->s);
-      else fd_solve(g->fdp, u[lt], rhs[lt], g->s);
+      fd_solve(g->fdp, u[lt], rhs[lt], g->fd_tmp, g->s);
     } else {
       p_coarse<T>(g->levels[L - 1].d, u[L - 1], rhs[L - 1], coarse_sweeps(g->levels[L - 1].d), g->s);
     }
@@ -901,7 +899,8 @@ void build_levels(rbfib_grid* g) {
 }
 
 // Coarse levels of the FP32 V-cycles: the finest level whose grids all fit
-// one cluster's exact solve, for the velocity components and for the pressure.
+// the exact solve (usually the grid itself), for the velocity components and
+// for the pressure.
 void build_fd(rbfib_grid* g) {
   std::vector<float> tab;
   g->fd_vel = g->fd_p = -1;
