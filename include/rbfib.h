@@ -144,9 +144,11 @@ int rbfib_saddle_layout(const rbfib_grid* g, int64_t offsets[7]);
  * accumulated in FP64 for either dtype. */
 int rbfib_apply_saddle(rbfib_grid* g, const void* x, void* y, int32_t dtype);
 
-/* z = P^{-1} r: the block preconditioner used inside the Krylov solves (the
+/* z = P^{-1} r: the block preconditioner of the Krylov solves (the
  * paper defers its preconditioner to the cited rigid-multiblob work; this one
- * is ours): a projection-method multigrid V-cycle pair for the Stokes block
+ * is ours): a projection-method pair of exact or multigrid V-cycle solves for
+ * the Stokes block (inside the solves its pressure -eta q also takes a
+ * multiple of the projection's potential, for the drag of no-slip walls)
  * and, for the bodies, the Schur complement with the blob mobility replaced
  * by free-space Rotne-Prager-Yamakawa blocks.  r, z: device FP64 saddle
  * vectors; computed in FP32 internally. */

@@ -72,10 +72,10 @@ template <typename T> void vel_coarse(const Dims&, T eta, T* u, const T* rhs, in
 template <typename T> void p_rbgs(const Dims&, int color, T* u, const T* rhs, cudaStream_t, int block = 256);
 template <typename T> void p_prolong(const Dims&, const Dims&, int3, const T*, T*, cudaStream_t);
 template <typename T> void p_coarse(const Dims&, T* u, T* rhs, int sweeps, cudaStream_t);
-// pi64 / v64: FP64 copies of the outputs (null: none)
-template <typename T> void div_q(const Dims&, T eta, const T* vt, const T* rpi, T* q, T* pi, double* pi64,
-                                 cudaStream_t);
-template <typename T> void add_grad(const Dims&, const T* phi, T* v, double* v64, cudaStream_t);
+template <typename T> void div_q(const Dims&, const T* vt, const T* rpi, T* q, cudaStream_t);
+// z: faces (in: v~) then cells (out); z64: FP64 copy of the output (null: none)
+template <typename T> void add_grad(const Dims&, T eta, T kappa, const T* phi, const T* q, T* z, double* z64,
+                                    cudaStream_t);
 
 // Exact solve on a coarse multigrid level by fast diagonalisation (k_fdsolve.cu).
 // The level operator of each grid (a velocity component of -eta LL, or the

@@ -144,6 +144,7 @@ struct rbfib_grid {
   Walls walls{};
   i64 nf = 0, nc = 0, nfl = 0;
   double dV = 1.0;
+  double kappa = 0.0;   // pressure_kappa
   StressLayout stress{};
   // bodies
   int nb = 0, nbl = 0;
@@ -455,6 +456,22 @@ void vcycle_p(rbfib_grid* g, T* u0, T* rhs0) {
   }
 }
 
+// kappa of the pressure block: per axis the walls' share of the viscous drag
+// on a flow across it, 12 / H^2 between two no-slip walls, 3 / H^2 (half a
+// channel of height 2 H) with one of them free-slip; the smallest sum over
+// the two axes across a direction, which is that of the longest waves.
+// Krylov iterations of a fluid-driven and a sphere's solve to 1e-8: two-sphere
+// box 33 -> 27 (rigid), slit of 384 x 48 x 12 57 -> 35 (fluid).
+double pressure_kappa(const Dims& d) {
+  double drag[3];
+  for (int b = 0; b < 3; ++b) {
+    const double H = d.n[b] * d.h[b];
+    const int noslip = d.per[b] ? 0 : (d.gd[2 * b] > 0) + (d.gd[2 * b + 1] > 0);
+    drag[b] = noslip == 2 ? 12.0 / (H * H) : (noslip == 1 ? 3.0 / (H * H) : 0.0);
+  }
+  return std::min(drag[0] + drag[1], std::min(drag[0] + drag[2], drag[1] + drag[2]));
+}
+
 template <typename T> T* sres_of(rbfib_grid* g);
 template <> double* sres_of<double>(rbfib_grid* g) { return g->sres; }
 template <> float* sres_of<float>(rbfib_grid* g) { return g->sres32; }
@@ -462,24 +479,29 @@ template <> float* sres_of<float>(rbfib_grid* g) { return g->sres32; }
 // ---------------------------------------------------------- preconditioner
 // Block lower-triangular preconditioner of the saddle operator.
 // Fluid block (projection method): v~ = (-eta LL)^{-1} r_v (V-cycle),
-// q = r_pi + D v~, phi = (-D G)^{-1} q (V-cycle), v = v~ + G phi, pi = -eta q.
+// q = r_pi + D v~, phi = (-D G)^{-1} q (V-cycle), v = v~ + G phi,
+// pi = -eta (q + kappa phi).  -eta q alone (kappa = 0) is exact for periodic
+// boxes.  Between no-slip walls a distance H apart a long pressure wave (k H
+// small) drives Poiseuille flow instead, for which the pressure operator
+// D (-LL)^{-1} G is k^2 H^2 / 12, not 1: kappa = 12 / H^2 adds that limit, as
+// the mass term's part does in preconditioners of the unsteady Stokes
+// problem (Cahouet and Chabard).  See pressure_kappa.
 // Body block: Schur complement [-M K; K^T 0] with M replaced per body by the
 // free-space RPY blob mobility of its shape, right-hand side
 // (r_lam + J v, r_U).
 // z64 (optional): the result is also written in FP64 there by the kernels
 // that produce each block, which saves a conversion launch.
 template <typename T>
-void precond(rbfib_grid* g, const T* r, T* z, bool with_bodies, double* z64 = nullptr) {
+void precond(rbfib_grid* g, const T* r, T* z, bool with_bodies, double* z64, double kappa) {
   const Dims& d = g->d;
   T* zv = z;
-  T* zp = z + g->nf;
   MGStore<T>& M = mg_of<T>(g);
   vcycle_vel<T>(g, zv, r);
   T* q = *M.prhs[0];
   T* phi = *M.pu[0];
-  div_q<T>(d, (T)g->desc.eta, zv, r + g->nf, q, zp, z64 ? z64 + g->nf : nullptr, g->s);
+  div_q<T>(d, zv, r + g->nf, q, g->s);
   vcycle_p<T>(g, phi, q);
-  add_grad<T>(d, phi, zv, z64, g->s);
+  add_grad<T>(d, (T)g->desc.eta, (T)kappa, phi, q, z, z64, g->s);
   if (with_bodies && g->nb > 0) {
     const T* rl = r + g->nfl;
     const T* rU = rl + 3 * (i64)g->nbl;
@@ -510,10 +532,10 @@ void precond(rbfib_grid* g, const T* r, T* z, bool with_bodies, double* z64 = nu
 void precond_any(rbfib_grid* g, const double* r, double* z, bool with_bodies, bool r32_ready = false) {
   const i64 n = with_bodies ? g->n_total() : g->nfl;
   if (!r32_ready) convert<double, float>(r, g->f32a, n, g->s);
-  precond<float>(g, g->f32a, g->f32b, with_bodies, z);
+  precond<float>(g, g->f32a, g->f32b, with_bodies, z, g->kappa);
 }
 void precond_any(rbfib_grid* g, const float* r, float* z, bool with_bodies, bool = false) {
-  precond<float>(g, r, z, with_bodies);
+  precond<float>(g, r, z, with_bodies, nullptr, g->kappa);
 }
 // Where the basis kernels put the FP32 copy of a new FP64 basis vector (the
 // FP32 Krylov mode keeps f32a for the right-hand side of its inner solve).
@@ -1339,6 +1361,7 @@ int rbfib_create_grid(const rbfib_grid_desc* desc, void* stream, rbfib_grid** ou
     g->nc = g->d.nc;
     g->nfl = g->nf + g->nc;
     g->dV = D.h * D.h * D.h;
+    g->kappa = pressure_kappa(g->d);
     build_stress_layout(g);
     g->nparts = 152 * 4;
     g->part.alloc(part_buffer_doubles(g->nparts));
@@ -1585,7 +1608,8 @@ int rbfib_set_bodies(rbfib_grid* g, int32_t n_bodies, const int32_t* blob_offset
 int rbfib_apply_preconditioner(rbfib_grid* g, const double* r, double* z) {
   if (!g || !r || !z) return fail(g, RBFIB_EINVAL, "apply_preconditioner: null argument");
   try {
-    precond_any(g, r, z, true);
+    convert<double, float>(r, g->f32a, g->n_total(), g->s);
+    precond<float>(g, g->f32a, g->f32b, true, z, 0.0);
     ck(cudaGetLastError());
   } catch (CudaError& e) {
     return fail(g, e.code, std::string("apply_preconditioner: ") + e.what());
