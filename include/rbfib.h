@@ -150,7 +150,7 @@ int rbfib_apply_saddle(rbfib_grid* g, const void* x, void* y, int32_t dtype);
  * the Stokes block (inside the solves its pressure -eta q also takes a
  * multiple of the projection's potential, for the drag of no-slip walls)
  * and, for the bodies, the Schur complement with the blob mobility replaced
- * by free-space Rotne-Prager-Yamakawa blocks.  r, z: device FP64 saddle
+ * by the kernel's free-space blob mobility.  r, z: device FP64 saddle
  * vectors; computed in FP32 internally. */
 int rbfib_apply_preconditioner(rbfib_grid* g, const double* r, double* z);
 
@@ -256,16 +256,16 @@ int rbfib_batch_set_one_graph(rbfib_batch* b, int32_t on);
 int64_t rbfib_batch_graph_steps(const rbfib_batch* b);
 
 /* Body block of the preconditioner: dense = 1 when it is the coupled
- * all-blob RPY block (at least two bodies, 3 N_bl <= 1536, 6 N_b <= 384),
- * else 0 (per-shape blocks).  The coupled block's inverse RPY matrix is
+ * block over all blobs (at least two bodies, 3 N_bl <= 1536, 6 N_b <= 384),
+ * else 0 (per-shape blocks).  The coupled block's inverse mobility matrix is
  * rebuilt for every new configuration (rbfib_set_bodies,
  * rbfib_set_blob_positions, each SEM step): by Gauss-Jordan after
- * rbfib_set_bodies; otherwise by eight Newton-Schulz steps from the previous
- * inverse, rotated with each body's rotation since it was built (when the
- * orientations are known: not after rbfib_set_blob_positions), if that
- * start's residual ||I - M X||_F is at most 0.95, else by Gauss-Jordan.
- * warm_starts counts the builds that took the Newton-Schulz path.  Either
- * pointer may be NULL. */
+ * rbfib_set_bodies and where 3 N_bl > 256; otherwise by four Newton-Schulz
+ * steps from the previous inverse, rotated with each body's rotation since it
+ * was built (when the orientations are known: not after
+ * rbfib_set_blob_positions), if that start's residual ||I - M X||_F is at
+ * most 0.25, else by Gauss-Jordan.  warm_starts counts the builds that took
+ * the Newton-Schulz path.  Either pointer may be NULL. */
 int rbfib_body_block_info(const rbfib_grid* g, int32_t* dense, int64_t* warm_starts);
 
 /* *device_driven = 1 if the grid's last SEM step ran as the device-driven

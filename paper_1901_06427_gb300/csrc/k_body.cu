@@ -1,11 +1,10 @@
 // Coupled body block of the preconditioner for suspensions with few blobs:
 // the Schur complement [-M K; K^T 0] of the saddle operator with the blob
-// mobility M replaced by the free-space Rotne-Prager-Yamakawa mobility of all
-// blobs of all bodies (inter-body coupling included).  Built once per
-// configuration: dense RPY matrix; its inverse (FP32) by in-place
-// Gauss-Jordan (no pivoting: the RPY matrix is symmetric positive definite)
-// or, when the previous configuration's inverse is close, by two
-// Newton-Schulz steps from it; P = M^-1 K; N = (K^T M^-1 K)^-1 (FP64).
+// mobility M replaced by the free-space mobility of all blobs of all bodies
+// (pair_mobility.cuh; inter-body coupling included).  Built once per
+// configuration: dense M; its inverse (FP32) by blocked Gauss-Jordan or, for
+// small matrices close to the previous configuration's, by Newton-Schulz
+// steps from its inverse; P = M^-1 K; N = (K^T M^-1 K)^-1 (FP64).
 // Applied by one cluster of CTAs.
 #include <algorithm>
 #include <cmath>
@@ -14,73 +13,128 @@
 
 #include "common.cuh"
 #include "kernels.cuh"
+#include "pair_mobility.cuh"
 
 namespace rbfib {
 
 static inline unsigned nblk(i64 n, int bs) { return (unsigned)((n + bs - 1) / bs); }
 
-__global__ void k_rpy_full(int nbl, const double* __restrict__ r, double a, double eta, float* __restrict__ M) {
+// M of all blobs, one thread per blob pair.
+__global__ void k_mobility_full(int nbl, const double* __restrict__ r, PairMobility P, double ih, double scale,
+                                float* __restrict__ M) {
   pdl_entry();
-  const i64 n3 = 3 * (i64)nbl;
   const i64 t = (i64)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= n3 * n3) return;
-  const int row = (int)(t / n3), col = (int)(t - (i64)row * n3);
-  const int i = row / 3, p = row % 3, j = col / 3, q = col % 3;
-  const double c0 = 1.0 / (6.0 * M_PI * eta * a);
-  double v;
-  if (i == j) {
-    v = (p == q) ? c0 : 0.0;
-  } else {
-    const double d[3] = {r[3 * i] - r[3 * j], r[3 * i + 1] - r[3 * j + 1], r[3 * i + 2] - r[3 * j + 2]};
-    const double rr2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
-    const double rr = sqrt(rr2);
-    double fI, fR;
-    if (rr >= 2.0 * a) {
-      const double c = 1.0 / (8.0 * M_PI * eta * rr);
-      fI = c * (1.0 + 2.0 * a * a / (3.0 * rr2));
-      fR = c * (1.0 - 2.0 * a * a / rr2);
-    } else {
-      fI = c0 * (1.0 - 9.0 * rr / (32.0 * a));
-      fR = c0 * (3.0 * rr / (32.0 * a));
-    }
-    v = (p == q ? fI : 0.0) + fR * d[p] * d[q] / rr2;
-  }
-  M[t] = (float)v;
+  if (t >= (i64)nbl * nbl) return;
+  const int i = (int)(t / nbl), j = (int)(t - (i64)i * nbl);
+  const double d[3] = {(r[3 * i] - r[3 * j]) * ih, (r[3 * i + 1] - r[3 * j + 1]) * ih, (r[3 * i + 2] - r[3 * j + 2]) * ih};
+  double B[9];
+  pair_block(P, d, i == j, B);
+  float* Mb = M + (i64)(3 * i) * (3 * nbl) + 3 * j;
+  for (int p = 0; p < 3; ++p)
+    for (int q = 0; q < 3; ++q) Mb[(i64)p * (3 * nbl) + q] = (float)(scale * B[3 * p + q]);
 }
 
-// In-place Gauss-Jordan inverse of an n x n matrix by one block (no
-// pivoting; the matrices are symmetric positive definite).  Per pivot k the
-// pivot column and row are staged in shared memory, then each warp updates
-// whole rows (lanes along the row).  status is set to 1 on a zero pivot.
+// One step of a blocked Gauss-Jordan inversion (no pivoting; the matrices
+// are symmetric positive definite), out of place: with the kGJ pivots from
+// k0 (block row and column P), every 32 x 32 tile (I, J) of B is
+//   (P, P): D = A_PP^-1;  (P, J): D A_PJ;  (I, P): -A_IP D;
+//   (I, J): A_IJ - A_IP D A_PJ.
+// Every block inverts the pivot block again (32 pivots, one barrier each,
+// two buffers) rather than wait for a launch of its own.  Bound by latency:
+// n / 32 launches of a few microseconds, where one block stepping through n
+// pivots took 2.35 ms at n = 252 and a chain of FP32 Newton-Schulz products
+// (k_ns_gemm) grows with n^3.  Entries past n are those of the identity.
+// status = 1 on a zero pivot.
+constexpr int kGJ = 32;
 template <typename R>
-__global__ void k_gj_inverse(R* __restrict__ A, int n, int* __restrict__ status) {
+__global__ void __launch_bounds__(256) k_gj_step(int n, int k0, const R* __restrict__ A, R* __restrict__ B,
+                                                 int* __restrict__ status) {
   pdl_entry();
-  extern __shared__ unsigned char shraw[];
-  R* col = (R*)shraw;   // column k
-  R* prow = col + n;    // row k
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  for (int k = 0; k < n; ++k) {
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-      col[i] = A[(i64)i * n + k];
-      prow[i] = A[(i64)k * n + i];
+  __shared__ R D[2][kGJ][kGJ + 1], U[kGJ][kGJ + 1], L[kGJ][kGJ + 1];
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  const int i0 = blockIdx.y * kGJ, j0 = blockIdx.x * kGJ;
+  R c[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int r = ty + 8 * q;
+    const bool rk = k0 + r < n, ri = i0 + r < n, ck = k0 + tx < n, cj = j0 + tx < n;
+    D[0][r][tx] = rk && ck ? A[(i64)(k0 + r) * n + k0 + tx] : (r == tx ? R(1) : R(0));
+    U[r][tx] = rk && cj ? A[(i64)(k0 + r) * n + j0 + tx] : R(0);
+    L[r][tx] = ri && ck ? A[(i64)(i0 + r) * n + k0 + tx] : R(0);
+    c[q] = ri && cj ? A[(i64)(i0 + r) * n + j0 + tx] : R(0);
+  }
+  __syncthreads();
+  const int np = min(kGJ, n - k0);
+  int cur = 0;
+  for (int k = 0; k < np; ++k) {
+    const R p = D[cur][k][k];
+    const bool ok = p > R(0) || p < R(0);
+    if (!ok && threadIdx.x == 0) *status = 1;
+    const R ip = ok ? R(1) / p : R(0), row = D[cur][k][tx] * ip;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int r = ty + 8 * q;
+      const R f = D[cur][r][k];
+      R v;
+      if (r == k) v = tx == k ? ip : row;
+      else v = tx == k ? -f * ip : D[cur][r][tx] - f * row;
+      D[cur ^ 1][r][tx] = v;
     }
+    cur ^= 1;
     __syncthreads();
-    const R p = prow[k];
-    if (!(p > R(0) || p < R(0))) {
-      if (threadIdx.x == 0) *status = 1;
-      return;
+  }
+  const bool rowP = i0 == k0, colP = j0 == k0;
+  R out[4];
+  if (rowP && colP) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) out[q] = D[cur][ty + 8 * q][tx];
+  } else {
+    // left factor D (for the pivot rows) or L, right factor U or D
+    R t[4] = {R(0), R(0), R(0), R(0)};
+#pragma unroll 8
+    for (int k = 0; k < kGJ; ++k) {
+      const R u = colP ? D[cur][k][tx] : U[k][tx];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) t[q] += (colP ? L[ty + 8 * q][k] : D[cur][ty + 8 * q][k]) * u;
     }
-    const R ip = R(1) / p;
-    for (int i = wid; i < n; i += nw) {
-      R* Ai = A + (i64)i * n;
-      if (i == k) {
-        for (int j = lane; j < n; j += 32) Ai[j] = (j == k) ? ip : prow[j] * ip;
-      } else {
-        const R f = col[i] * ip;
-        for (int j = lane; j < n; j += 32) Ai[j] = (j == k) ? -f : Ai[j] - f * prow[j];
+    if (rowP) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) out[q] = t[q];
+    } else if (colP) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) out[q] = -t[q];
+    } else {
+      __syncthreads();
+#pragma unroll
+      for (int q = 0; q < 4; ++q) U[ty + 8 * q][tx] = t[q];
+      __syncthreads();
+#pragma unroll 8
+      for (int k = 0; k < kGJ; ++k) {
+        const R u = U[k][tx];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) c[q] -= L[ty + 8 * q][k] * u;
       }
+#pragma unroll
+      for (int q = 0; q < 4; ++q) out[q] = c[q];
     }
-    __syncthreads();
+  }
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int r = i0 + ty + 8 * q;
+    if (r < n && j0 + tx < n) B[(i64)r * n + j0 + tx] = out[q];
+  }
+}
+
+// X = M^-1 (n x n), M kept; tmp: n x n work.
+template <typename R>
+void gj_inverse(int n, const R* M, R* X, R* tmp, int* status, cudaStream_t s) {
+  const int nt = (n + kGJ - 1) / kGJ;
+  const R* in = M;
+  for (int k = 0; k < nt; ++k) {
+    R* out = (nt - 1 - k) % 2 == 0 ? X : tmp;   // the last step lands in X
+    launch_k(k_gj_step<R>, dim3(nt, nt), 256, 0, s, n, k * kGJ, in, out, status);
+    note_launch();
+    in = out;
   }
 }
 
@@ -229,8 +283,8 @@ void ns_gemm(int n, const float* A, const float* B, const float* D, float* C, do
 
 // Rotates the previous configuration's inverse with each body's rotation
 // since then: X_ij <- D_b(i) X_ij D_b(j)^T for the 3 x 3 blocks (blobs i, j
-// of bodies b(i), b(j)), D_p = R(quat_new_p) R(quat_old_p)^T.  The RPY tensor
-// is rotation-covariant, so rotating each body rigidly about its centre turns
+// of bodies b(i), b(j)), D_p = R(quat_new_p) R(quat_old_p)^T.  M's blocks
+// are rotation-covariant, so rotating each body rigidly about its centre turns
 // the intra-body blocks of M into exactly these; for a single body the
 // rotated inverse is exact.  With several bodies the start's error comes from
 // the inter-body blocks of M, which the move also changes.  One thread per
@@ -270,40 +324,41 @@ __global__ void k_rotate_inverse(int nbl, const int* __restrict__ bob, const dou
 
 // Build the coupled body block for a new configuration: M^-1, P = M^-1 K and
 // N = (K^T M^-1 K)^-1.
-//  - warm: Minv holds the inverse of the previous configuration's M, built
-//    at the body orientations qold (NULL: unknown).  The start X0 is that
-//    inverse rotated with each body's rotation since (k_rotate_inverse).
-//    The configuration moves little between SEM steps, so X0 is a close
-//    start for the Newton-Schulz iteration X <- X + X (I - M X), which
-//    converges quadratically while ||I - M X|| < 1 (the spectral norm, which
-//    the Frobenius norm bounds).  With ||R0||_F = ||I - M X0||_F at most
-//    kNSMaxStart, kNSIters iterations leave a residual of at most
-//    kNSMaxStart^(2^kNSIters) (FP32 roundoff in practice); each iteration is
-//    two n x n products on the whole GPU, against n sequential pivot steps on
-//    one SM for Gauss-Jordan.
+//  - warm (small matrices, dense_body_warm): Minv holds the inverse of the
+//    previous configuration's M, built at the body orientations qold (NULL:
+//    unknown).  The start X0 is that inverse rotated with each body's
+//    rotation since (k_rotate_inverse).  If ||R0||_F = ||I - M X0||_F (which
+//    bounds the spectral norm) is at most kNSMaxStart, kNSIters Newton-Schulz
+//    steps X <- X + X (I - M X) leave at most kNSMaxStart^(2^kNSIters) (FP32
+//    roundoff in practice).
 //  - otherwise, or when R0 is larger (a first configuration, a large move):
-//    in-place Gauss-Jordan.
-// Mw, Tw, Uw: n3 x n3 FP32 work matrices; ss: one device double; ss_host:
-// pinned host double (the choice needs one read of ||R0||).  Returns true
-// when the warm start was taken.
-constexpr double kNSMaxStart = 0.95;
-constexpr int kNSIters = 8;   // even: the result lands in Minv
+//    blocked Gauss-Jordan (k_gj_step).
+// Mw, Tw, Uw: n3 x n3 FP32 work matrices; Nw: 2 (6 nb)^2 FP64; ss: one device
+// double; ss_host: pinned host double (the choice needs one read of ||R0||).
+constexpr double kNSMaxStart = 0.25;
+constexpr int kNSIters = 4;   // even: the result lands in Minv
+// Up to this size the warm start's eight products take about as long as the
+// blocked inversion (40 us each at n = 252); above it they grow with n^3
+// while the inversion's launches grow with n.
+constexpr int kNSMaxRows = 256;
+bool dense_body_warm(int nbl) { return 3 * nbl <= kNSMaxRows; }
 // The pieces of the set-up, also used one by one by the device-driven SEM
 // step (where the warm-start decision is an IF/ELSE graph node).
-// Warm start: Mw = M of the new configuration, X0 = Minv rotated with each
-// body's rotation since it was built (when qnew and qold are known), and
-// Tw = R0 = I - M X0 with ss[0] = ||R0||_F^2.
-void dense_body_warm_start(int nbl, const int* bob, const double* r, const double* qnew, const double* qold,
-                           double a, double eta, float* Minv, float* Mw, float* Tw, double* ss, cudaStream_t s) {
-  const i64 n3 = 3 * (i64)nbl;
-  launch_k(k_rpy_full, nblk(n3 * n3, 256), 256, 0, s, nbl, r, a, eta, Mw);
+void dense_body_mobility(int nbl, const double* r, const PairMobility& pm, double h, double eta, float* Mw,
+                         cudaStream_t s) {
+  launch_k(k_mobility_full, nblk((i64)nbl * nbl, 128), 128, 0, s, nbl, r, pm, 1.0 / h, 1.0 / (eta * h), Mw);
   note_launch();
+}
+// Warm start: X0 = Minv rotated with each body's rotation since it was built
+// (when qnew and qold are known), and Tw = R0 = I - M X0 with ss[0] = ||R0||_F^2.
+void dense_body_warm_start(int nbl, const int* bob, const double* qnew, const double* qold, float* Minv,
+                           const float* Mw, float* Tw, double* ss, cudaStream_t s) {
   if (qnew && qold) {
     launch_k(k_rotate_inverse, nblk((i64)nbl * nbl, 128), 128, 0, s, nbl, bob, qnew, qold, Minv);
     note_launch();
   }
   cudaMemsetAsync(ss, 0, sizeof(double), s);
-  ns_gemm<0>((int)n3, Mw, Minv, nullptr, Tw, ss, s);
+  ns_gemm<0>(3 * nbl, Mw, Minv, nullptr, Tw, ss, s);
 }
 // kNSIters Newton-Schulz steps from X0 = Minv with R0 in Tw; the result
 // lands in Minv (kNSIters is even).
@@ -317,24 +372,18 @@ void dense_body_ns(int nbl, float* Minv, const float* Mw, float* Tw, float* Uw, 
     float* t = X; X = Y; Y = t;
   }
 }
-// Gauss-Jordan inverse of M into Minv (from Mw when it is not null, else
-// Minv holds M); status = 1 on a zero pivot.
-void dense_body_gj(int nbl, float* Minv, const float* Mw, int* status, cudaStream_t s) {
-  const i64 n3 = 3 * (i64)nbl;
-  if (Mw) cudaMemcpyAsync(Minv, Mw, sizeof(float) * n3 * n3, cudaMemcpyDeviceToDevice, s);
-  launch_k(k_gj_inverse<float>, 1, 1024, 2 * sizeof(float) * n3, s, Minv, (int)n3, status);
-  note_launch();
+void dense_body_gj(int nbl, float* Minv, const float* Mw, float* Uw, int* status, cudaStream_t s) {
+  gj_inverse<float>(3 * nbl, Mw, Minv, Uw, status, s);
 }
-// P = M^-1 K and N = (K^T P)^-1 (FP64 Gauss-Jordan; status = 1 on a zero pivot).
+// P = M^-1 K and N = (K^T P)^-1 (FP64; status = 1 on a zero pivot).
 void dense_body_finish(int nbl, int nb, const int* boff, const double* arm, const float* Minv, float* P, double* N,
-                       int* status, cudaStream_t s) {
+                       double* Nw, int* status, cudaStream_t s) {
   const i64 n3 = 3 * (i64)nbl, m = 6 * (i64)nb;
   launch_k(k_mk, nblk(n3 * m, 256), 256, 0, s, nbl, nb, boff, arm, Minv, P);
   note_launch();
-  launch_k(k_ktp, nblk(m * m, 256), 256, 0, s, nbl, nb, boff, arm, P, N);
+  launch_k(k_ktp, nblk(m * m, 256), 256, 0, s, nbl, nb, boff, arm, P, Nw);
   note_launch();
-  launch_k(k_gj_inverse<double>, 1, 1024, 2 * sizeof(double) * m, s, N, (int)m, status);
-  note_launch();
+  gj_inverse<double>((int)m, Nw, N, Nw + m * m, status, s);
 }
 
 // IF/ELSE condition of the device-driven warm start: ||R0||_F <= kNSMaxStart;
@@ -352,33 +401,25 @@ void ns_decide(const double* ss, cudaGraphConditionalHandle h, long long* warm, 
 }
 
 cudaError_t dense_body_build(int nbl, int nb, const int* boff, const int* bob, const double* r, const double* arm,
-                             const double* qnew, const double* qold, double a, double eta, float* Minv, float* P,
-                             double* N, int* status, float* Mw, float* Tw, float* Uw, double* ss, double* ss_host,
-                             bool warm, cudaStream_t s, bool* used_out) {
-  const i64 n3 = 3 * (i64)nbl;
+                             const double* qnew, const double* qold, const PairMobility& pm, double h, double eta,
+                             float* Minv, float* P, double* N, int* status, float* Mw, float* Tw, float* Uw,
+                             double* Nw, double* ss, double* ss_host, bool warm, cudaStream_t s, bool* used_out) {
   cudaError_t e;
 #define RB_CK(call)                      \
   if ((e = (call)) != cudaSuccess) return e
   RB_CK(cudaMemsetAsync(status, 0, sizeof(int), s));
   bool used = false;
   *used_out = false;
-  if (warm) {
-    dense_body_warm_start(nbl, bob, r, qnew, qold, a, eta, Minv, Mw, Tw, ss, s);
+  dense_body_mobility(nbl, r, pm, h, eta, Mw, s);
+  if (warm && dense_body_warm(nbl)) {
+    dense_body_warm_start(nbl, bob, qnew, qold, Minv, Mw, Tw, ss, s);
     RB_CK(cudaMemcpyAsync(ss_host, ss, sizeof(double), cudaMemcpyDeviceToHost, s));
     RB_CK(cudaStreamSynchronize(s));
-    const double r0 = std::sqrt(std::max(ss_host[0], 0.0));
-    if (r0 <= kNSMaxStart) {
-      dense_body_ns(nbl, Minv, Mw, Tw, Uw, ss, s);
-      used = true;
-    } else {
-      dense_body_gj(nbl, Minv, Mw, status, s);
-    }
-  } else {
-    launch_k(k_rpy_full, nblk(n3 * n3, 256), 256, 0, s, nbl, r, a, eta, Minv);
-    note_launch();
-    dense_body_gj(nbl, Minv, nullptr, status, s);
+    used = std::sqrt(std::max(ss_host[0], 0.0)) <= kNSMaxStart;
   }
-  dense_body_finish(nbl, nb, boff, arm, Minv, P, N, status, s);
+  if (used) dense_body_ns(nbl, Minv, Mw, Tw, Uw, ss, s);
+  else dense_body_gj(nbl, Minv, Mw, Uw, status, s);
+  dense_body_finish(nbl, nb, boff, arm, Minv, P, N, Nw, status, s);
   *used_out = used;
   return cudaGetLastError();
 #undef RB_CK

@@ -8,6 +8,8 @@
 
 namespace rbfib {
 
+struct PairMobility;   // pair_mobility.cuh
+
 struct Walls { double v[6][3]; };   // wall velocities, walls -x,+x,-y,+y,-z,+z
 
 // Device views of the bodies of one configuration.
@@ -160,15 +162,18 @@ void adjoint_positions(const Dims&, int nbl, const int* bob, const double* r, co
 
 // k_body.cu
 cudaError_t dense_body_build(int nbl, int nb, const int* boff, const int* bob, const double* r, const double* arm,
-                             const double* qnew, const double* qold, double a, double eta, float* Minv, float* P,
-                             double* N, int* status, float* Mw, float* Tw, float* Uw, double* ss, double* ss_host,
-                             bool warm, cudaStream_t, bool* used);
-void dense_body_warm_start(int nbl, const int* bob, const double* r, const double* qnew, const double* qold,
-                           double a, double eta, float* Minv, float* Mw, float* Tw, double* ss, cudaStream_t);
+                             const double* qnew, const double* qold, const PairMobility& pm, double h, double eta,
+                             float* Minv, float* P, double* N, int* status, float* Mw, float* Tw, float* Uw,
+                             double* Nw, double* ss, double* ss_host, bool warm, cudaStream_t, bool* used);
+bool dense_body_warm(int nbl);   // whether this size takes the warm start at all
+void dense_body_mobility(int nbl, const double* r, const PairMobility& pm, double h, double eta, float* Mw,
+                         cudaStream_t);
+void dense_body_warm_start(int nbl, const int* bob, const double* qnew, const double* qold, float* Minv,
+                           const float* Mw, float* Tw, double* ss, cudaStream_t);
 void dense_body_ns(int nbl, float* Minv, const float* Mw, float* Tw, float* Uw, double* ss, cudaStream_t);
-void dense_body_gj(int nbl, float* Minv, const float* Mw, int* status, cudaStream_t);
+void dense_body_gj(int nbl, float* Minv, const float* Mw, float* Uw, int* status, cudaStream_t);
 void dense_body_finish(int nbl, int nb, const int* boff, const double* arm, const float* Minv, float* P, double* N,
-                       int* status, cudaStream_t);
+                       double* Nw, int* status, cudaStream_t);
 void ns_decide(const double* ss, cudaGraphConditionalHandle h, long long* warm, cudaStream_t);
 // With tab (the configuration's stencil table of type T), the kernel forms
 // its input s = rl + J v itself and stores it in sres_out; sres is unused.

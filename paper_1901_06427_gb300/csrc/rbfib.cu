@@ -15,6 +15,7 @@
 #include "../../include/rbfib.h"
 #include "common.cuh"
 #include "kernels.cuh"
+#include "pair_mobility.cuh"
 
 using namespace rbfib;
 
@@ -29,10 +30,6 @@ namespace {
 
 const double kDeltaDefault = 6.0554544523933395e-06;   // eps^(1/3), eps = 2^-52
 const double kInnerTol = 1e-4;   // relative reduction asked of each FP32 refinement sweep
-// Hydrodynamic radius of a blob in units of h, for the free-space RPY
-// mobilities of the body-block preconditioner only: 0.91 for the
-// three-point kernel; 1.47 for the six-point kernel (Sec. III.C).
-double blob_radius(int kw) { return kw == 6 ? 1.47 : 0.91; }
 const int kDenseBodyMaxRows = 1536;                      // 3 N_bl limit of the coupled body block
 const int kDenseBodyMaxBodyRows = 384;                   // 6 N_b limit of the coupled body block
 
@@ -160,8 +157,9 @@ struct rbfib_grid {
   DBuf<float> minv32, sres32;
   // coupled (all-blob) body block for small suspensions
   bool dense_body = false;
+  PairMobility pair{};   // blob pair functions of the grid's kernel
   DBuf<float> dM, dP;
-  DBuf<double> dN;
+  DBuf<double> dN, dNw;
   DBuf<int> dstatus;
   // Newton-Schulz update of dM from the previous configuration's inverse:
   // work matrices, the residual norm, whether dM holds a valid inverse, and
@@ -487,7 +485,7 @@ template <> float* sres_of<float>(rbfib_grid* g) { return g->sres32; }
 // the mass term's part does in preconditioners of the unsteady Stokes
 // problem (Cahouet and Chabard).  See pressure_kappa.
 // Body block: Schur complement [-M K; K^T 0] with M replaced per body by the
-// free-space RPY blob mobility of its shape, right-hand side
+// free-space blob mobility of its shape (pair_mobility.cuh), right-hand side
 // (r_lam + J v, r_U).
 // z64 (optional): the result is also written in FP64 there by the kernels
 // that produce each block, which saves a conversion launch.
@@ -997,31 +995,17 @@ bool spd_inverse(std::vector<double>& A, int n) {
   return true;
 }
 
-// free-space Rotne-Prager-Yamakawa blob mobility of blobs x (n x 3), radius a
-void rpy_matrix(const double* x, int nbp, double a, double eta, std::vector<double>& M) {
+// free-space mobility of blobs x (n x 3) (pair_mobility.cuh)
+void pair_matrix(const double* x, int nbp, const PairMobility& P, double h, double eta, std::vector<double>& M) {
   const int n3 = 3 * nbp;
   M.assign((size_t)n3 * n3, 0.0);
-  const double c0 = 1.0 / (6.0 * M_PI * eta * a);
   for (int i = 0; i < nbp; ++i)
     for (int j = 0; j < nbp; ++j) {
-      double dvec[3] = {x[3 * i] - x[3 * j], x[3 * i + 1] - x[3 * j + 1], x[3 * i + 2] - x[3 * j + 2]};
-      const double r = std::sqrt(dvec[0] * dvec[0] + dvec[1] * dvec[1] + dvec[2] * dvec[2]);
-      double fI, fR;
-      if (i == j) { fI = c0; fR = 0.0; }
-      else if (r >= 2.0 * a) {
-        const double c = 1.0 / (8.0 * M_PI * eta * r);
-        fI = c * (1.0 + 2.0 * a * a / (3.0 * r * r));
-        fR = c * (1.0 - 2.0 * a * a / (r * r));
-      } else {
-        fI = c0 * (1.0 - 9.0 * r / (32.0 * a));
-        fR = c0 * (3.0 * r / (32.0 * a));
-      }
+      const double d[3] = {(x[3 * i] - x[3 * j]) / h, (x[3 * i + 1] - x[3 * j + 1]) / h, (x[3 * i + 2] - x[3 * j + 2]) / h};
+      double B[9];
+      pair_block(P, d, i == j, B);
       for (int p = 0; p < 3; ++p)
-        for (int q = 0; q < 3; ++q) {
-          double v = (p == q ? fI : 0.0);
-          if (i != j) v += fR * dvec[p] * dvec[q] / (r * r);
-          M[(size_t)(3 * i + p) * n3 + 3 * j + q] = v;
-        }
+        for (int q = 0; q < 3; ++q) M[(size_t)(3 * i + p) * n3 + 3 * j + q] = B[3 * p + q] / (eta * h);
     }
 }
 
@@ -1061,16 +1045,20 @@ void build_body_block(rbfib_grid* g, const double* r, const double* arm, const d
     // captured: the warm start (the step graph is built only when the block
     // holds a valid inverse) with the choice between Newton-Schulz and
     // Gauss-Jordan made on the device; the status goes to dinfo[13]
-    const double a = blob_radius(g->d.kw) * g->desc.h;
     ck(cudaMemsetAsync(g->dstatus, 0, sizeof(int), g->s));
-    dense_body_warm_start(g->nbl, g->bob, r, quat, qold, a, g->desc.eta, g->dM, g->dMw, g->dTw, g->dss, g->s);
-    const cudaGraphConditionalHandle h = new_handle(g, 0u);
-    ns_decide(g->dss, h, g->dwarm, g->s);
-    cond_node(g, h, cudaGraphCondTypeIf, 2, [&](int branch) {
-      if (branch == 0) dense_body_ns(g->nbl, g->dM, g->dMw, g->dTw, g->dUw, g->dss, g->s);
-      else dense_body_gj(g->nbl, g->dM, g->dMw, g->dstatus, g->s);
-    });
-    dense_body_finish(g->nbl, g->nb, g->boff, arm, g->dM, g->dP, g->dN, g->dstatus, g->s);
+    dense_body_mobility(g->nbl, r, g->pair, g->desc.h, g->desc.eta, g->dMw, g->s);
+    if (dense_body_warm(g->nbl)) {
+      dense_body_warm_start(g->nbl, g->bob, quat, qold, g->dM, g->dMw, g->dTw, g->dss, g->s);
+      const cudaGraphConditionalHandle h = new_handle(g, 0u);
+      ns_decide(g->dss, h, g->dwarm, g->s);
+      cond_node(g, h, cudaGraphCondTypeIf, 2, [&](int branch) {
+        if (branch == 0) dense_body_ns(g->nbl, g->dM, g->dMw, g->dTw, g->dUw, g->dss, g->s);
+        else dense_body_gj(g->nbl, g->dM, g->dMw, g->dUw, g->dstatus, g->s);
+      });
+    } else {
+      dense_body_gj(g->nbl, g->dM, g->dMw, g->dUw, g->dstatus, g->s);
+    }
+    dense_body_finish(g->nbl, g->nb, g->boff, arm, g->dM, g->dP, g->dN, g->dNw, g->dstatus, g->s);
     ck(cudaMemcpyAsync(g->dinfo.p + 13, g->dstatus.p, sizeof(int), cudaMemcpyDeviceToDevice, g->s));
     if (quat) ck(cudaMemcpyAsync(g->dquat.p, quat, sizeof(double) * 4 * g->nb, cudaMemcpyDeviceToDevice, g->s));
     return;
@@ -1078,9 +1066,8 @@ void build_body_block(rbfib_grid* g, const double* r, const double* arm, const d
   bool used = false;
   const bool warm = g->dM_valid;
   g->dM_valid = false;
-  ck(dense_body_build(g->nbl, g->nb, g->boff, g->bob, r, arm, quat, qold, blob_radius(g->d.kw) * g->desc.h, g->desc.eta,
-                      g->dM, g->dP, g->dN, g->dstatus, g->dMw, g->dTw, g->dUw, g->dss, g->h_pinned + 40, warm, g->s,
-                      &used));
+  ck(dense_body_build(g->nbl, g->nb, g->boff, g->bob, r, arm, quat, qold, g->pair, g->desc.h, g->desc.eta, g->dM, g->dP,
+                      g->dN, g->dstatus, g->dMw, g->dTw, g->dUw, g->dNw, g->dss, g->h_pinned + 40, warm, g->s, &used));
   int* hstat = (int*)(g->h_pinned + 42);
   ck(cudaMemcpyAsync(hstat, g->dstatus, sizeof(int), cudaMemcpyDeviceToHost, g->s));
   ck(cudaStreamSynchronize(g->s));
@@ -1362,6 +1349,7 @@ int rbfib_create_grid(const rbfib_grid_desc* desc, void* stream, rbfib_grid** ou
     g->nfl = g->nf + g->nc;
     g->dV = D.h * D.h * D.h;
     g->kappa = pressure_kappa(g->d);
+    g->pair = pair_mobility(D.kernel);
     build_stress_layout(g);
     g->nparts = 152 * 4;
     g->part.alloc(part_buffer_doubles(g->nparts));
@@ -1497,6 +1485,7 @@ int rbfib_set_bodies(rbfib_grid* g, int32_t n_bodies, const int32_t* blob_offset
       g->dquat.alloc(4 * (size_t)nb);
       g->dP.alloc((size_t)18 * nbl * nb);
       g->dN.alloc((size_t)36 * nb * nb);
+      g->dNw.alloc((size_t)72 * nb * nb);
       g->dstatus.alloc(1);
     }
     refresh_config(g, g->cur, true);
@@ -1530,7 +1519,7 @@ int rbfib_set_bodies(rbfib_grid* g, int32_t n_bodies, const int32_t* blob_offset
     }
     g->Lp.alloc(std::max(nb, 1));
     ck(cudaMemcpyAsync(g->Lp, Lp.data(), sizeof(double) * std::max(nb, 1), cudaMemcpyHostToDevice, g->s));
-    // per-shape RPY inverse and body mobility
+    // per-shape inverse blob mobility and body mobility
     const int ns = (int)shape_rep.size();
     std::vector<i64> moff(std::max(ns, 1), 0);
     std::vector<double> minv_all, nmat(36 * (size_t)std::max(ns, 1), 0.0);
@@ -1540,7 +1529,7 @@ int rbfib_set_bodies(rbfib_grid* g, int32_t n_bodies, const int32_t* blob_offset
       const int n = off[p + 1] - off[p];
       const double* x = href.data() + 3 * (size_t)off[p];
       std::vector<double> M;
-      rpy_matrix(x, n, blob_radius(g->d.kw) * g->desc.h, g->desc.eta, M);
+      pair_matrix(x, n, g->pair, g->desc.h, g->desc.eta, M);
       if (!spd_inverse(M, 3 * n)) return fail(g, RBFIB_EINVAL, "set_bodies: blob mobility of a shape is singular");
       moff[s] = (i64)minv_all.size();
       srep[s] = off[p];
