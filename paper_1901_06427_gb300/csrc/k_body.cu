@@ -4,10 +4,13 @@
 // (pair_mobility.cuh; inter-body coupling included).  Built once per
 // configuration: dense M; its inverse (FP32) by blocked Gauss-Jordan or, for
 // small matrices close to the previous configuration's, by Newton-Schulz
-// steps from its inverse; P = M^-1 K; N = (K^T M^-1 K)^-1 (FP64).
-// Applied by one cluster of CTAs.
+// steps from its inverse; P = M^-1 K; N = (K^T M^-1 K)^-1 (FP64); then one
+// matrix that maps the block's input to its output.  Other suspensions use
+// one such matrix per body shape.
 #include <algorithm>
 #include <cmath>
+#include <mutex>
+#include <utility>
 
 #include <cooperative_groups.h>
 
@@ -27,8 +30,18 @@ __global__ void k_mobility_full(int nbl, const double* __restrict__ r, PairMobil
   if (t >= (i64)nbl * nbl) return;
   const int i = (int)(t / nbl), j = (int)(t - (i64)i * nbl);
   const double d[3] = {(r[3 * i] - r[3 * j]) * ih, (r[3 * i + 1] - r[3 * j + 1]) * ih, (r[3 * i + 2] - r[3 * j + 2]) * ih};
+  double raise = 0.0;
+  if (i == j) {
+    int near = 0;
+    for (int k = 0; k < nbl; ++k) {
+      const float x = (float)((r[3 * i] - r[3 * k]) * ih), y = (float)((r[3 * i + 1] - r[3 * k + 1]) * ih),
+                  z = (float)((r[3 * i + 2] - r[3 * k + 2]) * ih);
+      near += x * x + y * y + z * z < (float)(kPairNear * kPairNear);
+    }
+    raise = pair_raise(P, near);
+  }
   double B[9];
-  pair_block(P, d, i == j, B);
+  pair_block(P, d, raise, B);
   float* Mb = M + (i64)(3 * i) * (3 * nbl) + 3 * j;
   for (int p = 0; p < 3; ++p)
     for (int q = 0; q < 3; ++q) Mb[(i64)p * (3 * nbl) + q] = (float)(scale * B[3 * p + q]);
@@ -425,133 +438,211 @@ cudaError_t dense_body_build(int nbl, int nb, const int* boff, const int* bob, c
 #undef RB_CK
 }
 
-// Apply on one cluster of kBodyCtas CTAs: t = M^-1 s; f = r_U + K^T t;
-// U = N f; lam = M^-1 (K U - s) = P U - t with P = M^-1 K from the set-up.
-// The rows of t, U and lam are split over the CTAs; t and U are exchanged
-// through distributed shared memory.  s, r_U in, lam, U out (type T;
-// internal FP32 / FP64).  With tab set, the kernel first forms
-// s = r_lam + J v itself (one warp per blob component over the cluster,
-// written to sres, then a cluster barrier), which saves a launch.
-constexpr int kBodyCtas = 8;
-
-template <typename T>
-__global__ void __cluster_dims__(kBodyCtas, 1, 1) __launch_bounds__(512)
-    k_dense_body_apply(int nbl, int nb, const int* __restrict__ boff, const int* __restrict__ bob,
-                       const double* __restrict__ arm, const float* __restrict__ Mi, const float* __restrict__ P,
-                       const double* __restrict__ N, const T* __restrict__ sres, const T* __restrict__ rU,
-                       T* __restrict__ zlam, T* __restrict__ zU, double* __restrict__ zlam64,
-                       double* __restrict__ zU64, Dims d, const BlobStencil<T>* __restrict__ tab,
-                       const T* __restrict__ v, const T* __restrict__ rl, T* __restrict__ sres_out) {
+// The block as one matrix.  With P = M^-1 K and N = (K^T P)^-1 the solution
+// of [-M K; K^T 0] (lambda, U) = (-s, r_U) is linear in (s, r_U):
+//   [lambda]   [E P^T - M^-1  E] [s  ]
+//   [U     ] = [E^T           N] [r_U],   E = P N,
+// so one product replaces the chain M^-1 s -> K^T -> N -> P U - t, whose four
+// dependent steps cost a cluster barrier or a run of FP64 latency each.
+// E: one thread per entry, FP64 sums.
+__global__ void k_body_e(int n3, int m, const float* __restrict__ P, const double* __restrict__ N,
+                         float* __restrict__ E) {
   pdl_entry();
-  namespace cg = cooperative_groups;
-  cg::cluster_group cl = cg::this_cluster();
-  extern __shared__ unsigned char shraw[];
-  const int n3 = 3 * nbl, m = 6 * nb;
-  const int rank = (int)cl.block_rank();
-  const int rpc = (n3 + kBodyCtas - 1) / kBodyCtas, upc = (m + kBodyCtas - 1) / kBodyCtas;
-  const int r0 = rank * rpc, r1 = min(n3, r0 + rpc);
-  const int u0 = rank * upc, u1 = min(m, u0 + upc);
-  double* f = (double*)shraw;      // m
-  double* Uall = f + m;            // m
-  double* Uloc = Uall + m;         // upc (this CTA's rows of U)
-  float* sv = (float*)(Uloc + upc);   // n3
-  float* tloc = sv + n3;              // rpc (this CTA's rows of t)
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  if (tab) {
-    for (int c = rank * nw + wid; c < n3; c += kBodyCtas * nw) {
-      const T jv = warp_interp<T>(d, c % 3, tab + c, v, lane);
-      if (lane == 0) sres_out[c] = rl[c] + jv;
-    }
-    cl.sync();   // release / acquire at cluster scope: every CTA's rows of s are visible
-    for (int i = threadIdx.x; i < n3; i += blockDim.x) sv[i] = (float)__ldcg(sres_out + i);
-  } else {
-    for (int i = threadIdx.x; i < n3; i += blockDim.x) sv[i] = (float)sres[i];
+  const i64 t = (i64)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= (i64)n3 * m) return;
+  const int r = (int)(t / m), c = (int)(t - (i64)r * m);
+  double a0 = 0.0, a1 = 0.0;
+  int k = 0;
+  for (; k + 1 < m; k += 2) {
+    a0 = fma((double)P[(i64)r * m + k], N[(i64)k * m + c], a0);
+    a1 = fma((double)P[(i64)r * m + k + 1], N[(i64)(k + 1) * m + c], a1);
   }
-  __syncthreads();
-  // rows of t = M^-1 s, one warp per row
-  for (int row = r0 + wid; row < r1; row += nw) {
-    const float* Mr = Mi + (i64)row * n3;
-    float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
-    int c = lane;
-    for (; c + 96 < n3; c += 128) {
-      a0 = fmaf(Mr[c], sv[c], a0);
-      a1 = fmaf(Mr[c + 32], sv[c + 32], a1);
-      a2 = fmaf(Mr[c + 64], sv[c + 64], a2);
-      a3 = fmaf(Mr[c + 96], sv[c + 96], a3);
-    }
-    for (; c < n3; c += 32) a0 = fmaf(Mr[c], sv[c], a0);
-    float acc = (a0 + a1) + (a2 + a3);
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) tloc[row - r0] = acc;
-  }
-  cl.sync();
-  // f = r_U + K^T t (every CTA, t read from its owners)
-  for (int p = wid; p < nb; p += nw) {
-    double acc[6] = {0, 0, 0, 0, 0, 0};
-    for (int i = boff[p] + lane; i < boff[p + 1]; i += 32) {
-      double t3[3];
-      for (int a = 0; a < 3; ++a) {
-        const int row = 3 * i + a, owner = row / rpc;
-        const float* tr = cl.map_shared_rank(tloc, owner);
-        t3[a] = tr[row - owner * rpc];
-      }
-      const double x = t3[0], y = t3[1], z = t3[2];
-      const double* d = arm + 3 * i;
-      acc[0] += x; acc[1] += y; acc[2] += z;
-      acc[3] += d[1] * z - d[2] * y;
-      acc[4] += d[2] * x - d[0] * z;
-      acc[5] += d[0] * y - d[1] * x;
-    }
-    for (int c = 0; c < 6; ++c)
-      for (int o = 16; o > 0; o >>= 1) acc[c] += __shfl_xor_sync(0xffffffffu, acc[c], o);
-    if (lane < 6) f[6 * p + lane] = acc[lane] + (double)rU[6 * p + lane];
-  }
-  __syncthreads();
-  // this CTA's rows of U = N f
-  for (int r = u0 + (int)threadIdx.x; r < u1; r += blockDim.x) {
-    double acc = 0.0;
-    for (int c = 0; c < m; ++c) acc = fma(N[(i64)r * m + c], f[c], acc);
-    Uloc[r - u0] = acc;
-    zU[r] = (T)acc;
-    if (zU64) zU64[r] = (double)(T)acc;
-  }
-  cl.sync();
-  for (int c = threadIdx.x; c < m; c += blockDim.x) {
-    const int owner = c / upc;
-    Uall[c] = cl.map_shared_rank(Uloc, owner)[c - owner * upc];
-  }
-  __syncthreads();
-  // this CTA's rows of lam = P U - t
-  for (int row = r0 + (int)threadIdx.x; row < r1; row += blockDim.x) {
-    const float* Pr = P + (i64)row * m;
-    float acc = -tloc[row - r0];
-    for (int c = 0; c < m; ++c) acc = fmaf(Pr[c], (float)Uall[c], acc);
-    zlam[row] = (T)acc;
-    if (zlam64) zlam64[row] = (double)(T)acc;
-  }
-  cl.sync();   // no CTA leaves while another may still read its shared memory
+  if (k < m) a0 = fma((double)P[(i64)r * m + k], N[(i64)k * m + c], a0);
+  E[t] = (float)(a0 + a1);
 }
 
-template <typename T>
-void dense_body_apply(int nbl, int nb, const int* boff, const int* bob, const double* arm, const float* Minv,
-                      const float* P, const double* N, const T* sres, const T* rU, T* zlam, T* zU, double* zlam64,
-                      double* zU64, cudaStream_t s, const Dims* d, const BlobStencil<T>* tab, const T* v,
-                      const T* rl, T* sres_out) {
-  const int n3 = 3 * nbl, m = 6 * nb;
-  const int rpc = (n3 + kBodyCtas - 1) / kBodyCtas, upc = (m + kBodyCtas - 1) / kBodyCtas;
-  const size_t shm = sizeof(double) * (2 * (size_t)m + upc) + sizeof(float) * ((size_t)n3 + rpc);
-  launch_k(k_dense_body_apply<T>, kBodyCtas, 512, shm, s, nbl, nb, boff, bob, arm, Minv, P, N, sres, rU, zlam, zU,
-           zlam64, zU64, d ? *d : Dims{}, tab, v, rl, sres_out);
+// The matrix B (rows of ld floats), 32 x 32 tiles of 256 threads.
+__global__ void __launch_bounds__(256) k_body_matrix(int n3, int m, int ld, const float* __restrict__ Mi,
+                                                     const float* __restrict__ P, const float* __restrict__ E,
+                                                     const double* __restrict__ N, float* __restrict__ B) {
+  pdl_entry();
+  __shared__ float Es[32][33], Ps[32][33];
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  const int r0 = blockIdx.y * 32, c0 = blockIdx.x * 32, n = n3 + m;
+  float acc[4] = {0.f, 0.f, 0.f, 0.f};
+  for (int k0 = 0; k0 < m; k0 += 32) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int r = r0 + ty + 8 * q, c = c0 + ty + 8 * q, k = k0 + tx;
+      Es[ty + 8 * q][tx] = r < n3 && k < m ? E[(i64)r * m + k] : 0.f;
+      Ps[ty + 8 * q][tx] = c < n3 && k < m ? P[(i64)c * m + k] : 0.f;
+    }
+    __syncthreads();
+    for (int k = 0; k < 32; ++k)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) acc[q] = fmaf(Es[ty + 8 * q][k], Ps[tx][k], acc[q]);
+    __syncthreads();
+  }
+  const int c = c0 + tx;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int r = r0 + ty + 8 * q;
+    if (r >= n || c >= ld) continue;
+    float v = 0.f;
+    if (c < n) {
+      if (r < n3) v = c < n3 ? acc[q] - Mi[(i64)r * n3 + c] : E[(i64)r * m + c - n3];
+      else v = c < n3 ? E[(i64)c * m + r - n3] : (float)N[(i64)(r - n3) * m + c - n3];
+    }
+    B[(i64)r * ld + c] = v;
+  }
+}
+
+void dense_body_matrix(int nbl, int nb, const float* Minv, const float* P, const double* N, float* E, float* B,
+                       cudaStream_t s) {
+  const int n3 = 3 * nbl, m = 6 * nb, ld = body_ld(n3 + m);
+  launch_k(k_body_e, nblk((i64)n3 * m, 256), 256, 0, s, n3, m, P, N, E);
+  note_launch();
+  launch_k(k_body_matrix, dim3((ld + 31) / 32, (n3 + m + 31) / 32), 256, 0, s, n3, m, ld, Minv, P, E, N, B);
   note_launch();
 }
 
-template void dense_body_apply<float>(int, int, const int*, const int*, const double*, const float*, const float*,
-                                      const double*, const float*, const float*, float*, float*, double*, double*,
-                                      cudaStream_t, const Dims*, const BlobStencil<float>*, const float*, const float*,
-                                      float*);
-template void dense_body_apply<double>(int, int, const int*, const int*, const double*, const float*,
-                                       const float*, const double*, const double*, const double*, double*, double*,
-                                       double*, double*, cudaStream_t, const Dims*, const BlobStencil<double>*,
-                                       const double*, const double*, double*);
+// One row of the block's matrix times x (shared memory), by a warp; the row's
+// first kBodyPre 16-byte words of each lane come from registers.
+constexpr int kBodyPre = 3;
+RBFIB_DEVFN float4 body_word(const float* __restrict__ row, int ld, int w) {
+  return 4 * w < ld ? __ldg(reinterpret_cast<const float4*>(row) + w) : make_float4(0.f, 0.f, 0.f, 0.f);
+}
+RBFIB_DEVFN float body_row(const float* __restrict__ row, const float4 pre[kBodyPre], const float* x, int ld, int lane) {
+  float a[4] = {0.f, 0.f, 0.f, 0.f};
+  auto add = [&](const float4& b, int w) {
+    if (4 * w >= ld) return;
+    const float4 v = *reinterpret_cast<const float4*>(x + 4 * w);
+    a[0] = fmaf(b.x, v.x, a[0]);
+    a[1] = fmaf(b.y, v.y, a[1]);
+    a[2] = fmaf(b.z, v.z, a[2]);
+    a[3] = fmaf(b.w, v.w, a[3]);
+  };
+#pragma unroll
+  for (int q = 0; q < kBodyPre; ++q) add(pre[q], lane + 32 * q);
+  for (int w = lane + 32 * kBodyPre; 4 * w < ld; w += 32) add(body_word(row, ld, w), w);
+  float t = (a[0] + a[1]) + (a[2] + a[3]);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  return t;
+}
+
+// Coupled block, z = B (r_lambda + J v, r_U).  Every cluster of 8 CTAs forms
+// the whole input, one warp per blob component over the cluster, each value
+// written to all eight CTAs through distributed shared memory; after the one
+// cluster barrier (the gather's latency hides the first rows' loads, issued
+// before it) the rows are split over the CTAs of all clusters.
+constexpr int kBodyCtas = 8, kBodyThreads = 512;
+__global__ void __cluster_dims__(kBodyCtas, 1, 1) __launch_bounds__(kBodyThreads)
+    k_dense_body_apply(int n3, int m, int ld, const float* __restrict__ B, const float* __restrict__ r,
+                       float* __restrict__ z, double* __restrict__ z64, Dims d, const BlobStencil<float>* __restrict__ tab,
+                       const float* __restrict__ v) {
+  pdl_entry();
+  namespace cg = cooperative_groups;
+  cg::cluster_group cl = cg::this_cluster();
+  extern __shared__ __align__(16) float sv[];   // ld
+  const int n = n3 + m;
+  const int rpc = (n + gridDim.x - 1) / gridDim.x;
+  const int r0 = blockIdx.x * rpc, r1 = min(n, r0 + rpc);
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = kBodyThreads / 32;
+  // every CTA of the cluster must have started before its memory is written
+  auto started = cl.barrier_arrive();
+  float4 pre[kBodyPre];
+  if (r0 + wid < r1)
+#pragma unroll
+    for (int q = 0; q < kBodyPre; ++q) pre[q] = body_word(B + (i64)(r0 + wid) * ld, ld, lane + 32 * q);
+  cl.barrier_wait(std::move(started));
+  for (int c = (int)cl.block_rank() * nw + wid; c < n3; c += kBodyCtas * nw) {
+    const float s = r[c] + warp_interp<float>(d, c % 3, tab + c, v, lane);
+    if (lane < kBodyCtas) cl.map_shared_rank(sv, lane)[c] = s;
+  }
+  for (int i = n3 + threadIdx.x; i < ld; i += kBodyThreads) sv[i] = i < n ? r[i] : 0.f;
+  cl.sync();
+  for (int row = r0 + wid; row < r1; row += nw) {
+    if (row != r0 + wid)
+#pragma unroll
+      for (int q = 0; q < kBodyPre; ++q) pre[q] = body_word(B + (i64)row * ld, ld, lane + 32 * q);
+    const float t = body_row(B + (i64)row * ld, pre, sv, ld, lane);
+    if (lane == 0) {
+      z[row] = t;
+      if (z64) z64[row] = (double)t;
+    }
+  }
+}
+
+void dense_body_apply(int nbl, int nb, const float* B, const float* r, float* z, double* z64, const Dims& d,
+                      const BlobStencil<float>* tab, const float* v, cudaStream_t s) {
+  const int n3 = 3 * nbl, m = 6 * nb, ld = body_ld(n3 + m);
+  // about four rows per warp at most
+  const int clusters = std::max(1, (n3 + m + 4 * kBodyCtas * (kBodyThreads / 32) - 1) / (4 * kBodyCtas * (kBodyThreads / 32)));
+  launch_k(k_dense_body_apply, kBodyCtas * clusters, kBodyThreads, sizeof(float) * ld, s, n3, m, ld, B, r, z, z64, d, tab, v);
+  note_launch();
+}
+
+// Per-body block: the matrix of each body's shape (B_s, in the body frame, of
+// n_s = 3 blobs + 6 rows; host-built, all shapes one after the other), one
+// CTA per body: input gathered, its three-vectors (blob velocities, force,
+// torque) turned into the body frame, product, turned back.
+__global__ void __launch_bounds__(256) k_body_apply(int nbl, const int* __restrict__ boff, const int* __restrict__ shape_of,
+                                                    const i64* __restrict__ shape_off, const float* __restrict__ Bs,
+                                                    const double* __restrict__ quat, const float* __restrict__ r,
+                                                    float* __restrict__ z, double* __restrict__ z64, Dims d,
+                                                    const BlobStencil<float>* __restrict__ tab, const float* __restrict__ v) {
+  pdl_entry();
+  extern __shared__ __align__(16) float sh[];
+  const int p = blockIdx.x, b0 = boff[p], n3 = 3 * (boff[p + 1] - b0), n = n3 + 6, ld = body_ld(n);
+  const float* B = Bs + shape_off[shape_of[p]];
+  float* x = sh;        // input in the lab, later the result in the body frame
+  float* y = sh + ld;   // input in the body frame
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  float4 pre[kBodyPre];
+  if (wid < n)
+#pragma unroll
+    for (int q = 0; q < kBodyPre; ++q) pre[q] = body_word(B + (i64)wid * ld, ld, lane + 32 * q);
+  double R[9];
+  quat_rot(quat + 4 * p, R);
+  for (int c = wid; c < n3; c += nw) {
+    const float s = r[3 * b0 + c] + warp_interp<float>(d, c % 3, tab + 3 * b0 + c, v, lane);
+    if (lane == 0) x[c] = s;
+  }
+  if (threadIdx.x < 6) x[n3 + threadIdx.x] = r[3 * nbl + 6 * p + threadIdx.x];
+  if (n + (int)threadIdx.x < ld) y[n + threadIdx.x] = 0.f;
+  __syncthreads();
+  for (int i = threadIdx.x; i < n / 3; i += blockDim.x)
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+      y[3 * i + a] = (float)(R[a] * (double)x[3 * i] + R[3 + a] * (double)x[3 * i + 1] + R[6 + a] * (double)x[3 * i + 2]);
+  __syncthreads();
+  for (int row = wid; row < n; row += nw) {
+    if (row != wid)
+#pragma unroll
+      for (int q = 0; q < kBodyPre; ++q) pre[q] = body_word(B + (i64)row * ld, ld, lane + 32 * q);
+    const float t = body_row(B + (i64)row * ld, pre, y, ld, lane);
+    if (lane == 0) x[row] = t;
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < n / 3; i += blockDim.x) {
+    const int o = 3 * i < n3 ? 3 * (b0 + i) : 3 * nbl + 6 * p + 3 * i - n3;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      const float t = (float)(R[3 * a] * (double)x[3 * i] + R[3 * a + 1] * (double)x[3 * i + 1] + R[3 * a + 2] * (double)x[3 * i + 2]);
+      z[o + a] = t;
+      if (z64) z64[o + a] = (double)t;
+    }
+  }
+}
+
+void body_apply(const BodyView& b, const ShapeView& sv, const float* r, float* z, double* z64, const Dims& d,
+                const float* v, cudaStream_t s) {
+  const size_t shm = 2 * sizeof(float) * (size_t)body_ld(3 * sv.max_blobs + 6);
+  static std::once_flag f;
+  std::call_once(f, [] { cudaFuncSetAttribute(k_body_apply, cudaFuncAttributeMaxDynamicSharedMemorySize, kBodyMaxSmem); });
+  launch_k(k_body_apply, b.nb, 256, shm, s, b.nbl, b.boff, sv.shape_of, sv.off, sv.B, b.quat, r, z, z64, d, b.st32, v);
+  note_launch();
+}
 
 }  // namespace rbfib

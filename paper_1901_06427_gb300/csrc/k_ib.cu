@@ -1,7 +1,6 @@
 // Immersed-boundary and rigid-body kernels (Sec. III.B): body geometry,
 // blob-to-cell binning, spreading S, interpolation J, the rigid maps K and
-// K^T, the fused body rows of the saddle operator, the body-block
-// preconditioner and the forces of Sec. V.
+// K^T, the fused body rows of the saddle operator and the forces of Sec. V.
 #include "common.cuh"
 #include "kernels.cuh"
 
@@ -266,27 +265,6 @@ RBFIB_DEVFN void warp_spread(const Dims& d, int a, const BlobStencil<T>* __restr
   }
 }
 
-// out = r_lam + J v  (body-block preconditioner input), warp per blob component
-template <typename T>
-__global__ void k_interp_res(Dims d, int nbl, const BlobStencil<T>* __restrict__ tab, const T* __restrict__ v,
-                             const T* __restrict__ rl, T* __restrict__ out) {
-  pdl_entry();
-  const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-  if (gw >= 3 * nbl) return;
-  const T jv = warp_interp<T>(d, gw % 3, tab + gw, v, lane);
-  if (lane == 0) out[gw] = rl[gw] + jv;
-}
-
-template <typename T>
-void interp_res(const Dims& d, const BodyView& b, const T* v, const T* rl, T* out, cudaStream_t s) {
-  if (b.nbl > 0) {
-    const BlobStencil<T>* tab = nullptr;
-    if constexpr (sizeof(T) == 8) tab = (const BlobStencil<T>*)b.st64; else tab = (const BlobStencil<T>*)b.st32;
-    launch_k(k_interp_res<T>, nblk(32 * 3 * (i64)b.nbl, 128), 128, 0, s, d, b.nbl, tab, v, rl, out);
-    note_launch();
-  }
-}
-
 // out = alpha * J v + beta * out with the configuration's table
 template <typename T>
 __global__ void k_interp_tab(Dims d, int nbl, const BlobStencil<T>* __restrict__ tab, const T* __restrict__ v,
@@ -465,120 +443,6 @@ void k_apply(int nbl, const int* bob, const double* arm, const double* U, double
   if (nbl > 0) { launch_k(k_k, nblk(3 * (i64)nbl, 128), 128, 0, s, nbl, bob, arm, U, alpha, beta, out); note_launch(); }
 }
 
-// ------------------------------------------------ body-block preconditioner
-// Per body p of shape s (body frame, rotated by R_p):
-//   s'  = R^T (r_lam + J v~)                (input sres already holds r_lam + J v~)
-//   U'  = N_s (R^T r_U + K_s^T M_s^-1 s')
-//   lam' = M_s^-1 (K_s U' - s')
-//   lam = R lam',  U = (R u', R w')
-// M_s: free-space RPY blob mobility of the shape's reference blobs; N_s =
-// (K_s^T M_s^-1 K_s)^-1; both precomputed on the host.
-template <typename T>
-__global__ void k_body_precond(int nb, const int* __restrict__ boff, const int* __restrict__ shape_of,
-                               const i64* __restrict__ shape_minv_off, const T* __restrict__ minv,
-                               const double* __restrict__ nmat, const int* __restrict__ shape_ref_blob,
-                               const double* __restrict__ ref, const double* __restrict__ quat,
-                               const T* __restrict__ sres, const T* __restrict__ rU,
-                               T* __restrict__ zlam, T* __restrict__ zU, double* __restrict__ zlam64,
-                               double* __restrict__ zU64) {
-  pdl_entry();
-  extern __shared__ unsigned char shraw[];
-  T* sh = (T*)shraw;
-  const int p = blockIdx.x;
-  if (p >= nb) return;
-  const int b0 = boff[p], nbp = boff[p + 1] - b0;
-  const int n3 = 3 * nbp;
-  const int s = shape_of[p];
-  const T* Mi = minv + shape_minv_off[s];
-  const double* Ns = nmat + 36 * s;
-  const double* rf = ref + 3 * shape_ref_blob[s];
-  T* sp = sh;            // n3: s'
-  T* tp = sh + n3;       // n3: M^-1 s', later K U' - s'
-  __shared__ double w6[6];
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  double R[9];
-  quat_rot(quat + 4 * p, R);
-  for (int i = threadIdx.x; i < nbp; i += blockDim.x) {
-    const T* x = sres + 3 * (b0 + i);
-    for (int a = 0; a < 3; ++a)
-      sp[3 * i + a] = (T)(R[a] * (double)x[0] + R[3 + a] * (double)x[1] + R[6 + a] * (double)x[2]);
-  }
-  __syncthreads();
-  // tp = M^-1 sp, one warp per row, lanes over columns (coalesced)
-  for (int row = wid; row < n3; row += nw) {
-    T acc = T(0);
-    for (int c = lane; c < n3; c += 32) acc += Mi[(i64)row * n3 + c] * sp[c];
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) tp[row] = acc;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double f[6] = {0, 0, 0, 0, 0, 0};
-    for (int i = 0; i < nbp; ++i) {
-      const double t0 = tp[3 * i], t1 = tp[3 * i + 1], t2 = tp[3 * i + 2];
-      const double* a = rf + 3 * i;
-      f[0] += t0; f[1] += t1; f[2] += t2;
-      f[3] += a[1] * t2 - a[2] * t1;
-      f[4] += a[2] * t0 - a[0] * t2;
-      f[5] += a[0] * t1 - a[1] * t0;
-    }
-    double ru[6];
-    for (int c = 0; c < 6; ++c) ru[c] = (double)rU[6 * p + c];
-    for (int h = 0; h < 2; ++h)
-      for (int a = 0; a < 3; ++a)
-        f[3 * h + a] += R[a] * ru[3 * h] + R[3 + a] * ru[3 * h + 1] + R[6 + a] * ru[3 * h + 2];
-    for (int r = 0; r < 6; ++r) {
-      double acc = 0.0;
-      for (int c = 0; c < 6; ++c) acc += Ns[6 * r + c] * f[c];
-      w6[r] = acc;
-    }
-  }
-  __syncthreads();
-  for (int i = threadIdx.x; i < nbp; i += blockDim.x) {
-    const double* a = rf + 3 * i;
-    const double kx = w6[0] + (w6[4] * a[2] - w6[5] * a[1]);
-    const double ky = w6[1] + (w6[5] * a[0] - w6[3] * a[2]);
-    const double kz = w6[2] + (w6[3] * a[1] - w6[4] * a[0]);
-    tp[3 * i] = (T)kx - sp[3 * i];
-    tp[3 * i + 1] = (T)ky - sp[3 * i + 1];
-    tp[3 * i + 2] = (T)kz - sp[3 * i + 2];
-  }
-  __syncthreads();
-  for (int row = wid; row < n3; row += nw) {
-    T acc = T(0);
-    for (int c = lane; c < n3; c += 32) acc += Mi[(i64)row * n3 + c] * tp[c];
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) sp[row] = acc;   // lam' (s' no longer needed)
-  }
-  __syncthreads();
-  for (int i = threadIdx.x; i < nbp; i += blockDim.x) {
-    const T* l = sp + 3 * i;
-    for (int a = 0; a < 3; ++a) {
-      const T x = (T)(R[3 * a] * (double)l[0] + R[3 * a + 1] * (double)l[1] + R[3 * a + 2] * (double)l[2]);
-      zlam[3 * (b0 + i) + a] = x;
-      if (zlam64) zlam64[3 * (b0 + i) + a] = (double)x;
-    }
-  }
-  if (threadIdx.x < 6) {
-    const int h = threadIdx.x / 3, a = threadIdx.x % 3;
-    const T u = (T)(R[3 * a] * w6[3 * h] + R[3 * a + 1] * w6[3 * h + 1] + R[3 * a + 2] * w6[3 * h + 2]);
-    zU[6 * p + threadIdx.x] = u;
-    if (zU64) zU64[6 * p + threadIdx.x] = (double)u;
-  }
-}
-
-template <typename T>
-void body_precond(const BodyView& b, const PrecondView& pv, const T* sres, const T* rU, T* zlam, T* zU,
-                  double* zlam64, double* zU64, cudaStream_t s) {
-  if (b.nb == 0) return;
-  const size_t shm = sizeof(T) * (2 * 3 * (size_t)pv.max_blobs + 8);
-  const T* mi = nullptr;
-  if constexpr (sizeof(T) == 8) mi = (const T*)pv.minv; else mi = (const T*)pv.minv32;
-  launch_k(k_body_precond<T>, b.nb, 256, shm, s, b.nb, b.boff, pv.shape_of, pv.minv_off, mi, pv.nmat,
-           pv.shape_ref_blob, b.ref, b.quat, sres, rU, zlam, zU, zlam64, zU64);
-  note_launch();
-}
-
 // ------------------------------------------------------------------ forces
 RBFIB_DEVFN double soft(double r, double phi0, double b, double dd) {
   return (phi0 / b) * (r < dd ? 1.0 : exp((dd - r) / b));
@@ -754,10 +618,7 @@ void outside_check(const Dims& d, int nbl, const double* r, int* flag, cudaStrea
                                  cudaStream_t);                                                          \
   template void spread<T>(const Dims&, int, const int*, const double*, const T*, double, T*, cudaStream_t); \
   template void interp<T>(const Dims&, const Walls&, int, const double*, const T*, double, double, double, \
-                          T*, cudaStream_t);                                                             \
-  template void body_precond<T>(const BodyView&, const PrecondView&, const T*, const T*, T*, T*, double*, double*,        \
-                                cudaStream_t);                                                          \
-  template void interp_res<T>(const Dims&, const BodyView&, const T*, const T*, T*, cudaStream_t);
+                          T*, cudaStream_t);
 INST(double)
 INST(float)
 #undef INST

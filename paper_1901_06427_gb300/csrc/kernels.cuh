@@ -27,14 +27,12 @@ struct BodyView {
   const BlobStencil<float>* st32 = nullptr;
 };
 
-struct PrecondView {
+// Body-block matrices of the body shapes (per-body form).
+struct ShapeView {
   int max_blobs = 0;
-  const int* shape_of = nullptr;
-  const i64* minv_off = nullptr;
-  const double* minv = nullptr;
-  const float* minv32 = nullptr;
-  const double* nmat = nullptr;
-  const int* shape_ref_blob = nullptr;
+  const int* shape_of = nullptr;   // nb
+  const i64* off = nullptr;        // of each shape's matrix in B
+  const float* B = nullptr;
 };
 
 struct Potentials {
@@ -136,10 +134,6 @@ template <typename T> void spread(const Dims&, int nbl, const int* perm, const d
                                   double scale, T* f, cudaStream_t);
 template <typename T> void interp(const Dims&, const Walls&, int nbl, const double* r, const T* v, double alpha,
                                   double beta, double gamma, T* out, cudaStream_t);
-template <typename T> void interp_res(const Dims&, const BodyView&, const T* v, const T* rl, T* out, cudaStream_t);
-// zlam64 / zU64: FP64 copies of the outputs (null: none)
-template <typename T> void body_precond(const BodyView&, const PrecondView&, const T* sres, const T* rU,
-                                        T* zlam, T* zU, double* zlam64, double* zU64, cudaStream_t);
 void stencil_build(const Dims&, int nbl, const double* r, BlobStencil<double>* s64, BlobStencil<float>* s32,
                    cudaStream_t);
 void interp_tab(const Dims&, const BodyView&, const double* v, double alpha, double beta, double* out, cudaStream_t);
@@ -175,14 +169,17 @@ void dense_body_gj(int nbl, float* Minv, const float* Mw, float* Uw, int* status
 void dense_body_finish(int nbl, int nb, const int* boff, const double* arm, const float* Minv, float* P, double* N,
                        double* Nw, int* status, cudaStream_t);
 void ns_decide(const double* ss, cudaGraphConditionalHandle h, long long* warm, cudaStream_t);
-// With tab (the configuration's stencil table of type T), the kernel forms
-// its input s = rl + J v itself and stores it in sres_out; sres is unused.
-template <typename T> void dense_body_apply(int nbl, int nb, const int* boff, const int* bob, const double* arm,
-                                            const float* Minv, const float* P, const double* N, const T* sres,
-                                            const T* rU, T* zlam, T* zU, double* zlam64, double* zU64,
-                                            cudaStream_t, const Dims* d = nullptr,
-                                            const BlobStencil<T>* tab = nullptr, const T* v = nullptr,
-                                            const T* rl = nullptr, T* sres_out = nullptr);
+// Rows of a body-block matrix over n unknowns, in floats.
+__host__ __device__ constexpr int body_ld(int n) { return (n + 3) & ~3; }
+constexpr int kBodyMaxSmem = 160 * 1024;   // the per-body form's input and output: up to 6824 blobs a body
+void dense_body_matrix(int nbl, int nb, const float* Minv, const float* P, const double* N, float* E, float* B,
+                       cudaStream_t);
+// z = block (r_lambda + J v, r_U); r and z: the lambda and U parts of a
+// saddle vector; z64: FP64 copy of the result (null: none)
+void dense_body_apply(int nbl, int nb, const float* B, const float* r, float* z, double* z64, const Dims& d,
+                      const BlobStencil<float>* tab, const float* v, cudaStream_t);
+void body_apply(const BodyView&, const ShapeView&, const float* r, float* z, double* z64, const Dims& d,
+                const float* v, cudaStream_t);
 
 // k_krylov.cu
 // A grid's partial-sum buffer: nparts x kPartCols doubles, 8 spare doubles,

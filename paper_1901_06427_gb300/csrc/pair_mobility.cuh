@@ -26,8 +26,7 @@ constexpr int kPairKnots = 25;          // r = 0, 1/4, ..., 6
 constexpr double kPairStep = 0.25;
 
 // Cubic pieces of f and g, the blob radius of the tail, and what the
-// diagonal of M is raised by: the averages are positive definite only to
-// their statistical error (three-point: the grid's own variation).
+// diagonal of M is raised by (pair_raise).
 struct PairMobility {
   double c[2][kPairKnots - 1][4];
   double a, shift;
@@ -104,14 +103,27 @@ __host__ __device__ inline void pair_functions(const PairMobility& P, double r, 
   }
 }
 
+// The averages are positive definite only to their statistical error
+// (three-point: the grid's own variation), which adds up over blobs that the
+// grid does not resolve.  A blob with more than 32 others (itself included)
+// within 2 h is raised by that much more: shells of 42 to 800 blobs of radius
+// 0.3 to 3 h have smallest eigenvalues down to -7e-4 (500 blobs, radius h / 2)
+// before and above zero after it; ordinary shells have about ten.
+constexpr double kPairNear = 2.0;
+__host__ __device__ inline double pair_raise(const PairMobility& P, int near) {
+  return P.shift * (near > 32 ? near / 32.0 : 1.0);
+}
+
 // The block of two blobs at d = r_i - r_j (in units of h), in units of
-// 1 / (eta h); same: one blob with itself.
-__host__ __device__ inline void pair_block(const PairMobility& P, const double d[3], bool same, double B[9]) {
+// 1 / (eta h).  Two blobs at one place, whose forces cannot be told apart,
+// give NaN: the inversion refuses the matrix.  raise: one blob with itself
+// (else 0).
+__host__ __device__ inline void pair_block(const PairMobility& P, const double d[3], double raise, double B[9]) {
   const double r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
   double f, g;
   pair_functions(P, sqrt(r2), f, g);
   const double w = r2 > 0.0 ? (g - f) / r2 : 0.0;
-  if (same) f += P.shift;
+  f = r2 > 0.0 || raise > 0.0 ? f + raise : nan("");
   for (int p = 0; p < 3; ++p)
     for (int q = 0; q < 3; ++q) B[3 * p + q] = (p == q ? f : 0.0) + w * d[p] * d[q];
 }

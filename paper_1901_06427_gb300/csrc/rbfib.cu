@@ -151,14 +151,13 @@ struct rbfib_grid {
   Config cur, plus, minus, next;
   // body-block preconditioner
   int max_blobs = 0;
-  DBuf<int> shape_of, shape_ref_blob;
-  DBuf<i64> minv_off;
-  DBuf<double> minv, nmat;
-  DBuf<float> minv32, sres32;
+  DBuf<int> shape_of;
+  DBuf<i64> shape_off;
+  DBuf<float> shape_B;
   // coupled (all-blob) body block for small suspensions
   bool dense_body = false;
   PairMobility pair{};   // blob pair functions of the grid's kernel
-  DBuf<float> dM, dP;
+  DBuf<float> dM, dP, dE, dB;
   DBuf<double> dN, dNw;
   DBuf<int> dstatus;
   // Newton-Schulz update of dM from the previous configuration's inverse:
@@ -169,7 +168,7 @@ struct rbfib_grid {
   bool dM_valid = false, dquat_valid = false;
   long long ns_warm = 0;
   // work vectors (FP64)
-  DBuf<double> part, scal, bvec, xvec, xrfd, rres, sres, fsharp, vsharp, fnoise, Wst;
+  DBuf<double> part, scal, bvec, xvec, xrfd, rres, fsharp, vsharp, fnoise, Wst;
   DBuf<double> bodyA, bodyB, bodyF, bodyW, bodyWn, blobA, blobB, blobC, blobD, blobS;
   double* h_pinned = nullptr;
   int nparts = 0;
@@ -290,13 +289,13 @@ BodyView view_of(rbfib_grid* g, Config& c) {
   return b;
 }
 
-PrecondView pview(rbfib_grid* g) {
-  PrecondView p;
-  p.max_blobs = g->max_blobs;
-  p.shape_of = g->shape_of; p.minv_off = g->minv_off; p.minv = g->minv; p.nmat = g->nmat;
-  p.minv32 = g->minv32;
-  p.shape_ref_blob = g->shape_ref_blob;
-  return p;
+ShapeView shapes_of(rbfib_grid* g) {
+  ShapeView v;
+  v.max_blobs = g->max_blobs;
+  v.shape_of = g->shape_of;
+  v.off = g->shape_off;
+  v.B = g->shape_B;
+  return v;
 }
 
 // --------------------------------------------------------------- multigrid
@@ -470,10 +469,6 @@ double pressure_kappa(const Dims& d) {
   return std::min(drag[0] + drag[1], std::min(drag[0] + drag[2], drag[1] + drag[2]));
 }
 
-template <typename T> T* sres_of(rbfib_grid* g);
-template <> double* sres_of<double>(rbfib_grid* g) { return g->sres; }
-template <> float* sres_of<float>(rbfib_grid* g) { return g->sres32; }
-
 // ---------------------------------------------------------- preconditioner
 // Block lower-triangular preconditioner of the saddle operator.
 // Fluid block (projection method): v~ = (-eta LL)^{-1} r_v (V-cycle),
@@ -500,23 +495,12 @@ void precond(rbfib_grid* g, const T* r, T* z, bool with_bodies, double* z64, dou
   div_q<T>(d, zv, r + g->nf, q, g->s);
   vcycle_p<T>(g, phi, q);
   add_grad<T>(d, (T)g->desc.eta, (T)kappa, phi, q, z, z64, g->s);
-  if (with_bodies && g->nb > 0) {
-    const T* rl = r + g->nfl;
-    const T* rU = rl + 3 * (i64)g->nbl;
-    T* zl = z + g->nfl;
-    T* zU = zl + 3 * (i64)g->nbl;
-    T* sres = sres_of<T>(g);
-    double* zl64 = z64 ? z64 + g->nfl : nullptr;
-    double* zU64 = z64 ? zl64 + 3 * (i64)g->nbl : nullptr;
-    if (g->dense_body) {
+  if constexpr (std::is_same<T, float>::value) {
+    if (with_bodies && g->nb > 0) {
       const BodyView bv = view_of(g, g->cur);
-      const BlobStencil<T>* tab = nullptr;
-      if constexpr (sizeof(T) == 8) tab = (const BlobStencil<T>*)bv.st64; else tab = (const BlobStencil<T>*)bv.st32;
-      dense_body_apply<T>(g->nbl, g->nb, g->boff, g->bob, g->cur.arm, g->dM, g->dP, g->dN, nullptr, rU, zl, zU, zl64,
-                          zU64, g->s, &d, tab, zv, rl, sres);
-    } else {
-      interp_res<T>(d, view_of(g, g->cur), zv, rl, sres, g->s);
-      body_precond<T>(view_of(g, g->cur), pview(g), sres, rU, zl, zU, zl64, zU64, g->s);
+      double* zb64 = z64 ? z64 + g->nfl : nullptr;
+      if (g->dense_body) dense_body_apply(g->nbl, g->nb, g->dB, r + g->nfl, z + g->nfl, zb64, d, bv.st32, zv, g->s);
+      else body_apply(bv, shapes_of(g), r + g->nfl, z + g->nfl, zb64, d, zv, g->s);
     }
   }
 }
@@ -999,14 +983,21 @@ bool spd_inverse(std::vector<double>& A, int n) {
 void pair_matrix(const double* x, int nbp, const PairMobility& P, double h, double eta, std::vector<double>& M) {
   const int n3 = 3 * nbp;
   M.assign((size_t)n3 * n3, 0.0);
-  for (int i = 0; i < nbp; ++i)
-    for (int j = 0; j < nbp; ++j) {
-      const double d[3] = {(x[3 * i] - x[3 * j]) / h, (x[3 * i + 1] - x[3 * j + 1]) / h, (x[3 * i + 2] - x[3 * j + 2]) / h};
-      double B[9];
-      pair_block(P, d, i == j, B);
-      for (int p = 0; p < 3; ++p)
-        for (int q = 0; q < 3; ++q) M[(size_t)(3 * i + p) * n3 + 3 * j + q] = B[3 * p + q] / (eta * h);
-    }
+  for (int i = 0; i < nbp; ++i) {
+    int near = 0;
+    for (int pass = 0; pass < 2; ++pass)   // neighbours counted, then the blocks
+      for (int j = 0; j < nbp; ++j) {
+        const double d[3] = {(x[3 * i] - x[3 * j]) / h, (x[3 * i + 1] - x[3 * j + 1]) / h, (x[3 * i + 2] - x[3 * j + 2]) / h};
+        if (pass == 0) {
+          near += d[0] * d[0] + d[1] * d[1] + d[2] * d[2] < kPairNear * kPairNear;
+          continue;
+        }
+        double B[9];
+        pair_block(P, d, i == j ? pair_raise(P, near) : 0.0, B);
+        for (int p = 0; p < 3; ++p)
+          for (int q = 0; q < 3; ++q) M[(size_t)(3 * i + p) * n3 + 3 * j + q] = B[3 * p + q] / (eta * h);
+      }
+  }
 }
 
 bool inverse6(double A[36]) {
@@ -1059,6 +1050,7 @@ void build_body_block(rbfib_grid* g, const double* r, const double* arm, const d
       dense_body_gj(g->nbl, g->dM, g->dMw, g->dUw, g->dstatus, g->s);
     }
     dense_body_finish(g->nbl, g->nb, g->boff, arm, g->dM, g->dP, g->dN, g->dNw, g->dstatus, g->s);
+    dense_body_matrix(g->nbl, g->nb, g->dM, g->dP, g->dN, g->dE, g->dB, g->s);
     ck(cudaMemcpyAsync(g->dinfo.p + 13, g->dstatus.p, sizeof(int), cudaMemcpyDeviceToDevice, g->s));
     if (quat) ck(cudaMemcpyAsync(g->dquat.p, quat, sizeof(double) * 4 * g->nb, cudaMemcpyDeviceToDevice, g->s));
     return;
@@ -1068,6 +1060,7 @@ void build_body_block(rbfib_grid* g, const double* r, const double* arm, const d
   g->dM_valid = false;
   ck(dense_body_build(g->nbl, g->nb, g->boff, g->bob, r, arm, quat, qold, g->pair, g->desc.h, g->desc.eta, g->dM, g->dP,
                       g->dN, g->dstatus, g->dMw, g->dTw, g->dUw, g->dNw, g->dss, g->h_pinned + 40, warm, g->s, &used));
+  dense_body_matrix(g->nbl, g->nb, g->dM, g->dP, g->dN, g->dE, g->dB, g->s);
   int* hstat = (int*)(g->h_pinned + 42);
   ck(cudaMemcpyAsync(hstat, g->dstatus, sizeof(int), cudaMemcpyDeviceToHost, g->s));
   ck(cudaStreamSynchronize(g->s));
@@ -1484,6 +1477,8 @@ int rbfib_set_bodies(rbfib_grid* g, int32_t n_bodies, const int32_t* blob_offset
       g->dss.alloc(1);
       g->dquat.alloc(4 * (size_t)nb);
       g->dP.alloc((size_t)18 * nbl * nb);
+      g->dE.alloc((size_t)18 * nbl * nb);
+      g->dB.alloc((size_t)(3 * nbl + 6 * nb) * body_ld(3 * nbl + 6 * nb));
       g->dN.alloc((size_t)36 * nb * nb);
       g->dNw.alloc((size_t)72 * nb * nb);
       g->dstatus.alloc(1);
@@ -1519,72 +1514,65 @@ int rbfib_set_bodies(rbfib_grid* g, int32_t n_bodies, const int32_t* blob_offset
     }
     g->Lp.alloc(std::max(nb, 1));
     ck(cudaMemcpyAsync(g->Lp, Lp.data(), sizeof(double) * std::max(nb, 1), cudaMemcpyHostToDevice, g->s));
-    // per-shape inverse blob mobility and body mobility
+    // per-shape body-block matrices in the body frame (k_body.cu), used where
+    // the coupled block is not
     const int ns = (int)shape_rep.size();
-    std::vector<i64> moff(std::max(ns, 1), 0);
-    std::vector<double> minv_all, nmat(36 * (size_t)std::max(ns, 1), 0.0);
-    std::vector<int> srep(std::max(ns, 1), 0);
-    for (int s = 0; s < ns; ++s) {
+    std::vector<i64> soff(std::max(ns, 1), 0);
+    std::vector<float> sB;
+    for (int s = 0; s < ns && !g->dense_body; ++s) {
       const int p = shape_rep[s];
-      const int n = off[p + 1] - off[p];
+      const int n = off[p + 1] - off[p], n3 = 3 * n, ld = body_ld(n3 + 6);
       const double* x = href.data() + 3 * (size_t)off[p];
       std::vector<double> M;
       pair_matrix(x, n, g->pair, g->desc.h, g->desc.eta, M);
-      if (!spd_inverse(M, 3 * n)) return fail(g, RBFIB_EINVAL, "set_bodies: blob mobility of a shape is singular");
-      moff[s] = (i64)minv_all.size();
-      srep[s] = off[p];
-      // K^T M^-1 K in the body frame
-      double A[36] = {0};
-      std::vector<double> Kc(3 * (size_t)n * 6, 0.0);   // K (3n x 6)
+      if (!spd_inverse(M, n3)) return fail(g, RBFIB_EINVAL, "set_bodies: blob mobility of a shape is singular");
+      std::vector<double> K((size_t)n3 * 6, 0.0), P((size_t)n3 * 6, 0.0), E((size_t)n3 * 6, 0.0);
       for (int i = 0; i < n; ++i) {
         const double* r = x + 3 * i;
-        for (int a = 0; a < 3; ++a) Kc[(size_t)(3 * i + a) * 6 + a] = 1.0;
+        for (int a = 0; a < 3; ++a) K[(size_t)(3 * i + a) * 6 + a] = 1.0;
         // w x r = -[r]_x w
-        Kc[(size_t)(3 * i + 0) * 6 + 4] = r[2];  Kc[(size_t)(3 * i + 0) * 6 + 5] = -r[1];
-        Kc[(size_t)(3 * i + 1) * 6 + 3] = -r[2]; Kc[(size_t)(3 * i + 1) * 6 + 5] = r[0];
-        Kc[(size_t)(3 * i + 2) * 6 + 3] = r[1];  Kc[(size_t)(3 * i + 2) * 6 + 4] = -r[0];
+        K[(size_t)(3 * i + 0) * 6 + 4] = r[2];  K[(size_t)(3 * i + 0) * 6 + 5] = -r[1];
+        K[(size_t)(3 * i + 1) * 6 + 3] = -r[2]; K[(size_t)(3 * i + 1) * 6 + 5] = r[0];
+        K[(size_t)(3 * i + 2) * 6 + 3] = r[1];  K[(size_t)(3 * i + 2) * 6 + 4] = -r[0];
       }
-      const int n3 = 3 * n;
-      std::vector<double> MK((size_t)n3 * 6, 0.0);
+      double N[36] = {0};
       for (int r = 0; r < n3; ++r)
-        for (int c = 0; c < 6; ++c) {
-          double acc = 0.0;
-          for (int k = 0; k < n3; ++k) acc += M[(size_t)r * n3 + k] * Kc[(size_t)k * 6 + c];
-          MK[(size_t)r * 6 + c] = acc;
+        for (int k = 0; k < n3; ++k)
+          for (int c = 0; c < 6; ++c) P[(size_t)r * 6 + c] += M[(size_t)r * n3 + k] * K[(size_t)k * 6 + c];
+      for (int k = 0; k < n3; ++k)
+        for (int r = 0; r < 6; ++r)
+          for (int c = 0; c < 6; ++c) N[6 * r + c] += K[(size_t)k * 6 + r] * P[(size_t)k * 6 + c];
+      if (!inverse6(N)) return fail(g, RBFIB_EINVAL, "set_bodies: body resistance is singular");
+      for (int r = 0; r < n3; ++r)
+        for (int c = 0; c < 6; ++c)
+          for (int k = 0; k < 6; ++k) E[(size_t)r * 6 + c] += P[(size_t)r * 6 + k] * N[6 * k + c];
+      soff[s] = (i64)sB.size();
+      for (int r = 0; r < n3 + 6; ++r)
+        for (int c = 0; c < ld; ++c) {
+          double v = 0.0;
+          if (c < n3 + 6) {
+            if (r < n3 && c < n3) {
+              v = -M[(size_t)r * n3 + c];
+              for (int k = 0; k < 6; ++k) v += E[(size_t)r * 6 + k] * P[(size_t)c * 6 + k];
+            } else if (r < n3) v = E[(size_t)r * 6 + c - n3];
+            else if (c < n3) v = E[(size_t)c * 6 + r - n3];
+            else v = N[6 * (r - n3) + c - n3];
+          }
+          sB.push_back((float)v);
         }
-      for (int r = 0; r < 6; ++r)
-        for (int c = 0; c < 6; ++c) {
-          double acc = 0.0;
-          for (int k = 0; k < n3; ++k) acc += Kc[(size_t)k * 6 + r] * MK[(size_t)k * 6 + c];
-          A[6 * r + c] = acc;
-        }
-      if (!inverse6(A)) return fail(g, RBFIB_EINVAL, "set_bodies: body resistance is singular");
-      std::memcpy(nmat.data() + 36 * (size_t)s, A, sizeof(A));
-      minv_all.insert(minv_all.end(), M.begin(), M.end());
     }
     g->shape_of.alloc(std::max(nb, 1));
     ck(cudaMemcpyAsync(g->shape_of, shape_of.data(), sizeof(int) * std::max(nb, 1), cudaMemcpyHostToDevice, g->s));
-    g->shape_ref_blob.alloc(std::max(ns, 1));
-    ck(cudaMemcpyAsync(g->shape_ref_blob, srep.data(), sizeof(int) * std::max(ns, 1), cudaMemcpyHostToDevice, g->s));
-    g->minv_off.alloc(std::max(ns, 1));
-    ck(cudaMemcpyAsync(g->minv_off, moff.data(), sizeof(i64) * std::max(ns, 1), cudaMemcpyHostToDevice, g->s));
-    g->minv.alloc(std::max<size_t>(minv_all.size(), 1));
-    if (!minv_all.empty())
-      ck(cudaMemcpyAsync(g->minv, minv_all.data(), sizeof(double) * minv_all.size(), cudaMemcpyHostToDevice, g->s));
-    {
-      std::vector<float> m32(minv_all.begin(), minv_all.end());
-      g->minv32.alloc(std::max<size_t>(m32.size(), 1));
-      if (!m32.empty())
-        ck(cudaMemcpyAsync(g->minv32, m32.data(), sizeof(float) * m32.size(), cudaMemcpyHostToDevice, g->s));
-      ck(cudaStreamSynchronize(g->s));
-    }
-    g->nmat.alloc(nmat.size());
-    ck(cudaMemcpyAsync(g->nmat, nmat.data(), sizeof(double) * nmat.size(), cudaMemcpyHostToDevice, g->s));
+    g->shape_off.alloc(std::max(ns, 1));
+    ck(cudaMemcpyAsync(g->shape_off, soff.data(), sizeof(i64) * std::max(ns, 1), cudaMemcpyHostToDevice, g->s));
+    g->shape_B.alloc(std::max<size_t>(sB.size(), 1));
+    if (!sB.empty())
+      ck(cudaMemcpyAsync(g->shape_B, sB.data(), sizeof(float) * sB.size(), cudaMemcpyHostToDevice, g->s));
+    ck(cudaStreamSynchronize(g->s));
     // body-sized work arrays
     const size_t b6 = 6 * (size_t)std::max(nb, 1), l3 = 3 * (size_t)std::max(nbl, 1);
     for (DBuf<double>* b : {&g->bodyA, &g->bodyB, &g->bodyF, &g->bodyW, &g->bodyWn}) b->alloc(b6);
-    for (DBuf<double>* b : {&g->blobA, &g->blobB, &g->blobC, &g->blobD, &g->blobS, &g->sres}) b->alloc(l3);
-    g->sres32.alloc(l3);
+    for (DBuf<double>* b : {&g->blobA, &g->blobB, &g->blobC, &g->blobD, &g->blobS}) b->alloc(l3);
     alloc_solver(g);
     ck(cudaStreamSynchronize(g->s));
     ck(cudaGetLastError());
