@@ -83,14 +83,8 @@ template <typename T> void add_grad(const Dims&, T eta, T kappa, const T* phi, c
 // orthonormal 1D eigenbases Q_x, Q_y, Q_z and eigenvalues l_x, l_y, l_z,
 // A^-1 = (Q_x (x) Q_y (x) Q_z) diag(1 / (s (l_x + l_y + l_z))) (Q_x (x) Q_y (x) Q_z)^T,
 // the zero mode of a singular operator dropped (pseudo-inverse).
-constexpr int kFDLine = 48;                 // points along one axis (short-line forms)
+constexpr int kFDLine = 48;                 // points along one axis (short-line form)
 constexpr int kFDLongest = 1024;            // points along one axis (long-line form)
-constexpr int kFDCtas = 8;           // CTAs (one cluster) per grid
-constexpr int kFDThreads = 256;
-// shared memory bound per CTA: table (3 axes, two padded e x e bases and e
-// eigenvalues each) and two slab buffers of ceil(e_z / kFDCtas) planes
-constexpr int kFDMaxSmem = (int)sizeof(float) * (3 * (2 * kFDLine * kFDLine + kFDLine) + 4 +
-                                                 2 * (((kFDLine + kFDCtas - 1) / kFDCtas) * kFDLine * kFDLine + 4));
 // One axis of the long-line form (k_fdl_*): its basis folded by the mirror
 // symmetry of its eigenvectors.  Pair p joins the points jA(p), jB(p) (see
 // fold_pair); hs symmetric and ha antisymmetric eigenvectors, stored in that
@@ -115,12 +109,10 @@ struct FDParams {
   int lines;       // 1: the long-line form (an axis longer than kFDLine)
   FDGrid g[3];
   const float* tab;
-  int smem;        // dynamic shared memory bytes of the largest grid
 };
 // Bases of every grid of a level; false if some grid exceeds the limits.
 bool fd_plan(const Dims& d, bool faces, double eta, std::vector<float>& tab, FDParams& P, std::string& why);
-// u = A^-1 rhs on the planned level; tmp holds as many floats as u.  The
-// form (one cluster per grid, whole GPU, long lines) is chosen by size.
+// u = A^-1 rhs on the planned level; tmp holds as many floats as u.
 void fd_solve(const FDParams& P, float* u, const float* rhs, float* tmp, cudaStream_t s);
 
 // k_ib.cu

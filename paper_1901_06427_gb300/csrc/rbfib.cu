@@ -323,8 +323,6 @@ SmallPtrs small_ptrs(rbfib_grid* g, int m) {
 template <typename T>
 MGStore<T>& mg_of(rbfib_grid* g);
 template <>
-MGStore<double>& mg_of<double>(rbfib_grid* g) { return g->mg64; }
-template <>
 MGStore<float>& mg_of<float>(rbfib_grid* g) { return g->mg32; }
 template <typename T>
 KrylovStore<T>& kr_of(rbfib_grid* g);
