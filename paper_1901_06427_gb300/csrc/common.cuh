@@ -221,6 +221,8 @@ struct AxisStencil {
 
 // Points p = p0 + t (t < kw) of a coordinate s in grid units: three points
 // from p0 = floor(s + 1/2) - 1, six from p0 = floor(s) - 2.
+// DERIV = false leaves the derivatives dw unset.
+template <bool DERIV = true>
 __device__ inline void axis_stencil(const Dims& d, int a, int ax, double x, AxisStencil& S) {
   const double o = (ax == a) ? 0.0 : 0.5;
   const double s = x / d.h[ax] - o;
@@ -234,10 +236,10 @@ __device__ inline void axis_stencil(const Dims& d, int a, int ax, double x, Axis
     const int p = i0 + t;
     if (kw == 6) {
       S.w[t] = w6[t];
-      S.dw[t] = dw6[t] / d.h[ax];
+      if (DERIV) S.dw[t] = dw6[t] / d.h[ax];
     } else {
       S.w[t] = phi3(s - (double)p);
-      S.dw[t] = dphi3(s - (double)p) / d.h[ax];
+      if (DERIV) S.dw[t] = dphi3(s - (double)p) / d.h[ax];
     }
     S.sgn[t] = 1;
     S.wall[t] = -1;

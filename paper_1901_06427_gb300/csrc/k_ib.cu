@@ -1,6 +1,8 @@
 // Immersed-boundary and rigid-body kernels (Sec. III.B): body geometry,
 // blob-to-cell binning, spreading S, interpolation J, the rigid maps K and
 // K^T, the fused body rows of the saddle operator and the forces of Sec. V.
+#include <algorithm>
+
 #include "common.cuh"
 #include "kernels.cuh"
 
@@ -125,92 +127,181 @@ void binning(const Dims& d, int nbl, const double* r, int* perm, int* off, int* 
 }
 
 // ----------------------------------------------------- spread / interpolate
-// Folded kw^3-point stencil of one blob and component.  For each point: flat
-// face index (within component a), folded weight, and affine ghost weight
-// (sum over folded tangential axes, in x,y,z order, of sign * 2 u_w).
-struct Stencil27 {
-  AxisStencil ax[3];
-};
+// at blob positions without a stencil table (displaced configurations, wall
+// parts).  A block takes pos_per_block(3 N_bl) blob components: one thread
+// per component and axis forms the folded stencils in shared memory (FP64
+// square roots, a warp instruction each whether 3 or 32 lanes are active, so
+// large suspensions fill the lanes), then one warp per component shares its
+// kw^3 points (one thread per component took 35 us with the three-point and
+// 80 us with the six-point kernel, a chain of 216 FP64 terms).
+constexpr int kPosThreads = 128, kPosMax = 40;
+struct PosStencil { AxisStencil ax[3]; };
+inline int pos_per_block(i64 n) { return (int)std::min<i64>(kPosMax, std::max<i64>(kPosThreads / 32, n / (152 * 4))); }
 
-RBFIB_DEVFN void load_stencil(const Dims& d, int a, const double* x, Stencil27& S) {
-  axis_stencil(d, a, 0, x[0], S.ax[0]);
-  axis_stencil(d, a, 1, x[1], S.ax[1]);
-  axis_stencil(d, a, 2, x[2], S.ax[2]);
+// Stencils of components [c0, c0 + per) below n at positions r; every thread
+// of the block calls it.
+RBFIB_DEVFN void pos_stencils(const Dims& d, int c0, int per, int n, const double* __restrict__ r, PosStencil* S) {
+  __syncthreads();
+  for (int t = threadIdx.x; t < 3 * per && c0 + t / 3 < n; t += kPosThreads) {
+    const int c = c0 + t / 3, ax = t % 3;
+    axis_stencil<false>(d, c % 3, ax, r[3 * (c / 3) + ax], S[t / 3].ax[ax]);
+  }
+  __syncthreads();
 }
 
-template <typename T>
-__global__ void k_spread(Dims d, int nbl, const int* __restrict__ perm, const double* __restrict__ r,
-                         const T* __restrict__ lam, double scale, T* __restrict__ f) {
+RBFIB_DEVFN double warp_add(double v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// (J v) of component a, in every lane
+RBFIB_DEVFN double pos_interp(const Dims& d, int a, const PosStencil& S, const double* __restrict__ v, int lane) {
+  const double* va = v + d.fo[a];
+  const int kw = d.kw, np = kw * kw * kw;
+  double jv = 0.0;
+  for (int p = lane; p < np; p += 32) {
+    const int x = p % kw, y = (p / kw) % kw, z = p / (kw * kw);
+    const AxisStencil &X = S.ax[0], &Y = S.ax[1], &Z = S.ax[2];
+    if (X.keep[x] && Y.keep[y] && Z.keep[z])
+      jv += X.w[x] * Y.w[y] * Z.w[z] * (double)(X.sgn[x] * Y.sgn[y] * Z.sgn[z]) *
+            va[flat3(d.fe[a], X.idx[x], Y.idx[y], Z.idx[z])];
+  }
+  return warp_add(jv);
+}
+
+// What moving walls add to J v: per point the tangential ghosts' 2 u_w, the
+// folds acting in x, y, z order.
+RBFIB_DEVFN double pos_wall(const Dims& d, const Walls& wl, int a, const PosStencil& S, int lane) {
+  const int kw = d.kw, np = kw * kw * kw;
+  double aff = 0.0;
+  for (int p = lane; p < np; p += 32) {
+    const int pt[3] = {p % kw, (p / kw) % kw, p / (kw * kw)};
+    double w = 1.0, sg = 1.0, af = 0.0;
+    bool keep = true;
+#pragma unroll
+    for (int ax = 0; ax < 3; ++ax) {
+      const AxisStencil& A = S.ax[ax];
+      keep = keep && A.keep[pt[ax]];
+      w *= A.w[pt[ax]];
+      if (A.sgn[pt[ax]] < 0) {
+        if (A.wall[pt[ax]] >= 0) af += sg * 2.0 * wl.v[A.wall[pt[ax]]][a];
+        sg = -sg;
+      }
+    }
+    if (keep) aff += w * af;
+  }
+  return warp_add(aff);
+}
+
+// f += scale (S(r+) - S(r-)) lam (no 1/dV)
+__global__ void __launch_bounds__(kPosThreads) k_spread_diff(Dims d, int nbl, int per, const double* __restrict__ rp,
+                                                             const double* __restrict__ rm,
+                                                             const double* __restrict__ lam, double scale,
+                                                             double* __restrict__ f) {
   pdl_entry();
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= 3 * nbl) return;
-  const int s = t / 3, a = t - 3 * s;
-  const int i = perm ? perm[s] : s;
-  const double val = (double)lam[3 * i + a] * scale;
-  if (val == 0.0) return;
-  Stencil27 S;
-  load_stencil(d, a, r + 3 * i, S);
-  T* fa = f + d.fo[a];
-  const int kw = d.kw;
-  for (int z = 0; z < kw; ++z) {
-    if (!S.ax[2].keep[z]) continue;
-    const double wz = S.ax[2].w[z] * S.ax[2].sgn[z];
-    for (int y = 0; y < kw; ++y) {
-      if (!S.ax[1].keep[y]) continue;
-      const double wyz = wz * S.ax[1].w[y] * S.ax[1].sgn[y];
-      for (int x = 0; x < kw; ++x) {
-        if (!S.ax[0].keep[x]) continue;
-        const double w = wyz * S.ax[0].w[x] * S.ax[0].sgn[x];
-        atomicAdd(fa + flat3(d.fe[a], S.ax[0].idx[x], S.ax[1].idx[y], S.ax[2].idx[z]), (T)(w * val));
+  __shared__ PosStencil Sh[kPosMax];
+  const int lane = threadIdx.x & 31, n = 3 * nbl, c0 = blockIdx.x * per;
+  const int kw = d.kw, np = kw * kw * kw;
+  for (int s = 0; s < 2; ++s) {
+    pos_stencils(d, c0, per, n, s ? rm : rp, Sh);
+    for (int q = threadIdx.x >> 5; q < per && c0 + q < n; q += kPosThreads / 32) {
+      const int c = c0 + q, a = c % 3;
+      const double val = (s ? -lam[c] : lam[c]) * scale;
+      if (val == 0.0) continue;
+      double* fa = f + d.fo[a];
+      const AxisStencil &X = Sh[q].ax[0], &Y = Sh[q].ax[1], &Z = Sh[q].ax[2];
+      for (int p = lane; p < np; p += 32) {
+        const int x = p % kw, y = (p / kw) % kw, z = p / (kw * kw);
+        if (X.keep[x] && Y.keep[y] && Z.keep[z])
+          atomicAdd(fa + flat3(d.fe[a], X.idx[x], Y.idx[y], Z.idx[z]),
+                    X.w[x] * Y.w[y] * Z.w[z] * (double)(X.sgn[x] * Y.sgn[y] * Z.sgn[z]) * val);
       }
     }
   }
 }
 
-// out[3i+a] = beta * out + alpha * (J v)_ia + gamma * (wall ghost part)_ia
-template <typename T>
-RBFIB_DEVFN void interp_one(const Dims& d, const Walls& wl, int a, const double* x, const T* __restrict__ v,
-                            double& jv, double& aff) {
-  Stencil27 S;
-  load_stencil(d, a, x, S);
-  const T* va = v + d.fo[a];
-  jv = 0.0; aff = 0.0;
-  const int kw = d.kw;
-  for (int z = 0; z < kw; ++z) {
-    if (!S.ax[2].keep[z]) continue;
-    for (int y = 0; y < kw; ++y) {
-      if (!S.ax[1].keep[y]) continue;
-      for (int xx = 0; xx < kw; ++xx) {
-        if (!S.ax[0].keep[xx]) continue;
-        const int pt[3] = {xx, y, z};
-        double w = 1.0, sg = 1.0, af = 0.0;
-        for (int ax = 0; ax < 3; ++ax) {
-          const AxisStencil& A = S.ax[ax];
-          w *= A.w[pt[ax]];
-          if (A.sgn[pt[ax]] < 0) {
-            if (A.wall[pt[ax]] >= 0) af += sg * 2.0 * wl.v[A.wall[pt[ax]]][a];
-            sg = -sg;
-          }
-        }
-        if (v) jv += w * sg * (double)va[flat3(d.fe[a], S.ax[0].idx[xx], S.ax[1].idx[y], S.ax[2].idx[z])];
-        aff += w * af;
+void spread_diff(const Dims& d, int nbl, const double* rp, const double* rm, const double* lam, double scale, double* f,
+                 cudaStream_t s) {
+  if (nbl > 0) {
+    const int per = pos_per_block(3 * (i64)nbl);
+    launch_k(k_spread_diff, nblk(3 * (i64)nbl, per), kPosThreads, 0, s, d, nbl, per, rp, rm, lam, scale, f);
+    note_launch();
+  }
+}
+
+// out = beta out + (moving walls' part of J)
+__global__ void __launch_bounds__(kPosThreads) k_interp_walls(Dims d, Walls wl, int nbl, int per,
+                                                              const double* __restrict__ r, double beta,
+                                                              double* __restrict__ out) {
+  pdl_entry();
+  __shared__ PosStencil Sh[kPosMax];
+  const int lane = threadIdx.x & 31, n = 3 * nbl, c0 = blockIdx.x * per;
+  pos_stencils(d, c0, per, n, r, Sh);
+  for (int q = threadIdx.x >> 5; q < per && c0 + q < n; q += kPosThreads / 32) {
+    const int c = c0 + q;
+    const double aff = pos_wall(d, wl, c % 3, Sh[q], lane);
+    if (lane == 0) out[c] = beta != 0.0 ? beta * out[c] + aff : aff;
+  }
+}
+
+void interp_walls(const Dims& d, const Walls& wl, int nbl, const double* r, double beta, double* out, cudaStream_t s) {
+  if (nbl > 0) {
+    const int per = pos_per_block(3 * (i64)nbl);
+    launch_k(k_interp_walls, nblk(3 * (i64)nbl, per), kPosThreads, 0, s, d, wl, nbl, per, r, beta, out);
+    note_launch();
+  }
+}
+
+RBFIB_DEVFN double rigid_velocity(const double* U, const double* ar, int a) {
+  const double w0 = U[3], w1 = U[4], w2 = U[5];
+  const double cr = a == 0 ? w1 * ar[2] - w2 * ar[1] : (a == 1 ? w2 * ar[0] - w0 * ar[2] : w0 * ar[1] - w1 * ar[0]);
+  return U[a] + cr;
+}
+
+// The random finite differences of the slip (Algorithm 1 step 5) in one
+// launch: out = slip + D^K - D^J - D^S with D^K = (K+ - K-) U / delta,
+// D^J = (J+ - J-) v / delta, D^S = J v# (the current configuration's table).
+__global__ void __launch_bounds__(kPosThreads) k_rfd_slip(Dims d, BodyView b, int per, const double* __restrict__ rp,
+                                                          const double* __restrict__ rm,
+                                                          const double* __restrict__ armp,
+                                                          const double* __restrict__ armm,
+                                                          const double* __restrict__ v, const double* __restrict__ U,
+                                                          const double* __restrict__ vsharp,
+                                                          const double* __restrict__ slip, double idelta,
+                                                          double* __restrict__ out) {
+  pdl_entry();
+  __shared__ PosStencil Sh[kPosMax];
+  __shared__ double jp[kPosMax];
+  const int lane = threadIdx.x & 31, n = 3 * b.nbl, c0 = blockIdx.x * per;
+  for (int s = 0; s < 2; ++s) {
+    pos_stencils(d, c0, per, n, s ? rm : rp, Sh);
+    for (int q = threadIdx.x >> 5; q < per && c0 + q < n; q += kPosThreads / 32) {
+      const int c = c0 + q, i = c / 3, a = c - 3 * i;
+      const double jv = pos_interp(d, a, Sh[q], v, lane);
+      if (s == 0) {
+        if (lane == 0) jp[q] = jv;   // read back by the same lane
+        continue;
+      }
+      const double js = warp_interp<double>(d, a, b.st64 + c, vsharp, lane);
+      if (lane == 0) {
+        const double* Up = U + 6 * b.bob[i];
+        const double dk = (rigid_velocity(Up, armp + 3 * i, a) - rigid_velocity(Up, armm + 3 * i, a)) * idelta;
+        out[c] = (slip ? slip[c] : 0.0) + dk - (jp[q] - jv) * idelta - js;
       }
     }
   }
 }
 
-template <typename T>
-__global__ void k_interp(Dims d, Walls wl, int nbl, const double* __restrict__ r, const T* __restrict__ v,
-                         double alpha, double beta, double gamma, T* __restrict__ out) {
-  pdl_entry();
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= 3 * nbl) return;
-  const int i = t / 3, a = t - 3 * i;
-  double jv, aff;
-  interp_one(d, wl, a, r + 3 * i, (alpha != 0.0) ? v : (const T*)nullptr, jv, aff);
-  double o = alpha * jv + gamma * aff;
-  if (beta != 0.0) o += beta * (double)out[t];
-  out[t] = (T)o;
+void rfd_slip(const Dims& d, const BodyView& b, const double* rp, const double* rm, const double* armp,
+              const double* armm, const double* v, const double* U, const double* vsharp, const double* slip,
+              double idelta, double* out, cudaStream_t s) {
+  if (b.nbl > 0) {
+    const int per = pos_per_block(3 * (i64)b.nbl);
+    launch_k(k_rfd_slip, nblk(3 * (i64)b.nbl, per), kPosThreads, 0, s, d, b, per, rp, rm, armp, armm, v, U, vsharp, slip,
+             idelta, out);
+    note_launch();
+  }
 }
 
 // -------------------------------------------- per-configuration stencil table
@@ -364,83 +455,44 @@ void saddle_bodies(const Dims& d, const BodyView& b, const T* v, const T* lam, c
   note_launch();
 }
 
-template <typename T>
-void spread(const Dims& d, int nbl, const int* perm, const double* r, const T* lam, double scale, T* f,
-            cudaStream_t s) {
-  if (nbl > 0) {
-    launch_k(k_spread<T>, nblk(3 * (i64)nbl, 128), 128, 0, s,
-             d, nbl, perm, r, lam, scale, f);
-    note_launch();
-  }
-}
-
-template <typename T>
-void interp(const Dims& d, const Walls& wl, int nbl, const double* r, const T* v, double alpha,
-            double beta, double gamma, T* out, cudaStream_t s) {
-  if (nbl > 0) {
-    launch_k(k_interp<T>, nblk(3 * (i64)nbl, 128), 128, 0, s,
-             d, wl, nbl, r, v, alpha, beta, gamma, out);
-    note_launch();
-  }
-}
-
-// K^T lam per body (FP64): out = alpha * K^T lam + beta * out
-template <typename T>
-__global__ void k_kt(int nb, const int* __restrict__ boff, const double* __restrict__ arm,
-                     const T* __restrict__ lam, double alpha, double beta, double* __restrict__ out) {
-  pdl_entry();
-  const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (warp >= nb) return;
-  double acc[6] = {0, 0, 0, 0, 0, 0};
-  for (int i = boff[warp] + lane; i < boff[warp + 1]; i += 32) {
-    const double lx = (double)lam[3 * i], ly = (double)lam[3 * i + 1], lz = (double)lam[3 * i + 2];
+// K^T lam of one body by a warp (FP64 sums), in every lane.
+RBFIB_DEVFN void warp_kt(int b0, int b1, const double* __restrict__ arm, const double* __restrict__ lam, int lane,
+                         double acc[6]) {
+#pragma unroll
+  for (int c = 0; c < 6; ++c) acc[c] = 0.0;
+  for (int i = b0 + lane; i < b1; i += 32) {
+    const double lx = lam[3 * i], ly = lam[3 * i + 1], lz = lam[3 * i + 2];
     const double* ar = arm + 3 * i;
     acc[0] += lx; acc[1] += ly; acc[2] += lz;
     acc[3] += ar[1] * lz - ar[2] * ly;
     acc[4] += ar[2] * lx - ar[0] * lz;
     acc[5] += ar[0] * ly - ar[1] * lx;
   }
-  for (int c = 0; c < 6; ++c)
-    for (int o = 16; o > 0; o >>= 1) acc[c] += __shfl_xor_sync(0xffffffffu, acc[c], o);
-  if (lane < 6) {
-    double o = alpha * acc[lane];
-    if (beta != 0.0) o += beta * out[6 * warp + lane];
-    out[6 * warp + lane] = o;
-  }
+#pragma unroll
+  for (int c = 0; c < 6; ++c) acc[c] = warp_add(acc[c]);
 }
 
-void kt_apply(int nb, const int* boff, const double* arm, const double* lam, double alpha, double beta,
-              double* out, cudaStream_t s) {
+// F -= D^{K^T} = (K+^T - K-^T) lam / delta (Algorithm 1 step 5), a warp per body
+__global__ void k_rfd_force(int nb, const int* __restrict__ boff, const double* __restrict__ armp,
+                            const double* __restrict__ armm, const double* __restrict__ lam, double idelta,
+                            double* __restrict__ F) {
+  pdl_entry();
+  const int p = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+  if (p >= nb) return;
+  double kp[6], km[6];
+  warp_kt(boff[p], boff[p + 1], armp, lam, lane, kp);
+  warp_kt(boff[p], boff[p + 1], armm, lam, lane, km);
+#pragma unroll
+  for (int c = 0; c < 6; ++c)
+    if (lane == c) F[6 * p + c] -= (kp[c] - km[c]) * idelta;
+}
+
+void rfd_force(int nb, const int* boff, const double* armp, const double* armm, const double* lam, double idelta,
+               double* F, cudaStream_t s) {
   if (nb > 0) {
-    launch_k(k_kt<double>, nblk(32 * (i64)nb, 128), 128, 0, s,
-             nb, boff, arm, lam, alpha, beta, out);
+    launch_k(k_rfd_force, nblk(32 * (i64)nb, 128), 128, 0, s, nb, boff, armp, armm, lam, idelta, F);
     note_launch();
   }
-}
-
-// K U per blob: out = alpha * (u + w x arm) + beta * out
-__global__ void k_k(int nbl, const int* __restrict__ bob, const double* __restrict__ arm,
-                    const double* __restrict__ U, double alpha, double beta, double* __restrict__ out) {
-  pdl_entry();
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= 3 * nbl) return;
-  const int i = t / 3, a = t - 3 * i;
-  const int p = bob[i];
-  const double* ar = arm + 3 * i;
-  const double w0 = U[6 * p + 3], w1 = U[6 * p + 4], w2 = U[6 * p + 5];
-  double cr;
-  if (a == 0) cr = w1 * ar[2] - w2 * ar[1];
-  else if (a == 1) cr = w2 * ar[0] - w0 * ar[2];
-  else cr = w0 * ar[1] - w1 * ar[0];
-  double o = alpha * (U[6 * p + a] + cr);
-  if (beta != 0.0) o += beta * out[t];
-  out[t] = o;
-}
-
-void k_apply(int nbl, const int* bob, const double* arm, const double* U, double alpha, double beta,
-             double* out, cudaStream_t s) {
-  if (nbl > 0) { launch_k(k_k, nblk(3 * (i64)nbl, 128), 128, 0, s, nbl, bob, arm, U, alpha, beta, out); note_launch(); }
 }
 
 // ------------------------------------------------------------------ forces
@@ -615,10 +667,7 @@ void outside_check(const Dims& d, int nbl, const double* r, int* flag, cudaStrea
 
 #define INST(T)                                                                                          \
   template void saddle_bodies<T>(const Dims&, const BodyView&, const T*, const T*, const T*, T*, T*, T*, \
-                                 cudaStream_t);                                                          \
-  template void spread<T>(const Dims&, int, const int*, const double*, const T*, double, T*, cudaStream_t); \
-  template void interp<T>(const Dims&, const Walls&, int, const double*, const T*, double, double, double, \
-                          T*, cudaStream_t);
+                                 cudaStream_t);
 INST(double)
 INST(float)
 #undef INST

@@ -122,18 +122,18 @@ void binning(const Dims&, int nbl, const double* r, int* perm, int* off, int* ke
              int* bsum, cudaStream_t);
 template <typename T> void saddle_bodies(const Dims&, const BodyView&, const T* v, const T* lam, const T* U,
                                          T* yv, T* ylam, T* yU, cudaStream_t);
-template <typename T> void spread(const Dims&, int nbl, const int* perm, const double* r, const T* lam,
-                                  double scale, T* f, cudaStream_t);
-template <typename T> void interp(const Dims&, const Walls&, int nbl, const double* r, const T* v, double alpha,
-                                  double beta, double gamma, T* out, cudaStream_t);
+void spread_diff(const Dims&, int nbl, const double* rp, const double* rm, const double* lam, double scale, double* f,
+                 cudaStream_t);
+void interp_walls(const Dims&, const Walls&, int nbl, const double* r, double beta, double* out, cudaStream_t);
+void rfd_slip(const Dims&, const BodyView&, const double* rp, const double* rm, const double* armp, const double* armm,
+              const double* v, const double* U, const double* vsharp, const double* slip, double idelta, double* out,
+              cudaStream_t);
+void rfd_force(int nb, const int* boff, const double* armp, const double* armm, const double* lam, double idelta,
+               double* F, cudaStream_t);
 void stencil_build(const Dims&, int nbl, const double* r, BlobStencil<double>* s64, BlobStencil<float>* s32,
                    cudaStream_t);
 void interp_tab(const Dims&, const BodyView&, const double* v, double alpha, double beta, double* out, cudaStream_t);
 void spread_tab(const Dims&, const BodyView&, const double* lam, double scale, double* f, cudaStream_t);
-void kt_apply(int nb, const int* boff, const double* arm, const double* lam, double alpha, double beta,
-              double* out, cudaStream_t);
-void k_apply(int nbl, const int* bob, const double* arm, const double* U, double alpha, double beta,
-             double* out, cudaStream_t);
 void body_forces(const Dims&, const Potentials&, const BodyView&, const double* fext, double* out, cudaStream_t);
 void wft(int nb, const double* wn, const double* Lp, double kT, double* out, cudaStream_t);
 void move_bodies(int nb, const double* q, const double* quat, const double* vec6, const double* Lp, double a,

@@ -139,6 +139,7 @@ struct rbfib_grid {
   DBuf<float> fd_tab, fd_tmp;
   Dims d{};
   Walls walls{};
+  bool walls_move = false;   // some wall velocity is not zero
   i64 nf = 0, nc = 0, nfl = 0;
   double dV = 1.0;
   double kappa = 0.0;   // pressure_kappa
@@ -168,8 +169,8 @@ struct rbfib_grid {
   bool dM_valid = false, dquat_valid = false;
   long long ns_warm = 0;
   // work vectors (FP64)
-  DBuf<double> part, scal, bvec, xvec, xrfd, rres, fsharp, vsharp, fnoise, Wst;
-  DBuf<double> bodyA, bodyB, bodyF, bodyW, bodyWn, blobA, blobB, blobC, blobD, blobS;
+  DBuf<double> part, scal, bvec, xvec, xrfd, rres, fnoise, Wst;
+  DBuf<double> bodyF, bodyW, bodyWn, blobS;
   double* h_pinned = nullptr;
   int nparts = 0;
   // precision-specific stores
@@ -1106,8 +1107,6 @@ void alloc_solver(rbfib_grid* g) {
   g->f32a.ensure(n);
   g->f32b.ensure(n);
   g->bvec.ensure(n); g->xvec.ensure(n); g->xrfd.ensure(n);
-  // the FP32 refinement keeps an FP64 residual and correction
-  g->blobA.ensure(std::max<i64>(3 * (i64)g->nbl, 1));
 }
 
 // ---------------------------------------------------------------- autotuner
@@ -1334,7 +1333,10 @@ int rbfib_create_grid(const rbfib_grid_desc* desc, void* stream, rbfib_grid** ou
     g->levels[0].d.kw = D.kernel;
     g->d = g->levels[0].d;
     for (int w = 0; w < 6; ++w)
-      for (int c = 0; c < 3; ++c) g->walls.v[w][c] = D.wall_vel[w][c];
+      for (int c = 0; c < 3; ++c) {
+        g->walls.v[w][c] = D.wall_vel[w][c];
+        if (D.wall_vel[w][c] != 0.0) g->walls_move = true;
+      }
     g->nf = g->d.fo[3];
     g->nc = g->d.nc;
     g->nfl = g->nf + g->nc;
@@ -1366,7 +1368,7 @@ int rbfib_create_grid(const rbfib_grid_desc* desc, void* stream, rbfib_grid** ou
     g->boff.alloc(1);
     ck(cudaMemsetAsync(g->boff, 0, sizeof(int), g->s));
     g->h_boff.assign(1, 0);
-    g->fsharp.alloc(g->nf); g->vsharp.alloc(g->nf); g->fnoise.alloc(g->nf);
+    g->fnoise.alloc(g->nf);
     g->Wst.alloc(g->stress.total);
     alloc_solver(g);
     autotune(g);
@@ -1569,8 +1571,8 @@ int rbfib_set_bodies(rbfib_grid* g, int32_t n_bodies, const int32_t* blob_offset
     ck(cudaStreamSynchronize(g->s));
     // body-sized work arrays
     const size_t b6 = 6 * (size_t)std::max(nb, 1), l3 = 3 * (size_t)std::max(nbl, 1);
-    for (DBuf<double>* b : {&g->bodyA, &g->bodyB, &g->bodyF, &g->bodyW, &g->bodyWn}) b->alloc(b6);
-    for (DBuf<double>* b : {&g->blobA, &g->blobB, &g->blobC, &g->blobD, &g->blobS}) b->alloc(l3);
+    for (DBuf<double>* b : {&g->bodyF, &g->bodyW, &g->bodyWn}) b->alloc(b6);
+    g->blobS.alloc(l3);
     alloc_solver(g);
     ck(cudaStreamSynchronize(g->s));
     ck(cudaGetLastError());
@@ -1619,10 +1621,10 @@ void build_rhs(rbfib_grid* g, const double* FT, const double* slip, const double
   const i64 n = g->n_total();
   ck(cudaMemsetAsync(b, 0, sizeof(double) * n, g->s));
   if (fluid) ck(cudaMemcpyAsync(b, fluid, sizeof(double) * g->nf, cudaMemcpyDeviceToDevice, g->s));
-  if (walls) wall_rhs<double>(g->d, g->walls, g->desc.eta, b, g->s);
+  if (walls && g->walls_move) wall_rhs<double>(g->d, g->walls, g->desc.eta, b, g->s);
   if (g->nbl > 0) {
     double* bl = b + g->nfl;
-    if (walls) interp<double>(g->d, g->walls, g->nbl, g->cur.r, (const double*)nullptr, 0.0, 0.0, 1.0, bl, g->s);
+    if (walls && g->walls_move) interp_walls(g->d, g->walls, g->nbl, g->cur.r, 0.0, bl, g->s);
     if (slip) axpby<double>(bl, slip, -1.0, 1.0, 3 * (i64)g->nbl, g->s);
   }
   if (g->nb > 0 && FT)
@@ -1882,8 +1884,7 @@ int rbfib_interpolate(rbfib_grid* g, const double* v, double* u, int32_t with_wa
   if (!g || !v || (g->nbl && !u)) return fail(g, RBFIB_EINVAL, "interpolate: null argument");
   try {
     interp_tab(g->d, view_of(g, g->cur), v, 1.0, 0.0, u, g->s);
-    if (with_walls)
-      interp<double>(g->d, g->walls, g->nbl, g->cur.r, (const double*)nullptr, 0.0, 1.0, 1.0, u, g->s);
+    if (with_walls && g->walls_move) interp_walls(g->d, g->walls, g->nbl, g->cur.r, 1.0, u, g->s);
     ck(cudaGetLastError());
   } catch (CudaError& e) {
     return fail(g, e.code, e.what());
@@ -2018,36 +2019,15 @@ int sem_step_body(rbfib_grid* g, const rbfib_sem_params* p, uint64_t seed, uint6
     refresh_config(g, g->plus, false);
     refresh_config(g, g->minus, false);
     // step 4: unconstrained Stokes solve with (S(Q+) - S(Q-)) lambda / delta
-    ck(cudaMemsetAsync(g->fsharp, 0, sizeof(double) * g->nf, s));
-    spread<double>(g->d, nbl, nullptr, g->plus.r, lam_rfd, 1.0 / (delta * g->dV), g->fsharp, s);
-    spread<double>(g->d, nbl, nullptr, g->minus.r, lam_rfd, -1.0 / (delta * g->dV), g->fsharp, s);
     ck(cudaMemsetAsync(g->bvec, 0, sizeof(double) * g->nfl, s));
-    ck(cudaMemcpyAsync(g->bvec, g->fsharp, sizeof(double) * g->nf, cudaMemcpyDeviceToDevice, s));
+    spread_diff(g->d, nbl, g->plus.r, g->minus.r, lam_rfd, 1.0 / (delta * g->dV), g->bvec, s);
     int st2 = solve_system(g, g->bvec, g->xvec, false, &loc.solve_stokes, 1);
     if (st2 && !st) st = st2;
-    ck(cudaMemcpyAsync(g->vsharp, g->xvec, sizeof(double) * g->nf, cudaMemcpyDeviceToDevice, s));
-    // step 5: random finite differences
-    Walls w0 = {};
-    kt_apply(nb, g->boff, g->plus.arm, lam_rfd, 1.0, 0.0, g->bodyA, s);
-    kt_apply(nb, g->boff, g->minus.arm, lam_rfd, 1.0, 0.0, g->bodyB, s);
-    axpby<double>(g->bodyA, g->bodyB, -1.0, 1.0, 6 * (i64)nb, s);          // A = KT+ - KT-
-    axpby<double>(g->bodyA, g->bodyA, 0.0, 1.0 / delta, 6 * (i64)nb, s);   // D^{K^T}
-    k_apply(nbl, g->bob, g->plus.arm, U_rfd, 1.0, 0.0, g->blobA, s);
-    k_apply(nbl, g->bob, g->minus.arm, U_rfd, 1.0, 0.0, g->blobB, s);
-    axpby<double>(g->blobA, g->blobB, -1.0, 1.0, 3 * (i64)nbl, s);
-    axpby<double>(g->blobA, g->blobA, 0.0, 1.0 / delta, 3 * (i64)nbl, s);  // D^K
-    interp<double>(g->d, w0, nbl, g->plus.r, v_rfd, 1.0, 0.0, 0.0, g->blobC, s);
-    interp<double>(g->d, w0, nbl, g->minus.r, v_rfd, 1.0, 0.0, 0.0, g->blobD, s);
-    axpby<double>(g->blobC, g->blobD, -1.0, 1.0, 3 * (i64)nbl, s);
-    axpby<double>(g->blobC, g->blobC, 0.0, 1.0 / delta, 3 * (i64)nbl, s);  // D^J
-    interp_tab(g->d, view_of(g, g->cur), g->vsharp, 1.0, 0.0, g->blobD, s);                          // D^S
-    // slip_tot = slip + D^K - D^J - D^S ; F_tot = F - D^{K^T}
-    if (p->slip) ck(cudaMemcpyAsync(g->blobS, p->slip, sizeof(double) * 3 * nbl, cudaMemcpyDeviceToDevice, s));
-    else ck(cudaMemsetAsync(g->blobS, 0, sizeof(double) * 3 * std::max(nbl, 1), s));
-    axpby<double>(g->blobS, g->blobA, 1.0, 1.0, 3 * (i64)nbl, s);
-    axpby<double>(g->blobS, g->blobC, -1.0, 1.0, 3 * (i64)nbl, s);
-    axpby<double>(g->blobS, g->blobD, -1.0, 1.0, 3 * (i64)nbl, s);
-    axpby<double>(g->bodyF, g->bodyA, -1.0, 1.0, 6 * (i64)nb, s);
+    // step 5: random finite differences; F_tot = F - D^{K^T},
+    // slip_tot = slip + D^K - D^J - D^S
+    rfd_force(nb, g->boff, g->plus.arm, g->minus.arm, lam_rfd, 1.0 / delta, g->bodyF, s);
+    rfd_slip(g->d, view_of(g, g->cur), g->plus.r, g->minus.r, g->plus.arm, g->minus.arm, v_rfd, U_rfd, g->xvec, p->slip,
+             1.0 / delta, g->blobS, s);
   }
   // step 6: fluctuating constrained solve
   normals(1u, g->stress.total, g->Wst);
