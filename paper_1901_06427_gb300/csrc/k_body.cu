@@ -591,7 +591,7 @@ __global__ void __launch_bounds__(256) k_body_apply(int nbl, const int* __restri
                                                     const i64* __restrict__ shape_off, const float* __restrict__ Bs,
                                                     const double* __restrict__ quat, const float* __restrict__ r,
                                                     float* __restrict__ z, double* __restrict__ z64, Dims d,
-                                                    const BlobStencil<float>* __restrict__ tab, const float* __restrict__ v) {
+                                                    const BlobStencil<float>* __restrict__ tab, const float* __restrict__ vel) {
   pdl_entry();
   extern __shared__ __align__(16) float sh[];
   const int p = blockIdx.x, b0 = boff[p], n3 = 3 * (boff[p + 1] - b0), n = n3 + 6, ld = body_ld(n);
@@ -603,19 +603,27 @@ __global__ void __launch_bounds__(256) k_body_apply(int nbl, const int* __restri
   if (wid < n)
 #pragma unroll
     for (int q = 0; q < kBodyPre; ++q) pre[q] = body_word(B + (i64)wid * ld, ld, lane + 32 * q);
-  double R[9];
-  quat_rot(quat + 4 * p, R);
+  // FP64 costs a warp instruction whatever its lanes do: the rotation by one
+  // warp, the turns by one thread per component
+  __shared__ double R[9];
+  if (wid == nw - 1) {
+    double Rr[9];
+    quat_rot(quat + 4 * p, Rr);
+#pragma unroll
+    for (int i = 0; i < 9; ++i)
+      if (lane == i) R[i] = Rr[i];
+  }
   for (int c = wid; c < n3; c += nw) {
-    const float s = r[3 * b0 + c] + warp_interp<float>(d, c % 3, tab + 3 * b0 + c, v, lane);
+    const float s = r[3 * b0 + c] + warp_interp<float>(d, c % 3, tab + 3 * b0 + c, vel, lane);
     if (lane == 0) x[c] = s;
   }
   if (threadIdx.x < 6) x[n3 + threadIdx.x] = r[3 * nbl + 6 * p + threadIdx.x];
   if (n + (int)threadIdx.x < ld) y[n + threadIdx.x] = 0.f;
   __syncthreads();
-  for (int i = threadIdx.x; i < n / 3; i += blockDim.x)
-#pragma unroll
-    for (int a = 0; a < 3; ++a)
-      y[3 * i + a] = (float)(R[a] * (double)x[3 * i] + R[3 + a] * (double)x[3 * i + 1] + R[6 + a] * (double)x[3 * i + 2]);
+  for (int t = threadIdx.x; t < n; t += blockDim.x) {
+    const int i = t / 3, a = t - 3 * i;
+    y[t] = (float)(R[a] * (double)x[3 * i] + R[3 + a] * (double)x[3 * i + 1] + R[6 + a] * (double)x[3 * i + 2]);
+  }
   __syncthreads();
   for (int row = wid; row < n; row += nw) {
     if (row != wid)
@@ -625,14 +633,12 @@ __global__ void __launch_bounds__(256) k_body_apply(int nbl, const int* __restri
     if (lane == 0) x[row] = t;
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < n / 3; i += blockDim.x) {
-    const int o = 3 * i < n3 ? 3 * (b0 + i) : 3 * nbl + 6 * p + 3 * i - n3;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      const float t = (float)(R[3 * a] * (double)x[3 * i] + R[3 * a + 1] * (double)x[3 * i + 1] + R[3 * a + 2] * (double)x[3 * i + 2]);
-      z[o + a] = t;
-      if (z64) z64[o + a] = (double)t;
-    }
+  for (int t = threadIdx.x; t < n; t += blockDim.x) {
+    const int i = t / 3, a = t - 3 * i;
+    const float v = (float)(R[3 * a] * (double)x[3 * i] + R[3 * a + 1] * (double)x[3 * i + 1] + R[3 * a + 2] * (double)x[3 * i + 2]);
+    const i64 o = t < n3 ? 3 * (i64)b0 + t : 3 * (i64)nbl + 6 * p + t - n3;
+    z[o] = v;
+    if (z64) z64[o] = (double)v;
   }
 }
 

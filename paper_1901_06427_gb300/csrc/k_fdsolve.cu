@@ -336,10 +336,10 @@ __global__ void __launch_bounds__(256) k_fdw_z(FDParams P, float* __restrict__ d
 // badly): driven monolayer step 299 -> 177 ms (704 -> 399 iterations),
 // 128 x 128 x 64 gradient 365 -> 104 ms (about 600 -> 230), boomerang slit
 // step 18.4 -> 14.0 ms.
-RBFIB_DEVFN void fold_pair(const FDAxis& X, int p, int& a, int& b) {
-  a = p;
-  b = X.fold == kFoldMirror ? X.e - 1 - p : (X.fold == kFoldPeriodic && p > 0 ? X.e - p : p);
-}
+// b = sum - p, but for the points that are their own mirror (fold_sum; the
+// point 0 of a periodic axis, every point without a mirror).
+RBFIB_DEVFN int fold_sum(const FDAxis& X) { return X.fold == kFoldMirror ? X.e - 1 : (X.fold == kFoldPeriodic ? X.e : -1); }
+RBFIB_DEVFN int fold_partner(int sum, int e, int p) { const int b = sum - p; return sum < 0 || b >= e ? p : b; }
 
 // Shape of a pass: 128 threads, 64 entries along the contiguous dimension of
 // memory (16 threads x 4 interleaved, so that stores of a warp are
@@ -457,8 +457,10 @@ __global__ void __launch_bounds__(kFLThreads) k_fdl_fwd(FDParams P, int axis, in
   typedef FdlTile<AX, TM> Tl;
   __shared__ __align__(16) Tl S;
   const FDGrid& G = P.g[blockIdx.z];
-  const FDAxis& X = G.ax[axis];
-  const int nl = G.e[0] * G.e[1] * G.e[2] / X.e, l0 = blockIdx.x * Tl::LT;
+  // in registers: a read of the parameters by a run-time index per staged
+  // entry would stall each one
+  const FDAxis X = G.ax[axis];
+  const int e0 = G.e[0], nl = e0 * G.e[1] * G.e[2] / X.e, l0 = blockIdx.x * Tl::LT, sum = fold_sum(X);
   const int nS = (X.hs + Tl::CT - 1) / Tl::CT, nA = (X.ha + Tl::CT - 1) / Tl::CT;
   if (l0 >= nl || (int)blockIdx.y >= nS + nA) return;
   const bool odd = (int)blockIdx.y >= nS;
@@ -477,13 +479,12 @@ __global__ void __launch_bounds__(kFLThreads) k_fdl_fwd(FDParams P, int axis, in
   fdl_product<AX, TM>(
       S, X.hs, P.tab + (odd ? X.fA : X.fS), odd ? X.pa : X.ps, c0,
       [&](int p, int l) {
-        int a, b;
-        fold_pair(X, p, a, b);
-        const float* line = src + (AX == 1 ? own : min(l0 + l, last) * G.e[0]);
+        const int b = fold_partner(sum, X.e, p);
+        const float* line = src + (AX == 1 ? own : min(l0 + l, last) * e0);
         // both points loaded without a branch, so that a stage's loads are in
         // flight together
-        const float va = line[a * st], vb = line[b * st];
-        return fmaf(a == b ? 0.f : sg, vb, va);
+        const float va = line[p * st], vb = line[b * st];
+        return fmaf(p == b ? 0.f : sg, vb, va);
       },
       acc);
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
@@ -515,8 +516,8 @@ __global__ void __launch_bounds__(kFLThreads) k_fdl_bwd(FDParams P, int axis, co
   typedef FdlTile<AX, TM> Tl;
   __shared__ __align__(16) Tl S;
   const FDGrid& G = P.g[blockIdx.z];
-  const FDAxis& X = G.ax[axis];
-  const int nl = G.e[0] * G.e[1] * G.e[2] / X.e, l0 = blockIdx.x * Tl::LT, p0 = blockIdx.y * Tl::CT;
+  const FDAxis X = G.ax[axis];
+  const int e0 = G.e[0], nl = e0 * G.e[1] * G.e[2] / X.e, l0 = blockIdx.x * Tl::LT, p0 = blockIdx.y * Tl::CT;
   if (l0 >= nl || p0 >= X.hs) return;
   const float* src = in + G.off;
   const int st = fdl_stride(G, axis), last = nl - 1;
@@ -528,12 +529,12 @@ __global__ void __launch_bounds__(kFLThreads) k_fdl_bwd(FDParams P, int axis, co
     for (int i = 0; i < 4; ++i) { ev[r][i] = 0.f; od[r][i] = 0.f; }
   fdl_product<AX, TM>(
       S, X.hs, P.tab + X.bS, X.ps, p0,
-      [&](int c, int l) { return src[(AX == 1 ? own : min(l0 + l, last) * G.e[0]) + c * st]; }, ev);
+      [&](int c, int l) { return src[(AX == 1 ? own : min(l0 + l, last) * e0) + c * st]; }, ev);
   if (X.ha > 0)
     fdl_product<AX, TM>(
         S, X.ha, P.tab + X.bA, X.ps, p0,
-        [&](int c, int l) { return src[(AX == 1 ? own : min(l0 + l, last) * G.e[0]) + (X.hs + c) * st]; }, od);
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+        [&](int c, int l) { return src[(AX == 1 ? own : min(l0 + l, last) * e0) + (X.hs + c) * st]; }, od);
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4, sum = fold_sum(X);
   float* dst = out + G.off;
 #pragma unroll
   for (int r = 0; r < TM; ++r)
@@ -542,11 +543,10 @@ __global__ void __launch_bounds__(kFLThreads) k_fdl_bwd(FDParams P, int axis, co
       const int co = tx + 16 * i, ot = TM * ty + r;
       const int l = l0 + (AX == 0 ? ot : co), p = p0 + (AX == 0 ? co : ot);
       if (l >= nl || p >= X.hs) continue;
-      int a, b;
-      fold_pair(X, p, a, b);
+      const int b = fold_partner(sum, X.e, p);
       float* line = dst + fdl_base(G, axis, l);
-      line[a * st] = ev[r][i] + od[r][i];
-      if (a != b) line[b * st] = ev[r][i] - od[r][i];
+      line[p * st] = ev[r][i] + od[r][i];
+      if (p != b) line[b * st] = ev[r][i] - od[r][i];
     }
 }
 

@@ -348,11 +348,14 @@ RBFIB_DEVFN void warp_spread(const Dims& d, int a, const BlobStencil<T>* __restr
                              int lane) {
   if (val == T(0)) return;
   T* fa = f + d.fo[a];
-  const int kw = d.kw, np = kw * kw * kw;
-  for (int p = lane; p < np; p += 32) {
-    const int x = p % kw, y = (p / kw) % kw, z = p / (kw * kw);
+  auto point = [&](int x, int y, int z) {
     const T w = S->w[x] * S->w[kKMax + y] * S->w[2 * kKMax + z];
     if (w != T(0)) atomicAdd(fa + flat3(d.fe[a], S->idx[x], S->idx[kKMax + y], S->idx[2 * kKMax + z]), w * val);
+  };
+  if (d.kw == 3) {
+    if (lane < 27) point(lane % 3, (lane / 3) % 3, lane / 9);
+  } else {
+    for (int p = lane; p < 216; p += 32) point(p % 6, (p / 6) % 6, p / 36);
   }
 }
 
@@ -397,71 +400,14 @@ void spread_tab(const Dims& d, const BodyView& b, const double* lam, double scal
   }
 }
 
-// --------------------------------------------------- saddle body rows (fused)
-// warps [0, 3 N_bl): y_lam = -J v + K U            (warp per blob component)
-// warps [3 N_bl, 3 N_bl + N_b): y_U = K^T lam       (warp per body, FP64 sums)
-// warps beyond: y_v -= S lam / dV                  (warp per blob component, bin order)
-template <typename T>
-__global__ void k_saddle_bodies(Dims d, BodyView b, const T* __restrict__ v, const T* __restrict__ lam,
-                                const T* __restrict__ U, T* __restrict__ yv, T* __restrict__ ylam, T* __restrict__ yU,
-                                double inv_dV) {
-  pdl_entry();
-  const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-  const int nA = 3 * b.nbl, nB = b.nb;
-  const BlobStencil<T>* tab = table_of<T>(b);
-  if (gw < nA) {
-    const int i = gw / 3, a = gw - 3 * i;
-    const T jv = warp_interp<T>(d, a, tab + gw, v, lane);
-    if (lane == 0) {
-      const int p = b.bob[i];
-      const double* ar = b.arm + 3 * i;
-      const double w0 = (double)U[6 * p + 3], w1 = (double)U[6 * p + 4], w2 = (double)U[6 * p + 5];
-      double cr;
-      if (a == 0) cr = w1 * ar[2] - w2 * ar[1];
-      else if (a == 1) cr = w2 * ar[0] - w0 * ar[2];
-      else cr = w0 * ar[1] - w1 * ar[0];
-      ylam[gw] = (T)(-(double)jv + ((double)U[6 * p + a] + cr));
-    }
-  } else if (gw < nA + nB) {
-    const int p = gw - nA;
-    double acc[6] = {0, 0, 0, 0, 0, 0};
-    for (int i = b.boff[p] + lane; i < b.boff[p + 1]; i += 32) {
-      const double lx = (double)lam[3 * i], ly = (double)lam[3 * i + 1], lz = (double)lam[3 * i + 2];
-      const double* ar = b.arm + 3 * i;
-      acc[0] += lx; acc[1] += ly; acc[2] += lz;
-      acc[3] += ar[1] * lz - ar[2] * ly;
-      acc[4] += ar[2] * lx - ar[0] * lz;
-      acc[5] += ar[0] * ly - ar[1] * lx;
-    }
-#pragma unroll
-    for (int c = 0; c < 6; ++c)
-      for (int o = 16; o > 0; o >>= 1) acc[c] += __shfl_xor_sync(0xffffffffu, acc[c], o);
-    if (lane < 6) yU[6 * p + lane] = (T)acc[lane];
-  } else if (gw < 2 * nA + nB) {
-    const int s = gw - nA - nB;
-    const int sb = s / 3, a = s - 3 * sb;
-    const int i = b.perm ? b.perm[sb] : sb;
-    warp_spread<T>(d, a, tab + 3 * i + a, (T)(-(double)lam[3 * i + a] * inv_dV), yv, lane);
-  }
-}
-
-template <typename T>
-void saddle_bodies(const Dims& d, const BodyView& b, const T* v, const T* lam, const T* U,
-                   T* yv, T* ylam, T* yU, cudaStream_t s) {
-  if (b.nbl == 0) return;
-  const i64 warps = 2 * 3 * (i64)b.nbl + b.nb;
-  const double inv_dV = 1.0 / (d.h[0] * d.h[1] * d.h[2]);
-  launch_k(k_saddle_bodies<T>, nblk(32 * warps, 128), 128, 0, s, d, b, v, lam, U, yv, ylam, yU, inv_dV);
-  note_launch();
-}
-
 // K^T lam of one body by a warp (FP64 sums), in every lane.
-RBFIB_DEVFN void warp_kt(int b0, int b1, const double* __restrict__ arm, const double* __restrict__ lam, int lane,
+template <typename T>
+RBFIB_DEVFN void warp_kt(int b0, int b1, const double* __restrict__ arm, const T* __restrict__ lam, int lane,
                          double acc[6]) {
 #pragma unroll
   for (int c = 0; c < 6; ++c) acc[c] = 0.0;
   for (int i = b0 + lane; i < b1; i += 32) {
-    const double lx = lam[3 * i], ly = lam[3 * i + 1], lz = lam[3 * i + 2];
+    const double lx = (double)lam[3 * i], ly = (double)lam[3 * i + 1], lz = (double)lam[3 * i + 2];
     const double* ar = arm + 3 * i;
     acc[0] += lx; acc[1] += ly; acc[2] += lz;
     acc[3] += ar[1] * lz - ar[2] * ly;
@@ -470,6 +416,76 @@ RBFIB_DEVFN void warp_kt(int b0, int b1, const double* __restrict__ arm, const d
   }
 #pragma unroll
   for (int c = 0; c < 6; ++c) acc[c] = warp_add(acc[c]);
+}
+
+// --------------------------------------------------- saddle body rows (fused)
+// Blocks below nA take per blob components each, in bin order: a warp per
+// component gathers J v and scatters y_v -= S lam / dV with one reading of
+// its stencil; then a thread per component forms y_lam = -J v + K U in FP64
+// (an FP64 instruction costs the warp the same for one lane as for 32: with
+// one component per warp these few took half the time of the monolayer's
+// 36,864 components).  Small suspensions (split), whose blocks leave the GPU
+// idle, scatter in nA blocks of their own instead of after the gather (cavity
+// step 5.39 -> 5.2 ms).  The last blocks: a warp per body, y_U = K^T lam (FP64
+// sums).
+template <typename T>
+__global__ void __launch_bounds__(kPosThreads) k_saddle_bodies(Dims d, BodyView b, int per, int nA, int split,
+                                                               const T* __restrict__ v, const T* __restrict__ lam,
+                                                               const T* __restrict__ U, T* __restrict__ yv,
+                                                               T* __restrict__ ylam, T* __restrict__ yU, double inv_dV) {
+  pdl_entry();
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, n = 3 * b.nbl;
+  const BlobStencil<T>* tab = table_of<T>(b);
+  const int ncomp = split ? 2 * nA : nA;   // blocks of components
+  if ((int)blockIdx.x >= ncomp) {
+    const int p = ((int)blockIdx.x - ncomp) * (kPosThreads / 32) + wid;
+    if (p >= b.nb) return;
+    double acc[6];
+    warp_kt(b.boff[p], b.boff[p + 1], b.arm, lam, lane, acc);
+#pragma unroll
+    for (int c = 0; c < 6; ++c)
+      if (lane == c) yU[6 * p + c] = (T)acc[c];
+    return;
+  }
+  __shared__ T jv[kPosMax];
+  __shared__ int row[kPosMax];
+  const bool scatter = !split || (int)blockIdx.x >= nA, gather = !split || (int)blockIdx.x < nA;
+  const int c0 = ((int)blockIdx.x < nA ? (int)blockIdx.x : (int)blockIdx.x - nA) * per;
+  for (int q = wid; q < per && c0 + q < n; q += kPosThreads / 32) {
+    const int s = (c0 + q) / 3, a = c0 + q - 3 * s;
+    const int c = 3 * (b.perm ? b.perm[s] : s) + a;
+    if (gather) {
+      const T j = warp_interp<T>(d, a, tab + c, v, lane);
+      if (lane == 0) { jv[q] = j; row[q] = c; }
+    }
+    if (scatter) warp_spread<T>(d, a, tab + c, (T)(-(double)lam[c] * inv_dV), yv, lane);
+  }
+  if (!gather) return;
+  __syncthreads();
+  const int q = threadIdx.x;
+  if (q < per && c0 + q < n) {
+    const int c = row[q], i = c / 3, a = c - 3 * i, p = b.bob[i];
+    const double* ar = b.arm + 3 * i;
+    const double w0 = (double)U[6 * p + 3], w1 = (double)U[6 * p + 4], w2 = (double)U[6 * p + 5];
+    double cr;
+    if (a == 0) cr = w1 * ar[2] - w2 * ar[1];
+    else if (a == 1) cr = w2 * ar[0] - w0 * ar[2];
+    else cr = w0 * ar[1] - w1 * ar[0];
+    ylam[c] = (T)(-(double)jv[q] + ((double)U[6 * p + a] + cr));
+  }
+}
+
+template <typename T>
+void saddle_bodies(const Dims& d, const BodyView& b, const T* v, const T* lam, const T* U,
+                   T* yv, T* ylam, T* yU, cudaStream_t s) {
+  if (b.nbl == 0) return;
+  const int per = pos_per_block(3 * (i64)b.nbl);
+  const unsigned nA = nblk(3 * (i64)b.nbl, per);
+  const double inv_dV = 1.0 / (d.h[0] * d.h[1] * d.h[2]);
+  const int split = 2 * nA <= 4 * 152;
+  launch_k(k_saddle_bodies<T>, (split ? 2 : 1) * nA + nblk(b.nb, kPosThreads / 32), kPosThreads, 0, s, d, b, per, (int)nA,
+           split, v, lam, U, yv, ylam, yU, inv_dV);
+  note_launch();
 }
 
 // F -= D^{K^T} = (K+^T - K-^T) lam / delta (Algorithm 1 step 5), a warp per body
