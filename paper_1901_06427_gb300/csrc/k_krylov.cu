@@ -685,9 +685,13 @@ RBFIB_DEVFN double givens_core(double* H, int ldh, double* cs, double* sn, doubl
   }
   __syncthreads();
   if (threadIdx.x == 0) {
-    const double a = carry_out, b = sqrt(fmax(hnext2[0], 0.0));
-    const double r = hypot(a, b);
-    const double cj = r > 0 ? a / r : 1.0, sj = r > 0 ? b / r : 0.0;
+    // r = hypot(a, b), b = ||w||, from squares: b^2 is at hand, b is needed
+    // only beside the chain, and one reciprocal square root gives both 1 / r
+    // and r (the library's hypot and two divisions were half of this step)
+    const double a = carry_out, b2 = fmax(hnext2[0], 0.0), b = sqrt(b2);
+    const double d2 = fma(a, a, b2);
+    const double ir = d2 > 0.0 ? rsqrt(d2) : 0.0, r = d2 * ir;
+    const double cj = r > 0 ? a * ir : 1.0, sj = r > 0 ? b * ir : 0.0;
     cs[j] = cj; sn[j] = sj;
     h[j] = r;
     h[j + 1] = 0.0;
