@@ -277,27 +277,6 @@ __device__ inline void philox4x64_10(unsigned long long c[4], unsigned long long
   }
 }
 
-__device__ inline double philox_uniform(unsigned long long w) {
-  return (double)((w >> 12) * 2ULL + 1ULL) * 0x1.0p-53;
-}
-
-// Four standard normals of Philox block b of stream (seed, step, attempt, purpose).
-__device__ inline void philox_normals4(unsigned long long seed, unsigned long long step,
-                                       unsigned attempt, unsigned purpose,
-                                       unsigned long long b, double out[4]) {
-  unsigned long long c[4] = {b, step, ((unsigned long long)attempt << 32) | purpose, 0ULL};
-  philox4x64_10(c, seed, 0ULL);
-#pragma unroll
-  for (int pr = 0; pr < 2; ++pr) {
-    const double u0 = philox_uniform(c[2 * pr]), u1 = philox_uniform(c[2 * pr + 1]);
-    const double rad = sqrt(-2.0 * log(u0));
-    double sn, cs;
-    sincospi(2.0 * u1, &sn, &cs);
-    out[2 * pr] = rad * cs;
-    out[2 * pr + 1] = rad * sn;
-  }
-}
-
 #define RBFIB_DEVFN __device__ __forceinline__
 
 // (J v)_ia by one warp.  Three-point kernel: lane l < 27 takes kernel point

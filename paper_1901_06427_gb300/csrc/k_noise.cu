@@ -3,10 +3,34 @@
 // zero weights on free-slip wall edges.
 #include "common.cuh"
 #include "kernels.cuh"
+#include "normals.cuh"
 
 namespace rbfib {
 
 static inline unsigned nblk(i64 n, int bs) { return (unsigned)((n + bs - 1) / bs); }
+
+// Four standard normals of Philox block b of stream (seed, step, attempt, purpose).
+__device__ __forceinline__ void philox_normals4(unsigned long long seed, unsigned long long step, unsigned attempt,
+                                                unsigned purpose, unsigned long long b, double out[4]) {
+  unsigned long long c[4] = {b, step, ((unsigned long long)attempt << 32) | purpose, 0ULL};
+  philox4x64_10(c, seed, 0ULL);
+  box_muller(c[0], c[1], out[0], out[1]);
+  box_muller(c[2], c[3], out[2], out[3]);
+}
+
+// The normals of block b into out[4 b ..), up to count: two 16-byte stores
+// where out allows them.
+__device__ __forceinline__ void store4(const double z[4], i64 b, i64 count, double* __restrict__ out) {
+  if (4 * b + 3 < count && (reinterpret_cast<uintptr_t>(out) & 15) == 0) {
+    double2* o = reinterpret_cast<double2*>(out + 4 * b);
+    o[0] = make_double2(z[0], z[1]);
+    o[1] = make_double2(z[2], z[3]);
+    return;
+  }
+#pragma unroll
+  for (int l = 0; l < 4; ++l)
+    if (4 * b + l < count) out[4 * b + l] = z[l];
+}
 
 __global__ void k_philox_normals(unsigned long long seed, unsigned long long step, unsigned attempt,
                                  unsigned purpose, i64 count, double* __restrict__ out) {
@@ -15,9 +39,7 @@ __global__ void k_philox_normals(unsigned long long seed, unsigned long long ste
   if (4 * b >= count) return;
   double z[4];
   philox_normals4(seed, step, attempt, purpose, (unsigned long long)b, z);
-#pragma unroll
-  for (int l = 0; l < 4; ++l)
-    if (4 * b + l < count) out[4 * b + l] = z[l];
+  store4(z, b, count, out);
 }
 
 void philox_normals(unsigned long long seed, unsigned long long step, unsigned attempt, unsigned purpose,
@@ -39,9 +61,7 @@ __global__ void k_philox_normals_p(const unsigned long long* __restrict__ sp, un
   if (4 * b >= count) return;
   double z[4];
   philox_normals4(sp[0], sp[1], (unsigned)sp[2], purpose, (unsigned long long)b, z);
-#pragma unroll
-  for (int l = 0; l < 4; ++l)
-    if (4 * b + l < count) out[4 * b + l] = z[l];
+  store4(z, b, count, out);
 }
 
 void philox_normals_p(const unsigned long long* sp, unsigned purpose, i64 count, double* out, cudaStream_t s) {
