@@ -289,15 +289,35 @@ __global__ void __launch_bounds__(256) k_gs_dot(const T* __restrict__ w, const T
   __syncthreads();
   if (!last) return;
   __threadfence();
-  // one warp per column: partials of the blocks, then the body entries
+  // a warp per column (few blocks: per four columns, their chains in flight
+  // together): partials of the blocks, then the body entries
+  constexpr int U = R == 1 ? 4 : 1;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  for (int c = wid; c < k; c += nw) {
-    double t = 0.0, body = 0.0;
-    for (int i = lane; i < (int)gridDim.x; i += 32) t += __ldcg(part + (i64)c * gridDim.x + i);
+  for (int c = wid; c < k; c += U * nw) {
+    double t[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int cu = c + u * nw;
+      t[u] = 0.0;
+      if (cu < k)
+        for (int i = lane; i < (int)gridDim.x; i += 32) t[u] += __ldcg(part + (i64)cu * gridDim.x + i);
+    }
     if (wf != 1.0)
-      for (i64 i = nfl + lane; i < n; i += 32) body = fma((double)w[i], (double)V[(i64)c * ldv + i], body);
-    t = warp_sum(wf * t + (1.0 - wf) * body);
-    if (lane == 0) out[c] = t;
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int cu = c + u * nw;
+        double body = 0.0;
+        if (cu < k)
+          for (i64 i = nfl + lane; i < n; i += 32) body = fma((double)w[i], (double)V[(i64)cu * ldv + i], body);
+        t[u] = wf * t[u] + (1.0 - wf) * body;
+      }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+      for (int u = 0; u < U; ++u) t[u] += __shfl_xor_sync(0xffffffffu, t[u], o);
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (lane == 0 && c + u * nw < k) out[c + u * nw] = t[u];
   }
 }
 
@@ -319,7 +339,8 @@ __global__ void __launch_bounds__(256) k_gs_axpy(T* __restrict__ w, const T* __r
   for (int i = threadIdx.x; i < k; i += blockDim.x) cf[i] = (A)(sign * coef[i]);
   __syncthreads();
   const i64 nv = n / W;
-  const i64 chunk = 256 * (i64)R;
+  const int bd = blockDim.x;
+  const i64 chunk = bd * (i64)R;
   const i64 nchunks = (nv + chunk - 1) / chunk;
   VT* w4 = reinterpret_cast<VT*>(w);
   A nrm = (A)0;
@@ -328,7 +349,7 @@ __global__ void __launch_bounds__(256) k_gs_axpy(T* __restrict__ w, const T* __r
     VT x[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-      const i64 i = base + (i64)r * 256;
+      const i64 i = base + (i64)r * bd;
       if (i < nv) x[r] = w4[i]; else zero16(x[r]);
     }
     int c = 0;
@@ -339,7 +360,7 @@ __global__ void __launch_bounds__(256) k_gs_axpy(T* __restrict__ w, const T* __r
         const A f = cf[c + u];
 #pragma unroll
         for (int r = 0; r < R; ++r) {
-          const i64 i = base + (i64)r * 256;
+          const i64 i = base + (i64)r * bd;
           if (i < nv) axpy16(f, v4[i], x[r]);
         }
       }
@@ -349,13 +370,13 @@ __global__ void __launch_bounds__(256) k_gs_axpy(T* __restrict__ w, const T* __r
       const A f = cf[c];
 #pragma unroll
       for (int r = 0; r < R; ++r) {
-        const i64 i = base + (i64)r * 256;
+        const i64 i = base + (i64)r * bd;
         if (i < nv) axpy16(f, v4[i], x[r]);
       }
     }
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-      const i64 i = base + (i64)r * 256;
+      const i64 i = base + (i64)r * bd;
       if (i < nv) {
         w4[i] = x[r];
         nrm = dot16(x[r], x[r], nrm);
@@ -391,14 +412,20 @@ __global__ void __launch_bounds__(256) k_gs_axpy(T* __restrict__ w, const T* __r
   }
 }
 
-// Row blocks of a register-blocked sweep: one per chunk of 256 R vectors, so
+// Row blocks of a register-blocked sweep: one per chunk of vectors, so
 // that no block carries a second chunk while others idle (a block that does
 // finishes last and sets the launch's duration), capped by the partial
 // buffer's nparts slots per column on large grids.
-inline int gs_blocks(i64 nv, int R, int nparts) {
-  const i64 chunks = (nv + 256 * (i64)R - 1) / (256 * (i64)R);
-  return (int)std::max<i64>(1, std::min<i64>(chunks, nparts));
+inline int gs_blocks(i64 nv, i64 chunk, int nparts) {
+  return (int)std::max<i64>(1, std::min<i64>((nv + chunk - 1) / chunk, nparts));
 }
+// Vectors below which a sweep takes one per thread (multi-axpy: blocks of 64
+// threads): the 4 k unknowns of a 16 x 8 x 8 box fill two blocks of the wide
+// chunks, whose share of the FP64 pipe (2 FMAs per SM and clock) is then the
+// launch's time (step 5.18 -> 4.85 ms).  From some 32 k unknowns on the wide
+// chunks' fewer partial sums win (Stokes solve on 45 x 37 x 29: 2.51 against
+// 2.67 ms).
+constexpr i64 kGSNarrow = 16 * 1024;
 
 // plain sum of nparts partials
 __global__ void k_sum_finish(const double* __restrict__ part, int nparts, double* __restrict__ out) {
@@ -420,10 +447,11 @@ template <typename T>
 void multi_dot(const T* w, const T* V, i64 ldv, int ncols, i64 n, i64 nfl, double wf, double* part, int nparts,
                double* out, cudaStream_t s, const int* gate) {
   if (vec_ok(w, V, ldv, ncols) && ncols <= kGivensMaxCols) {
-    constexpr int R = 4;
     const int groups = (ncols + kCG - 1) / kCG;
-    const int nb = gs_blocks(n / Vec16<T>::w, R, nparts);
-    launch_k(k_gs_dot<T, R>, dim3(nb, groups), 256, 0, s, w, V, ldv, ncols, n, nfl, wf, part,
+    const i64 nv = n / Vec16<T>::w;
+    const bool wide = nv >= kGSNarrow;
+    const int nb = gs_blocks(nv, wide ? 1024 : 256, nparts);
+    launch_k(wide ? k_gs_dot<T, 4> : k_gs_dot<T, 1>, dim3(nb, groups), 256, 0, s, w, V, ldv, ncols, n, nfl, wf, part,
              part_counters(part, nparts) + kDotCounter, out, gate);
     note_launch();
     return;
@@ -539,9 +567,11 @@ void multi_axpy(T* w, const T* V, i64 ldv, int ncols, const double* coef, double
                 double* part, int nparts, double* nrm2, cudaStream_t s, const ReorthCtl* ctl, const int* gate) {
   const ReorthCtl c = (ctl && nrm2) ? *ctl : ReorthCtl{nullptr, nullptr, 0.0, 0, 0};
   if (vec_ok(w, V, ldv, ncols) && ncols <= kGivensMaxCols) {
-    constexpr int R = 2;
-    const int nb = gs_blocks(n / Vec16<T>::w, R, nparts);
-    launch_k(k_gs_axpy<T, R>, nb, 256, 0, s, w, V, ldv, ncols, coef, sign, n, nfl, wf, part,
+    const i64 nv = n / Vec16<T>::w;
+    const bool wide = nv >= kGSNarrow;
+    const int bs = wide ? 256 : 64;
+    const int nb = gs_blocks(nv, wide ? 512 : bs, nparts);
+    launch_k(wide ? k_gs_axpy<T, 2> : k_gs_axpy<T, 1>, nb, bs, 0, s, w, V, ldv, ncols, coef, sign, n, nfl, wf, part,
              part_counters(part, nparts) + kAxpyCounter, nrm2, c, gate);
     note_launch();
     return;
