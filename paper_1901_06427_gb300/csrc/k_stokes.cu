@@ -271,8 +271,8 @@ inline void launch_cols(dim3 gr, cudaStream_t s, const Dims& d, double eta, cons
 }
 
 // Pipelined 2.5D Stokes operator for large grids (uniform spacing).  A 32 x 8
-// block owns a 32 x 8 tile of all four grids and marches a chunk of kPZ
-// z-planes.  Each plane of the tile, with a one-point halo in x and y, is
+// block owns a 32 x 8 tile of all four grids and marches a chunk of pz
+// z-planes (pipe_planes).  Each plane of the tile, with a one-point halo in x and y, is
 // copied into a ring of kPS shared-memory stages by cp.async, kPD planes ahead
 // of the plane being computed, so every thread keeps several planes of loads
 // in flight instead of waiting on each one.  All neighbours (x, y from the
@@ -280,7 +280,7 @@ inline void launch_cols(dim3 gr, cudaStream_t s, const Dims& d, double eta, cons
 // one barrier per plane.  Each staged value is fetched from global memory
 // once per block (halo rows and planes are shared with neighbouring blocks
 // through L2).
-constexpr int kPX = 32, kPY = 8, kPZ = 32;
+constexpr int kPX = 32, kPY = 8;
 constexpr int kPW = kPX + 2, kPH = kPY + 2, kPSlots = kPW * kPH;   // staged plane of one grid
 constexpr int kPLoads = (kPSlots + kPX * kPY - 1) / (kPX * kPY);    // slots per thread
 // planes in flight ahead of the one computed, and ring stages (the planes
@@ -290,6 +290,20 @@ template <typename T> __host__ __device__ constexpr int pipe_depth() { return si
 template <typename T> __host__ __device__ constexpr int pipe_stages() { return pipe_depth<T>() + 3; }
 template <typename T>
 __host__ __device__ constexpr int pipe_smem_bytes() { return pipe_stages<T>() * 4 * kPSlots * (int)sizeof(T); }
+
+// Planes per block.  Grids that give every SM four blocks of kPZ planes take
+// those; smaller ones the z axis in even chunks of at most kPZSmall, for more
+// blocks (with 32 planes a 100 x 90 x 76 grid had 144, a third of them of 12
+// planes): FP64 matvec of 100 x 90 x 76 127 -> 101 us, 130 x 120 x 110 211 ->
+// 188 us, FP32 47.5 -> 45 us.  At 256^3 the short chunks' extra halo planes cost
+// 1.5%.
+constexpr int kPZ = 32, kPZSmall = 13;
+inline int pipe_planes(const Dims& d) {
+  const i64 tiles = (i64)((d.n[0] + kPX - 1) / kPX) * ((d.n[1] + kPY - 1) / kPY);
+  if (tiles * ((d.n[2] + kPZ - 1) / kPZ) >= 4 * 152) return kPZ;
+  const int chunks = (d.n[2] + kPZSmall - 1) / kPZSmall;
+  return (d.n[2] + chunks - 1) / chunks;
+}
 
 // Copies one element, or writes zero to the slot when nbytes == 0 (the source
 // is then not read).
@@ -313,15 +327,17 @@ RBFIB_DEVFN void cp_async_commit() { asm volatile("cp.async.commit_group;\n" :::
 template <int N>
 RBFIB_DEVFN void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
 
-template <typename T, bool PX, bool PY, bool PZ>
-RBFIB_DEVFN void stokes_pipe_body(const Dims& d, T eta, const T* __restrict__ v, const T* __restrict__ p,
+// CZ: planes per block when known at compile time (kPZ; 1% at 256^3), else 0.
+template <typename T, bool PX, bool PY, bool PZ, int CZ>
+RBFIB_DEVFN void stokes_pipe_body(const Dims& d, int rpz, T eta, const T* __restrict__ v, const T* __restrict__ p,
                                   T* __restrict__ yv, T* __restrict__ yp, T* sm) {
   constexpr int kPD = pipe_depth<T>(), kPS = pipe_stages<T>();
   const int tx = threadIdx.x, ty = threadIdx.y, tid = tx + kPX * ty;
   const int x0 = blockIdx.x * kPX, y0 = blockIdx.y * kPY;
-  const int k0 = blockIdx.z * kPZ;
+  const int pz = CZ > 0 ? CZ : rpz;
+  const int k0 = blockIdx.z * pz;
   const int nx = d.n[0], ny = d.n[1], nz = d.n[2];
-  const int k1 = min(k0 + kPZ, nz);
+  const int k1 = min(k0 + pz, nz);
   // grid g = 0, 1, 2: face components; g = 3: pressure cells
   const T* src[4] = {v + d.fo[0], v + d.fo[1], v + d.fo[2], p};
   unsigned psz[4];
@@ -446,8 +462,11 @@ RBFIB_DEVFN void stokes_pipe_body(const Dims& d, T eta, const T* __restrict__ v,
 #pragma unroll
     for (int g = 0; g < 4; ++g) zp[g] = Sp[g * kPSlots + c0];
     stm = st0;
-    // ghosts across the z walls for the tangential components
-    const T zadj = PZ ? T(0) : s * (T)((k == 0 ? d.gd[4] : 0) + (k == nz - 1 ? d.gd[5] : 0));
+    // ghosts across the z walls for the tangential components; in FP64 on the
+    // planes next to the walls only (block-uniform: no FP64 work elsewhere)
+    const bool zw = !PZ && (sizeof(T) == 4 || k == 0 || k == nz - 1);
+    T zadj = T(0);
+    if (zw) zadj = s * (T)((k == 0 ? d.gd[4] : 0) + (k == nz - 1 ? d.gd[5] : 0));
     const T pc = zc[3];
     T um[3], ux[3], uy[3];
 #pragma unroll
@@ -458,7 +477,8 @@ RBFIB_DEVFN void stokes_pipe_body(const Dims& d, T eta, const T* __restrict__ v,
       uy[a] = U0[c0 - kPW];
       const T yq = U0[c0 + kPW];
       const T nb = ((um[a] + ux[a]) + (uy[a] + yq)) + (zm[a] + zp[a]);
-      const T sd = a != 2 ? sdiag[a] + zadj : sdiag[a];
+      T sd = sdiag[a];
+      if (a != 2 && zw) sd += zadj;
       T dp;
       if (a == 0) dp = pxw ? S0[3 * kPSlots + c0 + 1] - pc : pc - S0[3 * kPSlots + c0 - 1];
       else if (a == 1) dp = pyw ? S0[3 * kPSlots + c0 + kPW] - pc : pc - S0[3 * kPSlots + c0 - kPW];
@@ -480,23 +500,29 @@ RBFIB_DEVFN void stokes_pipe_body(const Dims& d, T eta, const T* __restrict__ v,
   asm volatile("cp.async.wait_all;\n" ::: "memory");
 }
 
-template <typename T, bool PX, bool PY, bool PZ>
+template <typename T, bool PX, bool PY, bool PZ, int CZ>
 __global__ void __launch_bounds__(kPX * kPY, sizeof(T) == 4 ? 4 : 3)
-    k_stokes_pipe(Dims d, T eta, const T* __restrict__ v, const T* __restrict__ p, T* __restrict__ yv,
+    k_stokes_pipe(Dims d, int pz, T eta, const T* __restrict__ v, const T* __restrict__ p, T* __restrict__ yv,
                   T* __restrict__ yp) {
   pdl_entry();
   extern __shared__ __align__(16) unsigned char pipe_smem[];
-  stokes_pipe_body<T, PX, PY, PZ>(d, eta, v, p, yv, yp, reinterpret_cast<T*>(pipe_smem));
+  stokes_pipe_body<T, PX, PY, PZ, CZ>(d, pz, eta, v, p, yv, yp, reinterpret_cast<T*>(pipe_smem));
+}
+template <typename T, bool PX, bool PY, bool PZ, int CZ>
+void launch_pipe_cz(const Dims& d, int pz, cudaStream_t s, T eta, const T* v, const T* p, T* yv, T* yp) {
+  static std::once_flag f;
+  std::call_once(f, [] {
+    cudaFuncSetAttribute(k_stokes_pipe<T, PX, PY, PZ, CZ>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         pipe_smem_bytes<T>());
+  });
+  dim3 gr((d.n[0] + kPX - 1) / kPX, (d.n[1] + kPY - 1) / kPY, (d.n[2] + pz - 1) / pz);
+  launch_k(k_stokes_pipe<T, PX, PY, PZ, CZ>, gr, dim3(kPX, kPY), pipe_smem_bytes<T>(), s, d, pz, eta, v, p, yv, yp);
 }
 template <typename T, bool PX, bool PY, bool PZ>
 void launch_pipe_as(const Dims& d, cudaStream_t s, T eta, const T* v, const T* p, T* yv, T* yp) {
-  static std::once_flag f;
-  std::call_once(f, [] {
-    cudaFuncSetAttribute(k_stokes_pipe<T, PX, PY, PZ>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         pipe_smem_bytes<T>());
-  });
-  dim3 gr((d.n[0] + kPX - 1) / kPX, (d.n[1] + kPY - 1) / kPY, (d.n[2] + kPZ - 1) / kPZ);
-  launch_k(k_stokes_pipe<T, PX, PY, PZ>, gr, dim3(kPX, kPY), pipe_smem_bytes<T>(), s, d, eta, v, p, yv, yp);
+  const int pz = pipe_planes(d);
+  if (pz == kPZ) launch_pipe_cz<T, PX, PY, PZ, kPZ>(d, pz, s, eta, v, p, yv, yp);
+  else launch_pipe_cz<T, PX, PY, PZ, 0>(d, pz, s, eta, v, p, yv, yp);
 }
 template <typename T>
 void launch_pipe(const Dims& d, cudaStream_t s, T eta, const T* v, const T* p, T* yv, T* yp) {
