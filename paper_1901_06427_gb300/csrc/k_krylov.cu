@@ -91,9 +91,8 @@ RBFIB_DEVFN void reorth_decide(const ReorthCtl& ctl, double nrm2w, const double*
 template <typename T>
 __global__ void k_dot_part(const T* __restrict__ w, const T* __restrict__ V, i64 ldv, i64 n, i64 nfl, double wf,
                            double* __restrict__ part, unsigned* __restrict__ cnt, double* __restrict__ out,
-                           int vec, const int* __restrict__ gate) {
+                           int vec) {
   pdl_entry();
-  if (gate && *gate == 0) return;
   const int col = blockIdx.y;
   const T* v = V + (i64)col * ldv;
   const i64 stride = (i64)gridDim.x * blockDim.x, t0 = (i64)blockIdx.x * blockDim.x + threadIdx.x;
@@ -225,20 +224,23 @@ RBFIB_DEVFN double block_transpose_sum8(A acc[kCG]) {
 // the last block to finish (one counter for the launch) adds them up with
 // the body-entry weight correction.
 template <typename T, int R>
-__global__ void __launch_bounds__(256) k_gs_dot(const T* __restrict__ w, const T* __restrict__ V, i64 ldv, int k,
+__global__ void __launch_bounds__(256) k_gs_dot(const T* __restrict__ w, const T* __restrict__ V, i64 ldv, int kmax,
                                                 i64 n, i64 nfl, double wf, double* __restrict__ part,
                                                 unsigned* __restrict__ cnt, double* __restrict__ out,
-                                                const int* __restrict__ gate) {
+                                                const int* __restrict__ kdev) {
   pdl_entry();
-  if (gate && *gate == 0) return;
+  const int k = kdev ? min(kdev[0] + 1, kmax) : kmax;
+  // column groups in use (with kdev the grid has those of kmax columns)
+  const int groups = (k + kCG - 1) / kCG;
+  if ((int)blockIdx.y >= groups) return;
   typedef typename Vec16<T>::t VT;
   typedef typename Vec16<T>::acc A;
   constexpr int W = Vec16<T>::w;
   const i64 nv = n / W;
   const i64 chunk = 256 * (i64)R;
   const i64 nchunks = (nv + chunk - 1) / chunk;
-  // columns split evenly over the groups (gridDim.y): at most kCG each
-  const int cpg = (k + gridDim.y - 1) / gridDim.y;
+  // columns split evenly over the groups: at most kCG each
+  const int cpg = (k + groups - 1) / groups;
   const int c0 = blockIdx.y * cpg, c1 = min(k, c0 + cpg);
   const VT* w4 = reinterpret_cast<const VT*>(w);
   A acc[kCG];
@@ -283,7 +285,7 @@ __global__ void __launch_bounds__(256) k_gs_dot(const T* __restrict__ w, const T
   if (threadIdx.x == 0) {
     __threadfence();
     const unsigned done = atomicAdd(cnt, 1u);
-    last = done == gridDim.x * gridDim.y - 1;
+    last = done == gridDim.x * groups - 1;
     if (last) *cnt = 0u;
   }
   __syncthreads();
@@ -325,13 +327,12 @@ __global__ void __launch_bounds__(256) k_gs_dot(const T* __restrict__ w, const T
 // per chunk), then, when nrm2 is not null, nrm2[0] = ||w||_W^2 of the result
 // (block sums, the last block adds them up with the body correction).
 template <typename T, int R>
-__global__ void __launch_bounds__(256) k_gs_axpy(T* __restrict__ w, const T* __restrict__ V, i64 ldv, int k,
+__global__ void __launch_bounds__(256) k_gs_axpy(T* __restrict__ w, const T* __restrict__ V, i64 ldv, int kmax,
                                                  const double* __restrict__ coef, double sign, i64 n, i64 nfl,
                                                  double wf, double* __restrict__ part, unsigned* __restrict__ cnt,
-                                                 double* __restrict__ nrm2, ReorthCtl ctl,
-                                                 const int* __restrict__ gate) {
+                                                 double* __restrict__ nrm2, ReorthCtl ctl, int* __restrict__ kdev) {
   pdl_entry();
-  if (gate && *gate == 0) return;
+  const int k = kdev ? min(kdev[0] + 1, kmax) : kmax;
   typedef typename Vec16<T>::t VT;
   typedef typename Vec16<T>::acc A;
   constexpr int W = Vec16<T>::w;
@@ -403,7 +404,10 @@ __global__ void __launch_bounds__(256) k_gs_axpy(T* __restrict__ w, const T* __r
       body = fma(x, x, body);
     }
   t = block_sum(wf * t + (1.0 - wf) * body);
-  if (threadIdx.x == 0) nrm2[0] = t;
+  if (threadIdx.x == 0) {
+    nrm2[0] = t;
+    if (kdev) kdev[kColOffset] = k - 1;
+  }
   if (ctl.flag) {
     __shared__ double tt;
     if (threadIdx.x == 0) tt = t;
@@ -445,21 +449,21 @@ inline int dot_blocks(i64 n, int nparts) {
 
 template <typename T>
 void multi_dot(const T* w, const T* V, i64 ldv, int ncols, i64 n, i64 nfl, double wf, double* part, int nparts,
-               double* out, cudaStream_t s, const int* gate) {
+               double* out, cudaStream_t s, const int* kdev) {
   if (vec_ok(w, V, ldv, ncols) && ncols <= kGivensMaxCols) {
     const int groups = (ncols + kCG - 1) / kCG;
     const i64 nv = n / Vec16<T>::w;
     const bool wide = nv >= kGSNarrow;
     const int nb = gs_blocks(nv, wide ? 1024 : 256, nparts);
     launch_k(wide ? k_gs_dot<T, 4> : k_gs_dot<T, 1>, dim3(nb, groups), 256, 0, s, w, V, ldv, ncols, n, nfl, wf, part,
-             part_counters(part, nparts) + kDotCounter, out, gate);
+             part_counters(part, nparts) + kDotCounter, out, kdev);
     note_launch();
     return;
   }
   const int nb = dot_blocks(n, nparts);
   dim3 grid(nb, ncols);
   launch_k(k_dot_part<T>, grid, 256, 0, s, w, V, ldv, n, nfl, wf, part, part_counters(part, nparts), out,
-           vec_ok(w, V, ldv, ncols), gate);
+           vec_ok(w, V, ldv, ncols));
   note_launch();
 }
 
@@ -469,9 +473,8 @@ template <typename T>
 __global__ void k_multi_axpy(T* __restrict__ w, const T* __restrict__ V, i64 ldv, int ncols,
                              const double* __restrict__ coef, double sign, i64 n, i64 nfl, double wf,
                              double* __restrict__ part, unsigned* __restrict__ cnt, double* __restrict__ nrm2,
-                             int vec, ReorthCtl ctl, const int* __restrict__ gate) {
+                             int vec, ReorthCtl ctl) {
   pdl_entry();
-  if (gate && *gate == 0) return;
   __shared__ double c[128];
   for (int i = threadIdx.x; i < ncols; i += blockDim.x) c[i] = sign * coef[i];
   __syncthreads();
@@ -564,7 +567,7 @@ __global__ void k_multi_axpy(T* __restrict__ w, const T* __restrict__ V, i64 ldv
 
 template <typename T>
 void multi_axpy(T* w, const T* V, i64 ldv, int ncols, const double* coef, double sign, i64 n, i64 nfl, double wf,
-                double* part, int nparts, double* nrm2, cudaStream_t s, const ReorthCtl* ctl, const int* gate) {
+                double* part, int nparts, double* nrm2, cudaStream_t s, const ReorthCtl* ctl, int* kdev) {
   const ReorthCtl c = (ctl && nrm2) ? *ctl : ReorthCtl{nullptr, nullptr, 0.0, 0, 0};
   if (vec_ok(w, V, ldv, ncols) && ncols <= kGivensMaxCols) {
     const i64 nv = n / Vec16<T>::w;
@@ -572,12 +575,12 @@ void multi_axpy(T* w, const T* V, i64 ldv, int ncols, const double* coef, double
     const int bs = wide ? 256 : 64;
     const int nb = gs_blocks(nv, wide ? 512 : bs, nparts);
     launch_k(wide ? k_gs_axpy<T, 2> : k_gs_axpy<T, 1>, nb, bs, 0, s, w, V, ldv, ncols, coef, sign, n, nfl, wf, part,
-             part_counters(part, nparts) + kAxpyCounter, nrm2, c, gate);
+             part_counters(part, nparts) + kAxpyCounter, nrm2, c, kdev);
     note_launch();
     return;
   }
   launch_k(k_multi_axpy<T>, nparts, 256, 0, s, w, V, ldv, ncols, coef, sign, n, nfl, wf, part,
-           part_counters(part, nparts) + kAxpyCounter, nrm2, vec_ok(w, V, ldv, ncols), c, gate);
+           part_counters(part, nparts) + kAxpyCounter, nrm2, vec_ok(w, V, ldv, ncols), c);
   note_launch();
 }
 
@@ -870,7 +873,7 @@ void wall_rhs(const Dims& d, const Walls& wl, double eta, T* bv, cudaStream_t s)
   template void multi_dot<T>(const T*, const T*, i64, int, i64, i64, double, double*, int, double*, cudaStream_t, \
                              const int*);                                                                        \
   template void multi_axpy<T>(T*, const T*, i64, int, const double*, double, i64, i64, double, double*, int,    \
-                              double*, cudaStream_t, const ReorthCtl*, const int*);                              \
+                              double*, cudaStream_t, const ReorthCtl*, int*);                                    \
   template void scale_by<T>(T*, const T*, const double*, int, i64, cudaStream_t, float*);                       \
   template void axpby<T>(T*, const T*, double, double, i64, cudaStream_t);                                      \
   template void wall_rhs<T>(const Dims&, const Walls&, double, T*, cudaStream_t);
@@ -885,14 +888,15 @@ template void convert<float, double>(const float*, double*, i64, cudaStream_t);
 // =================================================================
 // Device-side state of one restart cycle of FGMRES run as a CUDA graph.
 // ist: [0] columns done in this cycle k, [1] total iterations, [2] continue
-// flag; dpar: [0] absolute tolerance, [1] max iterations, [2] ||w||^2 of the
+// flag, [4], [5] the second Gram-Schmidt pass (ReorthCtl), [kColOffset] the
+// column being finished; dpar: [0] absolute tolerance, [1] max iterations, [2] ||w||^2 of the
 // current residual w (written by the cycle's last reduction).
 namespace rbfib {
 
 template <typename T>
 __global__ void k_fg_start(T* __restrict__ V0, const T* __restrict__ w, i64 n, double* __restrict__ gvec, int m,
                            int* __restrict__ ist, const double* __restrict__ dpar, float* __restrict__ V0_32,
-                           IterConds conds) {
+                           cudaGraphConditionalHandle loop) {
   pdl_entry();
   __shared__ double bs, fs;   // one thread per block forms beta and 1 / beta
   if (threadIdx.x == 0) {
@@ -911,18 +915,15 @@ __global__ void k_fg_start(T* __restrict__ V0, const T* __restrict__ w, i64 n, d
     for (int i = 1; i <= m; ++i) gvec[i] = 0.0;
     ist[0] = 0;
     ist[2] = 1;
+    cudaGraphSetConditional(loop, 1u);
   }
-  if (blockIdx.x == 0 && (int)threadIdx.x < conds.n)
-    cudaGraphSetConditional(conds.h[threadIdx.x], threadIdx.x == 0 ? 1u : 0u);
 }
 
 template <typename T>
 void fg_start(T* V0, const T* w, i64 n, double* gvec, int m, int* ist, const double* dpar, cudaStream_t s,
-              float* V0_32, const IterConds* conds) {
+              float* V0_32, cudaGraphConditionalHandle loop) {
   const unsigned nb = (unsigned)std::min<i64>(nblk(n, 256), 152 * 8);
-  IterConds c{};
-  if (conds) c = *conds;
-  launch_k(k_fg_start<T>, nb, 256, 0, s, V0, w, n, gvec, m, ist, dpar, V0_32, c);
+  launch_k(k_fg_start<T>, nb, 256, 0, s, V0, w, n, gvec, m, ist, dpar, V0_32, loop);
   note_launch();
 }
 
@@ -940,22 +941,23 @@ RBFIB_DEVFN void givens_flag_body(double* H, int ldh, double* cs, double* sn, do
   ist[2] = cont ? 1 : 0;
 }
 
-// The last two steps of a captured Arnoldi iteration in one launch, since
-// neither needs the other: blocks [0, gridDim.x - 1) normalise the new basis
-// vector, v = w / sqrt(nrm2) (and its FP32 copy when out32 is not null);
-// the last block applies the Givens update of column j and sets the continue
-// flag, and with use_next also the condition of the next iteration's IF node
-// (so no launch of its own sets it).  The update's FP64 recurrence then runs
-// beside the scaling instead of in a launch of its own.
+// The last steps of a captured Arnoldi iteration in one launch, since none
+// needs the others: blocks [0, gridDim.x - 1) normalise the new basis vector,
+// V_{j+1} = w / sqrt(nrm2) (and its FP32 copy out32), and keep the
+// preconditioned vector, Z_j = z; the last block applies the Givens update of
+// column j and sets the loop's condition.  j is read from ist[kColOffset],
+// where the multi-axpy put it: the last block moves ist[0] on to j + 1 while
+// others may not have started.
 template <typename T>
-__global__ void k_scale_givens(T* __restrict__ out, const T* __restrict__ in, i64 n, float* __restrict__ out32,
-                               double* H, int ldh, double* cs, double* sn, double* g, int j, const double* hcol,
-                               const double* hcol2, const double* nrm2, double* res_out, int* ist,
-                               const double* dpar, cudaGraphConditionalHandle next, int use_next) {
+__global__ void k_scale_givens(T* __restrict__ V, T* __restrict__ Z, i64 ld, const T* __restrict__ in,
+                               const T* __restrict__ z, i64 n, float* __restrict__ out32, double* H, int m, double* cs,
+                               double* sn, double* g, const double* hcol, const double* hcol2, const double* nrm2,
+                               double* res_out, int* ist, const double* dpar, cudaGraphConditionalHandle loop) {
   pdl_entry();
+  const int j = ist[kColOffset];
   if (blockIdx.x == gridDim.x - 1) {
-    givens_flag_body(H, ldh, cs, sn, g, j, hcol, hcol2, nrm2, res_out, ist, dpar);
-    if (use_next && threadIdx.x == 0) cudaGraphSetConditional(next, ist[2] ? 1u : 0u);
+    givens_flag_body(H, m + 1, cs, sn, g, j, hcol, hcol2, nrm2, res_out, ist, dpar);
+    if (threadIdx.x == 0) cudaGraphSetConditional(loop, ist[2] && j + 1 < m ? 1u : 0u);
     return;
   }
   __shared__ double fs;
@@ -965,29 +967,32 @@ __global__ void k_scale_givens(T* __restrict__ out, const T* __restrict__ in, i6
   }
   __syncthreads();
   const double f = fs;
+  T* out = V + (i64)(j + 1) * ld;
+  T* zj = Z + (i64)j * ld;
   const i64 stride = (i64)(gridDim.x - 1) * blockDim.x;
   for (i64 i = (i64)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
     const T v = (T)((double)in[i] * f);
     out[i] = v;
-    if (out32) out32[i] = (float)v;
+    out32[i] = (float)v;
+    zj[i] = z[i];
   }
 }
 
 template <typename T>
-void scale_givens(T* out, const T* in, i64 n, float* out32, double* H, int ldh, double* cs, double* sn, double* g,
-                  int j, const double* hcol, const double* hcol2, const double* nrm2, double* res_out, int* ist,
-                  const double* dpar, cudaStream_t s, const cudaGraphConditionalHandle* next) {
+void scale_givens(T* V, T* Z, i64 ld, const T* in, const T* z, i64 n, float* out32, double* H, int m, double* cs,
+                  double* sn, double* g, const double* hcol, const double* hcol2, const double* nrm2, double* res_out,
+                  int* ist, const double* dpar, cudaGraphConditionalHandle loop, cudaStream_t s) {
   const unsigned nb = (unsigned)std::min<i64>(nblk(n, 256), 152 * 8);
-  launch_k(k_scale_givens<T>, nb + 1, 256, 0, s, out, in, n, out32, H, ldh, cs, sn, g, j, hcol, hcol2, nrm2,
-           res_out, ist, dpar, next ? *next : cudaGraphConditionalHandle{}, next ? 1 : 0);
+  launch_k(k_scale_givens<T>, nb + 1, 256, 0, s, V, Z, ld, in, z, n, out32, H, m, cs, sn, g, hcol, hcol2, nrm2, res_out,
+           ist, dpar, loop);
   note_launch();
 }
-template void scale_givens<double>(double*, const double*, i64, float*, double*, int, double*, double*, double*,
-                                   int, const double*, const double*, const double*, double*, int*, const double*,
-                                   cudaStream_t, const cudaGraphConditionalHandle*);
-template void scale_givens<float>(float*, const float*, i64, float*, double*, int, double*, double*, double*, int,
-                                  const double*, const double*, const double*, double*, int*, const double*,
-                                  cudaStream_t, const cudaGraphConditionalHandle*);
+template void scale_givens<double>(double*, double*, i64, const double*, const double*, i64, float*, double*, int,
+                                   double*, double*, double*, const double*, const double*, const double*, double*,
+                                   int*, const double*, cudaGraphConditionalHandle, cudaStream_t);
+template void scale_givens<float>(float*, float*, i64, const float*, const float*, i64, float*, double*, int, double*,
+                                  double*, double*, const double*, const double*, const double*, double*, int*,
+                                  const double*, cudaGraphConditionalHandle, cudaStream_t);
 
 __global__ void __launch_bounds__(kTriMax) k_tri_dev(const double* H, int ldh, const double* g, const int* ist,
                                                      double* y) {
@@ -1035,9 +1040,9 @@ void multi_axpy_dev(T* w, const T* V, i64 ldv, const int* ist, const double* coe
 }
 
 template void fg_start<double>(double*, const double*, i64, double*, int, int*, const double*, cudaStream_t,
-                               float*, const IterConds*);
+                               float*, cudaGraphConditionalHandle);
 template void fg_start<float>(float*, const float*, i64, double*, int, int*, const double*, cudaStream_t, float*,
-                              const IterConds*);
+                              cudaGraphConditionalHandle);
 template void multi_axpy_dev<double>(double*, const double*, i64, const int*, const double*, double, i64, int,
                                      cudaStream_t);
 template void multi_axpy_dev<float>(float*, const float*, i64, const int*, const double*, double, i64, int,

@@ -204,13 +204,16 @@ struct ReorthCtl {
   cudaGraphConditionalHandle handle;
   int use_handle;
 };
-// gate (may be null): device flag; the launch does nothing when it is 0.
+// kdev (may be null): the sweep takes kdev[0] + 1 columns, at most ncols (16-
+// byte aligned vectors only); multi_axpy then leaves kdev[0] in
+// kdev[kColOffset].
+constexpr int kColOffset = 6;
 template <typename T> void multi_dot(const T* w, const T* V, i64 ldv, int ncols, i64 n, i64 nfl, double wf,
                                      double* part, int nparts, double* out, cudaStream_t,
-                                     const int* gate = nullptr);
+                                     const int* kdev = nullptr);
 template <typename T> void multi_axpy(T* w, const T* V, i64 ldv, int ncols, const double* coef, double sign,
                                       i64 n, i64 nfl, double wf, double* part, int nparts, double* nrm2,
-                                      cudaStream_t, const ReorthCtl* ctl = nullptr, const int* gate = nullptr);
+                                      cudaStream_t, const ReorthCtl* ctl = nullptr, int* kdev = nullptr);
 void gpu_delay(long long cycles, cudaStream_t);
 void gpu_empty(cudaStream_t);
 // out = in * f with f = denom (invert 0), 1 / denom (1) or 1 / sqrt(denom) (2);
@@ -225,22 +228,15 @@ template <typename T> void axpby(T* y, const T* x, double a, double b, i64 n, cu
 template <typename T> void wall_rhs(const Dims&, const Walls&, double eta, T* bv, cudaStream_t);
 void project_mean(double* x, i64 n, double* part, int nparts, cudaStream_t);
 
-// FGMRES restart cycle as a graph (k_krylov.cu).  The IF conditions of a
-// cycle's iterations: iteration j's Givens update sets the condition of
-// iteration j + 1; the cycle start resets them all (condition 0 to 1, the
-// rest to 0), since a cycle that runs again inside a WHILE body keeps the
-// values of its previous pass.
-constexpr int kMaxRestart = 64;
-struct IterConds {
-  cudaGraphConditionalHandle h[kMaxRestart];
-  int n;
-};
+// FGMRES restart cycle as a graph (k_krylov.cu): the cycle start sets the
+// condition of the iteration loop, each iteration's Givens update whether
+// another one runs.
 template <typename T> void fg_start(T* V0, const T* w, i64 n, double* gvec, int m, int* ist, const double* dpar,
-                                    cudaStream_t, float* V0_32 = nullptr, const IterConds* conds = nullptr);
+                                    cudaStream_t, float* V0_32, cudaGraphConditionalHandle loop);
 template <typename T>
-void scale_givens(T* out, const T* in, i64 n, float* out32, double* H, int ldh, double* cs, double* sn, double* g,
-                  int j, const double* hcol, const double* hcol2, const double* nrm2, double* res_out, int* ist,
-                  const double* dpar, cudaStream_t s, const cudaGraphConditionalHandle* next = nullptr);
+void scale_givens(T* V, T* Z, i64 ld, const T* in, const T* z, i64 n, float* out32, double* H, int m, double* cs,
+                  double* sn, double* g, const double* hcol, const double* hcol2, const double* nrm2, double* res_out,
+                  int* ist, const double* dpar, cudaGraphConditionalHandle loop, cudaStream_t s);
 void tri_solve_dev(const double* H, int ldh, const double* g, const int* ist, double* y, cudaStream_t);
 // control of device-driven solves (k_krylov.cu)
 void solve_init(double* dpar, int* ist, double rtol, int maxit, const double* rtol_p, const int* maxit_p,

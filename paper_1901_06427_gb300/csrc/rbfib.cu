@@ -104,12 +104,18 @@ struct KrylovStore {
   int m = 0;
   i64 n = 0;
   DBuf<T> V, Z, w;
+  // captured iterations: FP32 copy of the newest basis vector and the
+  // preconditioned vector
+  DBuf<float> v32;
+  DBuf<T> z;
   void build(int m_, i64 n_) {
     // columns start on 32-byte boundaries (16-byte vector loads in FP64 and FP32)
     m = m_; n = (n_ + 3) & ~(i64)3;
     V.alloc((size_t)(m + 1) * n);
     Z.alloc((size_t)m * n);
     w.alloc(n);
+    v32.alloc(n);
+    z.alloc(n);
   }
 };
 
@@ -717,40 +723,45 @@ void cond_node(rbfib_grid* g, cudaGraphConditionalHandle h, cudaGraphConditional
   --g->cap_depth;
 }
 
-// Iteration j of a captured restart cycle (the body of its IF node).  The
+// One iteration of a captured restart cycle (the body of its loop).  The
+// column j = ist[0] is read on the device: the preconditioner takes its input
+// from a fixed FP32 copy of the newest basis vector and leaves its result in
+// a fixed vector, and only the sweeps and the last launch look j up.  The
 // second Gram-Schmidt pass sits in a nested IF node whose condition the
 // first pass's multi-axpy sets (ReorthCtl).
 template <typename T>
-void capture_iteration(rbfib_grid* g, int j, bool wb, const cudaGraphConditionalHandle* next) {
+void capture_iteration(rbfib_grid* g, bool wb, cudaGraphConditionalHandle loop) {
   KrylovStore<T>& K = kr_of<T>(g);
   const int m = K.m;
   const i64 n = wb ? g->n_total() : g->nfl, ld = K.n, nfl = g->nfl;
   const double wf = g->dV;
   SmallPtrs sp = small_ptrs(g, m);
   T* V = K.V;
-  T* Z = K.Z;
   T* w = K.w;
-  precond_any(g, V + (i64)j * ld, Z + (i64)j * ld, wb, true);
-  apply_A<T>(g, Z + (i64)j * ld, w, wb);
+  int* kdev = g->gst;
+  if constexpr (sizeof(T) == 8) precond<float>(g, K.v32, g->f32b, wb, K.z, g->kappa);
+  else precond<float>(g, K.v32, K.z, wb, nullptr, g->kappa);
+  apply_A<T>(g, K.z, w, wb);
   const cudaGraphConditionalHandle h2 = new_handle(g, 0u);
   const ReorthCtl rc{g->gst.p + 4, sp.hcol2, reorth_tau2(sizeof(T) == 8), h2, 1};
-  multi_dot<T>(w, V, ld, j + 1, n, nfl, wf, g->part, g->nparts, sp.hcol, g->s);
-  multi_axpy<T>(w, V, ld, j + 1, sp.hcol, -1.0, n, nfl, wf, g->part, g->nparts, sp.nrm2, g->s, &rc);
+  multi_dot<T>(w, V, ld, m, n, nfl, wf, g->part, g->nparts, sp.hcol, g->s, kdev);
+  multi_axpy<T>(w, V, ld, m, sp.hcol, -1.0, n, nfl, wf, g->part, g->nparts, sp.nrm2, g->s, &rc, kdev);
   cond_node(g, h2, cudaGraphCondTypeIf, 1, [&](int) {
-    multi_dot<T>(w, V, ld, j + 1, n, nfl, wf, g->part, g->nparts, sp.hcol2, g->s);
-    multi_axpy<T>(w, V, ld, j + 1, sp.hcol2, -1.0, n, nfl, wf, g->part, g->nparts, sp.nrm2, g->s);
+    multi_dot<T>(w, V, ld, m, n, nfl, wf, g->part, g->nparts, sp.hcol2, g->s, kdev);
+    multi_axpy<T>(w, V, ld, m, sp.hcol2, -1.0, n, nfl, wf, g->part, g->nparts, sp.nrm2, g->s, nullptr, kdev);
   });
-  scale_givens<T>(V + (i64)(j + 1) * ld, w, n, basis32<T>(g), sp.H, m + 1, sp.cs, sp.sn, sp.gv, j, sp.hcol,
-                  sp.hcol2, sp.nrm2, sp.res, g->gst, g->dpar, g->s, next);
+  scale_givens<T>(V, K.Z, ld, w, K.z, n, K.v32, sp.H, m, sp.cs, sp.sn, sp.gv, sp.hcol, sp.hcol2, sp.nrm2, sp.res, g->gst,
+                  g->dpar, loop, g->s);
 }
 
-// One restart cycle of FGMRES(m), captured on g->s: the cycle start, then m
-// Arnoldi iterations, iteration j inside an IF node whose condition
-// iteration j-1's Givens update sets from its continue decision (the
-// handles default to 0 at every launch, so an iteration runs only if the one
-// before it ran and chose to continue), then the solution update and the
-// true residual w = b - A x with its norm in dpar[2].  per_iter (if not null) receives the launches of one iteration
-// with its gated second pass (two launches).
+// One restart cycle of FGMRES(m), captured on g->s: the cycle start, the
+// Arnoldi iterations in a WHILE node whose condition each iteration's Givens
+// update sets (converged, budget, m columns), then the solution update and the
+// true residual w = b - A x with its norm in dpar[2].  The loop holds one
+// iteration's nodes where a chain of m IF nodes held m: skipped nodes cost
+// 1.5-2 us each, and capture and instantiation m times as many.  per_iter (if
+// not null) receives the launches of one iteration with its gated second pass
+// (two launches).
 template <typename T>
 void capture_cycle(rbfib_grid* g, const T* b, T* x, bool wb, long long* per_iter) {
   KrylovStore<T>& K = kr_of<T>(g);
@@ -758,17 +769,11 @@ void capture_cycle(rbfib_grid* g, const T* b, T* x, bool wb, long long* per_iter
   const i64 n = wb ? g->n_total() : g->nfl, ld = K.n, nfl = g->nfl;
   const double wf = g->dV;
   SmallPtrs sp = small_ptrs(g, m);
-  IterConds conds{};
-  conds.n = m;
-  for (int j = 0; j < m; ++j) conds.h[j] = new_handle(g, j == 0 ? 1u : 0u);
-  const cudaGraphConditionalHandle* hs = conds.h;
-  fg_start<T>(K.V, K.w, n, sp.gv, m, g->gst, g->dpar, g->s, basis32<T>(g), &conds);
-  for (int j = 0; j < m; ++j) {
-    const long long a0 = rbfib::g_launches.load();
-    cond_node(g, hs[j], cudaGraphCondTypeIf, 1,
-              [&](int) { capture_iteration<T>(g, j, wb, j + 1 < m ? &hs[j + 1] : nullptr); });
-    if (j == 0 && per_iter) *per_iter = (long long)rbfib::g_launches.load() - a0;
-  }
+  const cudaGraphConditionalHandle loop = new_handle(g, 1u);
+  fg_start<T>(K.V, K.w, n, sp.gv, m, g->gst, g->dpar, g->s, K.v32, loop);
+  const long long a0 = rbfib::g_launches.load();
+  cond_node(g, loop, cudaGraphCondTypeWhile, 1, [&](int) { capture_iteration<T>(g, wb, loop); });
+  if (per_iter) *per_iter = (long long)rbfib::g_launches.load() - a0;
   tri_solve_dev(sp.H, m + 1, sp.gv, g->gst, sp.y, g->s);
   multi_axpy_dev<T>(x, K.Z, ld, g->gst, sp.y, 1.0, n, g->nparts, g->s);
   apply_A<T>(g, x, K.w, wb);
@@ -780,7 +785,6 @@ void capture_cycle(rbfib_grid* g, const T* b, T* x, bool wb, long long* per_iter
 // one per restart and read three numbers).
 template <typename T>
 bool build_cycle_graph(rbfib_grid* g, const T* b, T* x, bool wb, rbfib_grid::CycleGraph& G) {
-  const int m = kr_of<T>(g).m;
   const i64 n = wb ? g->n_total() : g->nfl;
   cudaStream_t s0 = g->s, sc = nullptr;
   const int saved_timer = g->timer_kind;
@@ -816,7 +820,7 @@ bool build_cycle_graph(rbfib_grid* g, const T* b, T* x, bool wb, rbfib_grid::Cyc
   rbfib::g_launches.fetch_sub((unsigned long long)captured);   // captured, not launched
   // an iteration's launches, counting its gated second pass (two launches)
   G.per_iter = per_iter;
-  G.fixed = captured - (long long)m * G.per_iter;
+  G.fixed = captured - G.per_iter;
   G.b = b; G.x = x; G.n = n;
   return ok;
 }
@@ -1700,9 +1704,8 @@ int solve_system(rbfib_grid* g, const double* b, double* x, bool with_bodies, rb
                                &per_iter);
     else
       body = refine_dev(g, b, x, with_bodies, di, dr, &per_iter);
-    // one pass of the WHILE body: its fixed part plus m iterations
-    const int m = g->desc.precision == RBFIB_FP64 ? kr_of<double>(g).m : kr_of<float>(g).m;
-    g->cap_body_fixed[which] = body - (long long)m * per_iter;
+    // one pass of the WHILE body: its fixed part plus one captured iteration
+    g->cap_body_fixed[which] = body - per_iter;
     g->cap_per_iter[which] = per_iter;
     g->cap_bodies += body;
     project_mean(x + g->nf, g->nc, g->part, g->nparts, g->s);
