@@ -68,7 +68,7 @@ def parse():
     ap.add_argument("--msd-blobs", type=int, nargs="+", default=[12, 42], choices=[12, 42, 162])
     ap.add_argument("--monolayer-step", action="store_true",
                     help="run one FP32-refined SEM step of the driven monolayer and exit (a profiling case for "
-                         "the multigrid, per-shape body block and cluster coarse-solve kernels)")
+                         "the long-line level solves and the per-shape body block)")
     ap.add_argument("--boomerang", action="store_true",
                     help="run only the boomerang equilibrium experiment of App. A")
     ap.add_argument("--boomerang-replicas", type=int, default=64)
@@ -108,8 +108,8 @@ def workload_config(w):
             "kernel": "3-point Peskin", "dt": w.dt, "kT": w.kT, "rtol": 1e-8, "precision": "fp64",
             "krylov": "FGMRES(48), classical Gram-Schmidt with selective re-orthogonalisation; "
                       "preconditioner: projection with exact fast-diagonalisation solves of the finest "
-                      "level (multigrid V(2,2) cycles on grids above 48 points per axis), coupled RPY body "
-                      "block",
+                      "level (multigrid V(2,2) cycles above it on the largest grids), coupled body block of the "
+                      "kernel's blob mobility",
             "l2": "flushed (512 MiB write) between timed steps", "data": "synthetic, seeded"}
 
 

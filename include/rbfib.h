@@ -365,10 +365,9 @@ uint64_t rbfib_launch_count(void);
 /* Kernel timer for roofline reports.  which: 0 off, 1 saddle matvec (Stokes
  * stencil + body rows), 2 finest-level velocity smoothing half sweep, 3
  * Krylov multi-column inner product, 4 Krylov multi-axpy, 5 exact solve of
- * the coarse multigrid level by fast diagonalisation (one 8-CTA cluster per
- * grid).  While a class is selected, the stream first idles for about 25 us
- * before each of its launches (so that the host has queued the launch and its
- * closing event), CUDA events are recorded on the grid's stream around each
+ * a multigrid level by fast diagonalisation.  While a class is selected, the
+ * stream first idles for about 25 us before each of its launches (so that the
+ * host has queued the launch and its closing event), CUDA events are recorded on the grid's stream around each
  * launch, and the algorithmic bytes and floating-point operations of each
  * launch are added up:
  *   matvec: 2 n s + 24 N_bl + 56 N_b bytes; 10 N_f + 6 N_c + 400 N_bl operations
