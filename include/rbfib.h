@@ -130,7 +130,9 @@ const char* rbfib_last_error(const rbfib_grid* g);   /* g may be NULL */
  * r_i = q_p + R(quat_p) ref_i.  Builds the blob-to-cell binning and the
  * body-block preconditioner.  Synchronises the stream.  EINVAL: a body with
  * no blob, or whose blobs lie on one line (its rotation about that line
- * would be undetermined: fewer than three non-collinear blobs). */
+ * would be undetermined: fewer than three non-collinear blobs).  Two blobs at
+ * one place, whose forces cannot be told apart: EINVAL, or EINTERNAL from the
+ * coupled body block. */
 int rbfib_set_bodies(rbfib_grid* g, int32_t n_bodies, const int32_t* blob_offsets,
                      const double* ref_blobs, const double* q, const double* quat);
 

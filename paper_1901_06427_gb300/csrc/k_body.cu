@@ -48,7 +48,9 @@ __global__ void k_mobility_full(int nbl, const double* __restrict__ r, PairMobil
 }
 
 // One step of a blocked Gauss-Jordan inversion (no pivoting; the matrices
-// are symmetric positive definite), out of place: with the kGJ pivots from
+// are symmetric positive definite, M by its pair functions, with FP32 pivots
+// above 4e-5 of the unit of M for 512 blobs in cubes, slabs and dense clusters
+// and K^T M^-1 K with it), out of place: with the kGJ pivots from
 // k0 (block row and column P), every 32 x 32 tile (I, J) of B is
 //   (P, P): D = A_PP^-1;  (P, J): D A_PJ;  (I, P): -A_IP D;
 //   (I, J): A_IJ - A_IP D A_PJ.

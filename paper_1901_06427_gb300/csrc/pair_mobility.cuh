@@ -6,15 +6,35 @@
 //
 // M_ij = (f(r) (I - n n^T) + g(r) n n^T) / (eta h), r = |r_i - r_j| / h.
 // f and g are the velocity across and along n that a unit force spread by the
-// kernel gives a blob at distance r on the MAC grid, averaged over the
-// blobs' positions relative to the grid and over directions (periodic box of
-// 96 or 128 cells, Hasimoto's correction for its images), at r = 0, 1/4 ..,
-// 6; from r = 4 they go over to the Rotne-Prager-Yamakawa tensor, which the
-// fluid's response meets to 0.2% there.  Near r = 0 they are flat, where the
-// tensor has a corner, so the smallest eigenvalues of M, which set the
-// solver's iterations, are up to 20 times smaller than the tensor's: solves
-// to 1e-8 of two 42-blob spheres take 20 iterations (27 with the tensor)
-// with the three-point kernel and 27 (84) with the six-point kernel.
+// kernel gives a blob at distance r on the unbounded MAC grid, averaged over
+// the blobs' positions relative to the grid and over directions.  With Phi(k)
+// the kernel's Fourier transform and K_a = 2 sin(k_a / 2) the average over
+// positions is the transform of the positive semidefinite
+//   S(k) = Phi(k)^2 (I - K K^T / |K|^2) / |K|^2
+// over all of R^3 (the cross terms of different aliases average out), and the
+// average over directions keeps only its parts across and along k, both >= 0:
+// so every set of distinct blobs has a positive definite M.  Sampled averages
+// do not: noise of 1e-6 (six-point) and a tail that sets in over r = 4 .. 6
+// made M indefinite for cubes, plates, rods and packed shells.
+// Beyond r = 6 f and g are the Rotne-Prager-Yamakawa tensor's of radius P.a.
+// Its 1 / r^3 part is larger than the average's, by the dipole tensor times d =
+// 0.0562 (six-point), 0.0276 (three-point); so d times the dipole tensor of the
+// density (1 - r^2 / 36)^3 (unit integral, r < 6), whose field beyond 6 is
+// the point dipole's, is taken off the average: the two meet at 6 without a
+// step, at most 0.8% (0.4%) below the average, and only ripples of that
+// density's transform at short waves are left below zero (pair_raise).
+// The six-point table then adds 1.5e-5 (1 - r/6)^4 (4 r/6 + 1) to f and g (also
+// positive definite): a closed shell's uniform normal force, against which
+// the enclosed fluid hardly yields, has mobility 2e-6 on average but several
+// times that and less as the shell sits on the grid, and FP32 sweeps stall
+// when M takes it that small (22 shells of 42 blobs refined to 1e-10: 528
+// iterations without, 192 with; the sampled averages 190).
+// Near r = 0 f and g are flat, where the Rotne-Prager-Yamakawa tensor has a
+// corner, so the smallest eigenvalues of M, which set the solver's
+// iterations, are up to 50 times smaller than the tensor's.  Both constrained
+// solves of a step of two 42-blob spheres together: three-point kernel to 1e-8
+// 38 iterations, six-point, refined to 1e-10, 104 (with the tensor, and without
+// the wall drag in the pressure block, 68 and 404).
 #pragma once
 #include <cmath>
 
@@ -41,19 +61,23 @@ inline void pair_tail(double a, double r, double& f, double& g) {
 // r = 6.
 inline PairMobility pair_mobility(int kw) {
   static const double three[2][kPairKnots] = {
-    {0.0584973, 0.0572061, 0.0535623, 0.0481889, 0.0420517, 0.0359540, 0.0304755, 0.0259027, 0.0222550,
-     0.0194052, 0.0171763, 0.0154186, 0.0139978, 0.0128210, 0.0118300, 0.0109864, 0.0102584, 0.0096237,
-     0.0090650, 0.0085699, 0.0081268, 0.0077273, 0.0073650, 0.0070350, 0.0067332},
-    {0.0584973, 0.0578241, 0.0559409, 0.0530778, 0.0495507, 0.0456879, 0.0418248, 0.0381751, 0.0348471,
-     0.0318880, 0.0292932, 0.0270277, 0.0250510, 0.0233242, 0.0218065, 0.0204639, 0.0192695, 0.0182014,
-     0.0172394, 0.0163697, 0.0155805, 0.0148632, 0.0142086, 0.0136095, 0.0130595}};
+    {0.058383518, 0.057064867, 0.053407145, 0.048098018, 0.041981828, 0.035881263, 0.030397332, 0.025812839,
+     0.022161247, 0.019321799, 0.017112281, 0.015364997, 0.013952640, 0.012786548, 0.011806782, 0.010971495,
+     0.010250170, 0.009620144, 0.009064496, 0.008570304, 0.008127448, 0.007727941, 0.007365507, 0.007035210,
+     0.006733151},
+    {0.058383518, 0.057710540, 0.055814263, 0.052950333, 0.049426834, 0.045585682, 0.041733503, 0.038081219,
+     0.034752018, 0.031795009, 0.029204034, 0.026945855, 0.024977816, 0.023256849, 0.021744350, 0.020407711,
+     0.019219880, 0.018158527, 0.017205261, 0.016344867, 0.015564698, 0.014854215, 0.014204612, 0.013608474,
+     0.013059525}};
   static const double six[2][kPairKnots] = {
-    {0.0361263, 0.0358104, 0.0348888, 0.0334334, 0.0315512, 0.0293718, 0.0270319, 0.0246577, 0.0223541,
-     0.0201998, 0.0182437, 0.0165076, 0.0149924, 0.0136848, 0.0125624, 0.0115992, 0.0107697, 0.0100535,
-     0.0094310, 0.0088844, 0.0083996, 0.0079659, 0.0075750, 0.0072204, 0.0068968},
-    {0.0361263, 0.0359677, 0.0355013, 0.0347511, 0.0337551, 0.0325604, 0.0312193, 0.0297842, 0.0283041,
-     0.0268214, 0.0253708, 0.0239778, 0.0226593, 0.0214250, 0.0202787, 0.0192201, 0.0182456, 0.0173446,
-     0.0165107, 0.0157422, 0.0150354, 0.0143857, 0.0137884, 0.0132387, 0.0127322}};
+    {0.035868804, 0.035554658, 0.034637362, 0.033188571, 0.031316283, 0.029150271, 0.026825876, 0.024469031,
+     0.022184819, 0.020050849, 0.018115583, 0.016400845, 0.014907102, 0.013619957, 0.012516480, 0.011570452,
+     0.010756071, 0.010050131, 0.009432959, 0.008888509, 0.008404016, 0.007969476, 0.007577136, 0.007221065,
+     0.006896825},
+    {0.035868804, 0.035711162, 0.035246743, 0.034500010, 0.033508720, 0.032320066, 0.030986148, 0.029559454,
+     0.028088919, 0.026616988, 0.025177854, 0.023796872, 0.022490945, 0.021269600, 0.020136448, 0.019090725,
+     0.018128725, 0.017244997, 0.016433239, 0.015686939, 0.014999766, 0.014365806, 0.013779673, 0.013236548,
+     0.012732174}};
   PairMobility P;
   P.a = kw == 6 ? 1.47 : 0.91;
   P.shift = kw == 6 ? 3e-5 : 2e-4;
@@ -103,12 +127,15 @@ __host__ __device__ inline void pair_functions(const PairMobility& P, double r, 
   }
 }
 
-// The averages are positive definite only to their statistical error
-// (three-point: the grid's own variation), which adds up over blobs that the
-// grid does not resolve.  A blob with more than 32 others (itself included)
-// within 2 h is raised by that much more: shells of 42 to 800 blobs of radius
-// 0.3 to 3 h have smallest eigenvalues down to -7e-4 (500 blobs, radius h / 2)
-// before and above zero after it; ordinary shells have about ten.
+// What the diagonal is raised by.  The smallest eigenvalues are those of
+// motions that the kernel averages away, next to zero; splines, the step of
+// the digits and the correction above move them by less than 8e-6 (cubes of
+// up to 11^3 blobs at 0.9 to 1.5 h, plates, slabs, rods, 1200 blobs at random in
+// boxes of 6 to 20 h, packed shells), a quarter of the shift.  A blob with more
+// than 32 others (itself included) within 2 h is raised by that much more:
+// such a cluster's largest eigenvalue grows with its blobs, and with it the
+// rounding of the FP32 inverse (512 blobs at random within h / 20: largest
+// eigenvalue 30, smallest pivot 3e-3; 4.8e-4 with the six-point kernel).
 constexpr double kPairNear = 2.0;
 __host__ __device__ inline double pair_raise(const PairMobility& P, int near) {
   return P.shift * (near > 32 ? near / 32.0 : 1.0);

@@ -982,8 +982,10 @@ bool spd_inverse(std::vector<double>& A, int n) {
   return true;
 }
 
-// free-space mobility of blobs x (n x 3) (pair_mobility.cuh)
-void pair_matrix(const double* x, int nbp, const PairMobility& P, double h, double eta, std::vector<double>& M) {
+// free-space mobility of blobs x (n x 3) (pair_mobility.cuh), its diagonal
+// raised up times as much; false if two blobs share one place
+bool pair_matrix(const double* x, int nbp, const PairMobility& P, double h, double eta, double up,
+                 std::vector<double>& M) {
   const int n3 = 3 * nbp;
   M.assign((size_t)n3 * n3, 0.0);
   for (int i = 0; i < nbp; ++i) {
@@ -996,11 +998,25 @@ void pair_matrix(const double* x, int nbp, const PairMobility& P, double h, doub
           continue;
         }
         double B[9];
-        pair_block(P, d, i == j ? pair_raise(P, near) : 0.0, B);
+        pair_block(P, d, i == j ? up * pair_raise(P, near) : 0.0, B);
+        if (std::isnan(B[0])) return false;
         for (int p = 0; p < 3; ++p)
           for (int q = 0; q < 3; ++q) M[(size_t)(3 * i + p) * n3 + 3 * j + q] = B[3 * p + q] / (eta * h);
       }
   }
+  return true;
+}
+
+// Its inverse.  The pair functions are positive definite, so the diagonal as
+// it stands suffices for every body tried (pair_raise); should rounding leave
+// one that it does not, the diagonal grows until there is a factor, since this
+// matrix only preconditions: distinct blobs are never refused.
+bool pair_inverse(const double* x, int nbp, const PairMobility& P, double h, double eta, std::vector<double>& M) {
+  for (double up = 1.0; up < 1e8; up *= 4.0) {
+    if (!pair_matrix(x, nbp, P, h, eta, up, M)) return false;
+    if (spd_inverse(M, 3 * nbp)) return true;
+  }
+  return false;
 }
 
 bool inverse6(double A[36]) {
@@ -1528,8 +1544,8 @@ int rbfib_set_bodies(rbfib_grid* g, int32_t n_bodies, const int32_t* blob_offset
       const int n = off[p + 1] - off[p], n3 = 3 * n, ld = body_ld(n3 + 6);
       const double* x = href.data() + 3 * (size_t)off[p];
       std::vector<double> M;
-      pair_matrix(x, n, g->pair, g->desc.h, g->desc.eta, M);
-      if (!spd_inverse(M, n3)) return fail(g, RBFIB_EINVAL, "set_bodies: blob mobility of a shape is singular");
+      if (!pair_inverse(x, n, g->pair, g->desc.h, g->desc.eta, M))
+        return fail(g, RBFIB_EINVAL, "set_bodies: blob mobility of a shape is singular");
       std::vector<double> K((size_t)n3 * 6, 0.0), P((size_t)n3 * 6, 0.0), E((size_t)n3 * 6, 0.0);
       for (int i = 0; i < n; ++i) {
         const double* r = x + 3 * i;
