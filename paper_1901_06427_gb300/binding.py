@@ -210,12 +210,14 @@ class Grid:
         q = torch.as_tensor(np.asarray(q) if not isinstance(q, torch.Tensor) else q, dtype=torch.float64, device=dev).contiguous()
         quat = torch.as_tensor(np.asarray(quat) if not isinstance(quat, torch.Tensor) else quat, dtype=torch.float64, device=dev).contiguous()
         torch.cuda.current_stream().synchronize()   # the library may copy on another stream
-        self._check(lib().rbfib_set_bodies(
+        st = lib().rbfib_set_bodies(
             self._h, nb, off.ctypes.data_as(ctypes.POINTER(ctypes.c_int32)),
             _ptr(ref, numel=3 * nbl, name="ref_blobs") if nbl else None,
             _ptr(q, numel=3 * nb, name="q") if nb else None,
-            _ptr(quat, numel=4 * nb, name="quat") if nb else None))
-        self.n_bodies, self.n_blobs = nb, nbl
+            _ptr(quat, numel=4 * nb, name="quat") if nb else None)
+        lay = self.layout()   # the grid's bodies, also after a refusal
+        self.n_bodies, self.n_blobs = (lay[6] - lay[5]) // 6, (lay[5] - lay[4]) // 3
+        self._check(st)
 
     def layout(self):
         off = (ctypes.c_int64 * 7)()

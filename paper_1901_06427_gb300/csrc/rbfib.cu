@@ -110,12 +110,15 @@ struct KrylovStore {
   DBuf<T> z;
   void build(int m_, i64 n_) {
     // columns start on 32-byte boundaries (16-byte vector loads in FP64 and FP32)
-    m = m_; n = (n_ + 3) & ~(i64)3;
-    V.alloc((size_t)(m + 1) * n);
-    Z.alloc((size_t)m * n);
-    w.alloc(n);
-    v32.alloc(n);
-    z.alloc(n);
+    const i64 ld = (n_ + 3) & ~(i64)3;
+    n = 0;   // until all of it is there
+    m = m_;
+    V.alloc((size_t)(m + 1) * ld);
+    Z.alloc((size_t)m * ld);
+    w.alloc(ld);
+    v32.alloc(ld);
+    z.alloc(ld);
+    n = ld;
   }
 };
 
@@ -1129,6 +1132,67 @@ void alloc_solver(rbfib_grid* g) {
   g->bvec.ensure(n); g->xvec.ensure(n); g->xrfd.ensure(n);
 }
 
+// Appends the body-block matrix of a shape of n blobs x (body frame; k_body.cu)
+// to sB.  Returns why there is none, or null.
+const char* shape_matrix(const rbfib_grid* g, const double* x, int n, std::vector<float>& sB) {
+  const int n3 = 3 * n, ld = body_ld(n3 + 6);
+  std::vector<double> M;
+  if (!pair_inverse(x, n, g->pair, g->desc.h, g->desc.eta, M)) return "blob mobility of a shape is singular";
+  std::vector<double> K((size_t)n3 * 6, 0.0), P((size_t)n3 * 6, 0.0), E((size_t)n3 * 6, 0.0);
+  for (int i = 0; i < n; ++i) {
+    const double* r = x + 3 * i;
+    for (int a = 0; a < 3; ++a) K[(size_t)(3 * i + a) * 6 + a] = 1.0;
+    // w x r = -[r]_x w
+    K[(size_t)(3 * i + 0) * 6 + 4] = r[2];  K[(size_t)(3 * i + 0) * 6 + 5] = -r[1];
+    K[(size_t)(3 * i + 1) * 6 + 3] = -r[2]; K[(size_t)(3 * i + 1) * 6 + 5] = r[0];
+    K[(size_t)(3 * i + 2) * 6 + 3] = r[1];  K[(size_t)(3 * i + 2) * 6 + 4] = -r[0];
+  }
+  double N[36] = {0};
+  for (int r = 0; r < n3; ++r)
+    for (int k = 0; k < n3; ++k)
+      for (int c = 0; c < 6; ++c) P[(size_t)r * 6 + c] += M[(size_t)r * n3 + k] * K[(size_t)k * 6 + c];
+  for (int k = 0; k < n3; ++k)
+    for (int r = 0; r < 6; ++r)
+      for (int c = 0; c < 6; ++c) N[6 * r + c] += K[(size_t)k * 6 + r] * P[(size_t)k * 6 + c];
+  if (!inverse6(N)) return "body resistance is singular";
+  for (int r = 0; r < n3; ++r)
+    for (int c = 0; c < 6; ++c)
+      for (int k = 0; k < 6; ++k) E[(size_t)r * 6 + c] += P[(size_t)r * 6 + k] * N[6 * k + c];
+  for (int r = 0; r < n3 + 6; ++r)
+    for (int c = 0; c < ld; ++c) {
+      double v = 0.0;
+      if (c < n3 + 6) {
+        if (r < n3 && c < n3) {
+          v = -M[(size_t)r * n3 + c];
+          for (int k = 0; k < 6; ++k) v += E[(size_t)r * 6 + k] * P[(size_t)c * 6 + k];
+        } else if (r < n3) v = E[(size_t)r * 6 + c - n3];
+        else if (c < n3) v = E[(size_t)c * 6 + r - n3];
+        else v = N[6 * (r - n3) + c - n3];
+      }
+      sB.push_back((float)v);
+    }
+  return nullptr;
+}
+
+// The grid as it is without bodies, after a failure while they were being
+// replaced: no entry point may go on with sizes whose buffers are not there.
+void forget_bodies(rbfib_grid* g) {
+  g->nb = g->nbl = g->max_blobs = 0;
+  g->h_boff.assign(1, 0);
+  g->dense_body = g->dM_valid = g->dquat_valid = false;
+  try {
+    alloc_solver(g);
+  } catch (CudaError&) {   // no memory for the fluid alone: need_solver reports it
+  }
+}
+
+// Every entry point that solves or preconditions asks for its vectors first.
+void need_solver(rbfib_grid* g) {
+  const i64 n = g->n_total(), k = g->desc.precision == RBFIB_FP64 ? g->kr64.n : g->kr32.n;
+  if (k < n || (i64)std::min({g->f32a.n, g->f32b.n, g->bvec.n, g->xvec.n, g->xrfd.n}) < n)
+    throw CudaError{cudaErrorMemoryAllocation};
+}
+
 // ---------------------------------------------------------------- autotuner
 // For each tunable kernel and grid shape, time every candidate block size
 // (CUDA events on the grid's stream, best of a few launches) and keep the
@@ -1430,46 +1494,91 @@ int rbfib_set_bodies(rbfib_grid* g, int32_t n_bodies, const int32_t* blob_offset
                      const double* q, const double* quat) {
   if (!g || n_bodies < 0 || (n_bodies > 0 && (!blob_offsets || !ref_blobs || !q || !quat)))
     return fail(g, RBFIB_EINVAL, "set_bodies: bad arguments");
-  std::vector<int> off(n_bodies + 1, 0);
-  if (n_bodies > 0) {
-    std::memcpy(off.data(), blob_offsets, sizeof(int) * (n_bodies + 1));
-    if (off[0] != 0) return fail(g, RBFIB_EINVAL, "set_bodies: blob_offsets[0] must be 0");
-    for (int p = 0; p < n_bodies; ++p)
-      if (off[p + 1] <= off[p]) return fail(g, RBFIB_EINVAL, "set_bodies: every body needs at least one blob");
-  }
-  if (n_bodies > 0) {
-    // a rigid body needs three blobs off one line: with collinear blobs the
-    // rotation about their line is undetermined and the system is singular
-    std::vector<double> ref(3 * (size_t)off[n_bodies]);
-    if (cudaStreamSynchronize(g->s) != cudaSuccess ||
-        cudaMemcpy(ref.data(), ref_blobs, sizeof(double) * ref.size(), cudaMemcpyDeviceToHost) != cudaSuccess)
-      return fail(g, RBFIB_ECUDA, "set_bodies: cannot read ref_blobs");
-    for (int p = 0; p < n_bodies; ++p) {
-      const double* r0 = &ref[3 * (size_t)off[p]];
-      double u[3] = {0, 0, 0}, un = 0.0;
-      for (int i = off[p] + 1; i < off[p + 1]; ++i) {
-        const double* r = &ref[3 * (size_t)i];
-        const double d2 = (r[0] - r0[0]) * (r[0] - r0[0]) + (r[1] - r0[1]) * (r[1] - r0[1]) +
-                          (r[2] - r0[2]) * (r[2] - r0[2]);
-        if (d2 > un) { un = d2; for (int a = 0; a < 3; ++a) u[a] = r[a] - r0[a]; }
-      }
-      double worst = 0.0;
-      for (int i = off[p] + 1; i < off[p + 1] && un > 0.0; ++i) {
-        const double* r = &ref[3 * (size_t)i];
-        const double dv[3] = {r[0] - r0[0], r[1] - r0[1], r[2] - r0[2]};
-        const double cx = dv[1] * u[2] - dv[2] * u[1], cy = dv[2] * u[0] - dv[0] * u[2], cz = dv[0] * u[1] - dv[1] * u[0];
-        worst = std::max(worst, std::sqrt(cx * cx + cy * cy + cz * cz) / un);
-      }
-      if (!(worst > 1e-9)) return fail(g, RBFIB_EINVAL, "set_bodies: a body's blobs lie on one line");
-    }
-  }
+  bool replaced = false;   // whether the grid's previous bodies are gone
   try {
+    std::vector<int> off(n_bodies + 1, 0);
+    if (n_bodies > 0) {
+      std::memcpy(off.data(), blob_offsets, sizeof(int) * (n_bodies + 1));
+      if (off[0] != 0) return fail(g, RBFIB_EINVAL, "set_bodies: blob_offsets[0] must be 0");
+      for (int p = 0; p < n_bodies; ++p)
+        if (off[p + 1] <= off[p]) return fail(g, RBFIB_EINVAL, "set_bodies: every body needs at least one blob");
+    }
+    // all that can be refused is looked at before any state of the grid changes
+    const int nb = n_bodies, nbl = off[n_bodies];
+    std::vector<double> ref(3 * (size_t)nbl);
+    if (nb > 0) {
+      if (cudaStreamSynchronize(g->s) != cudaSuccess ||
+          cudaMemcpy(ref.data(), ref_blobs, sizeof(double) * ref.size(), cudaMemcpyDeviceToHost) != cudaSuccess)
+        return fail(g, RBFIB_ECUDA, "set_bodies: cannot read ref_blobs");
+      // a rigid body needs three blobs off one line: with collinear blobs the
+      // rotation about their line is undetermined and the system is singular
+      for (int p = 0; p < nb; ++p) {
+        const double* r0 = &ref[3 * (size_t)off[p]];
+        double u[3] = {0, 0, 0}, un = 0.0;
+        for (int i = off[p] + 1; i < off[p + 1]; ++i) {
+          const double* r = &ref[3 * (size_t)i];
+          const double d2 = (r[0] - r0[0]) * (r[0] - r0[0]) + (r[1] - r0[1]) * (r[1] - r0[1]) +
+                            (r[2] - r0[2]) * (r[2] - r0[2]);
+          if (d2 > un) { un = d2; for (int a = 0; a < 3; ++a) u[a] = r[a] - r0[a]; }
+        }
+        double worst = 0.0;
+        for (int i = off[p] + 1; i < off[p + 1] && un > 0.0; ++i) {
+          const double* r = &ref[3 * (size_t)i];
+          const double dv[3] = {r[0] - r0[0], r[1] - r0[1], r[2] - r0[2]};
+          const double cx = dv[1] * u[2] - dv[2] * u[1], cy = dv[2] * u[0] - dv[0] * u[2], cz = dv[0] * u[1] - dv[1] * u[0];
+          worst = std::max(worst, std::sqrt(cx * cx + cy * cy + cz * cz) / un);
+        }
+        if (!(worst > 1e-9)) return fail(g, RBFIB_EINVAL, "set_bodies: a body's blobs lie on one line");
+      }
+    }
+    // body lengths and shape table
+    std::vector<double> Lp(std::max(nb, 1), 0.0);
+    std::vector<int> shape_of(std::max(nb, 1), 0), shape_rep;
+    int max_blobs = 0;
+    for (int p = 0; p < nb; ++p) {
+      const int n = off[p + 1] - off[p];
+      max_blobs = std::max(max_blobs, n);
+      const double* x = ref.data() + 3 * (size_t)off[p];
+      double mx = 0.0;
+      for (int i = 0; i < n; ++i)
+        for (int j = i + 1; j < n; ++j) {
+          double dd = 0.0;
+          for (int a = 0; a < 3; ++a) dd += (x[3 * i + a] - x[3 * j + a]) * (x[3 * i + a] - x[3 * j + a]);
+          mx = std::max(mx, std::sqrt(dd));
+        }
+      Lp[p] = mx;
+      int found = -1;
+      for (size_t s = 0; s < shape_rep.size(); ++s) {
+        const int q0 = shape_rep[s];
+        if (off[q0 + 1] - off[q0] == n &&
+            std::memcmp(ref.data() + 3 * (size_t)off[q0], x, sizeof(double) * 3 * n) == 0) { found = (int)s; break; }
+      }
+      if (found < 0) { found = (int)shape_rep.size(); shape_rep.push_back(p); }
+      shape_of[p] = found;
+    }
+    // coupled body block when every blob pair fits a small dense matrix, else
+    // per-shape body-block matrices in the body frame (k_body.cu)
+    const bool dense = nb >= 2 && 3 * nbl <= kDenseBodyMaxRows && 6 * nb <= kDenseBodyMaxBodyRows;
+    const int ns = (int)shape_rep.size();
+    std::vector<i64> soff(std::max(ns, 1), 0);
+    std::vector<float> sB;
+    for (int s = 0; s < ns && !dense; ++s) {
+      const int p = shape_rep[s];
+      soff[s] = (i64)sB.size();
+      if (const char* why = shape_matrix(g, ref.data() + 3 * (size_t)off[p], off[p + 1] - off[p], sB))
+        return fail(g, RBFIB_EINVAL, std::string("set_bodies: ") + why);
+    }
+
     ck(cudaStreamSynchronize(g->s));
     drop_graphs(g);
-    g->nb = n_bodies;
-    g->nbl = off[n_bodies];
+    replaced = true;
+    g->nb = nb;
+    g->nbl = nbl;
     g->h_boff = off;
-    const int nb = g->nb, nbl = g->nbl;
+    g->max_blobs = max_blobs;
+    g->dense_body = dense;
+    g->dM_valid = false;
+    g->dquat_valid = false;
     g->boff.alloc(nb + 1);
     ck(cudaMemcpyAsync(g->boff, off.data(), sizeof(int) * (nb + 1), cudaMemcpyHostToDevice, g->s));
     std::vector<int> bob(nbl);
@@ -1485,11 +1594,7 @@ int rbfib_set_bodies(rbfib_grid* g, int32_t n_bodies, const int32_t* blob_offset
       ck(cudaMemcpyAsync(g->cur.quat, quat, sizeof(double) * 4 * nb, cudaMemcpyDeviceToDevice, g->s));
     }
     g->bkey.alloc(std::max(nbl, 1));
-    // coupled body block when every blob pair fits a small dense matrix
-    g->dense_body = nb >= 2 && 3 * nbl <= kDenseBodyMaxRows && 6 * nb <= kDenseBodyMaxBodyRows;
-    g->dM_valid = false;
-    g->dquat_valid = false;
-    if (g->dense_body) {
+    if (dense) {
       g->dM.alloc((size_t)9 * nbl * nbl);
       g->dMw.alloc((size_t)9 * nbl * nbl);
       g->dTw.alloc((size_t)9 * nbl * nbl);
@@ -1503,84 +1608,8 @@ int rbfib_set_bodies(rbfib_grid* g, int32_t n_bodies, const int32_t* blob_offset
       g->dNw.alloc((size_t)72 * nb * nb);
       g->dstatus.alloc(1);
     }
-    refresh_config(g, g->cur, true);
-    // host copy of the reference blobs: body lengths and shape table
-    std::vector<double> href(3 * (size_t)nbl);
-    if (nbl) ck(cudaMemcpyAsync(href.data(), ref_blobs, sizeof(double) * 3 * nbl, cudaMemcpyDeviceToHost, g->s));
-    ck(cudaStreamSynchronize(g->s));
-    std::vector<double> Lp(std::max(nb, 1), 0.0);
-    std::vector<int> shape_of(std::max(nb, 1), 0), shape_rep;
-    g->max_blobs = 0;
-    for (int p = 0; p < nb; ++p) {
-      const int n = off[p + 1] - off[p];
-      g->max_blobs = std::max(g->max_blobs, n);
-      const double* x = href.data() + 3 * (size_t)off[p];
-      double mx = 0.0;
-      for (int i = 0; i < n; ++i)
-        for (int j = i + 1; j < n; ++j) {
-          double dd = 0.0;
-          for (int a = 0; a < 3; ++a) dd += (x[3 * i + a] - x[3 * j + a]) * (x[3 * i + a] - x[3 * j + a]);
-          mx = std::max(mx, std::sqrt(dd));
-        }
-      Lp[p] = mx;
-      int found = -1;
-      for (size_t s = 0; s < shape_rep.size(); ++s) {
-        const int q0 = shape_rep[s];
-        if (off[q0 + 1] - off[q0] == n &&
-            std::memcmp(href.data() + 3 * (size_t)off[q0], x, sizeof(double) * 3 * n) == 0) { found = (int)s; break; }
-      }
-      if (found < 0) { found = (int)shape_rep.size(); shape_rep.push_back(p); }
-      shape_of[p] = found;
-    }
     g->Lp.alloc(std::max(nb, 1));
     ck(cudaMemcpyAsync(g->Lp, Lp.data(), sizeof(double) * std::max(nb, 1), cudaMemcpyHostToDevice, g->s));
-    // per-shape body-block matrices in the body frame (k_body.cu), used where
-    // the coupled block is not
-    const int ns = (int)shape_rep.size();
-    std::vector<i64> soff(std::max(ns, 1), 0);
-    std::vector<float> sB;
-    for (int s = 0; s < ns && !g->dense_body; ++s) {
-      const int p = shape_rep[s];
-      const int n = off[p + 1] - off[p], n3 = 3 * n, ld = body_ld(n3 + 6);
-      const double* x = href.data() + 3 * (size_t)off[p];
-      std::vector<double> M;
-      if (!pair_inverse(x, n, g->pair, g->desc.h, g->desc.eta, M))
-        return fail(g, RBFIB_EINVAL, "set_bodies: blob mobility of a shape is singular");
-      std::vector<double> K((size_t)n3 * 6, 0.0), P((size_t)n3 * 6, 0.0), E((size_t)n3 * 6, 0.0);
-      for (int i = 0; i < n; ++i) {
-        const double* r = x + 3 * i;
-        for (int a = 0; a < 3; ++a) K[(size_t)(3 * i + a) * 6 + a] = 1.0;
-        // w x r = -[r]_x w
-        K[(size_t)(3 * i + 0) * 6 + 4] = r[2];  K[(size_t)(3 * i + 0) * 6 + 5] = -r[1];
-        K[(size_t)(3 * i + 1) * 6 + 3] = -r[2]; K[(size_t)(3 * i + 1) * 6 + 5] = r[0];
-        K[(size_t)(3 * i + 2) * 6 + 3] = r[1];  K[(size_t)(3 * i + 2) * 6 + 4] = -r[0];
-      }
-      double N[36] = {0};
-      for (int r = 0; r < n3; ++r)
-        for (int k = 0; k < n3; ++k)
-          for (int c = 0; c < 6; ++c) P[(size_t)r * 6 + c] += M[(size_t)r * n3 + k] * K[(size_t)k * 6 + c];
-      for (int k = 0; k < n3; ++k)
-        for (int r = 0; r < 6; ++r)
-          for (int c = 0; c < 6; ++c) N[6 * r + c] += K[(size_t)k * 6 + r] * P[(size_t)k * 6 + c];
-      if (!inverse6(N)) return fail(g, RBFIB_EINVAL, "set_bodies: body resistance is singular");
-      for (int r = 0; r < n3; ++r)
-        for (int c = 0; c < 6; ++c)
-          for (int k = 0; k < 6; ++k) E[(size_t)r * 6 + c] += P[(size_t)r * 6 + k] * N[6 * k + c];
-      soff[s] = (i64)sB.size();
-      for (int r = 0; r < n3 + 6; ++r)
-        for (int c = 0; c < ld; ++c) {
-          double v = 0.0;
-          if (c < n3 + 6) {
-            if (r < n3 && c < n3) {
-              v = -M[(size_t)r * n3 + c];
-              for (int k = 0; k < 6; ++k) v += E[(size_t)r * 6 + k] * P[(size_t)c * 6 + k];
-            } else if (r < n3) v = E[(size_t)r * 6 + c - n3];
-            else if (c < n3) v = E[(size_t)c * 6 + r - n3];
-            else v = N[6 * (r - n3) + c - n3];
-          }
-          sB.push_back((float)v);
-        }
-    }
     g->shape_of.alloc(std::max(nb, 1));
     ck(cudaMemcpyAsync(g->shape_of, shape_of.data(), sizeof(int) * std::max(nb, 1), cudaMemcpyHostToDevice, g->s));
     g->shape_off.alloc(std::max(ns, 1));
@@ -1594,10 +1623,15 @@ int rbfib_set_bodies(rbfib_grid* g, int32_t n_bodies, const int32_t* blob_offset
     for (DBuf<double>* b : {&g->bodyF, &g->bodyW, &g->bodyWn}) b->alloc(b6);
     g->blobS.alloc(l3);
     alloc_solver(g);
+    refresh_config(g, g->cur, true);
     ck(cudaStreamSynchronize(g->s));
     ck(cudaGetLastError());
   } catch (CudaError& e) {
+    if (replaced) forget_bodies(g);
     return fail(g, e.code, std::string("set_bodies: ") + e.what());
+  } catch (std::exception& e) {
+    if (replaced) forget_bodies(g);
+    return fail(g, RBFIB_EINTERNAL, std::string("set_bodies: ") + e.what());
   }
   return RBFIB_OK;
 }
@@ -1605,6 +1639,7 @@ int rbfib_set_bodies(rbfib_grid* g, int32_t n_bodies, const int32_t* blob_offset
 int rbfib_apply_preconditioner(rbfib_grid* g, const double* r, double* z) {
   if (!g || !r || !z) return fail(g, RBFIB_EINVAL, "apply_preconditioner: null argument");
   try {
+    need_solver(g);
     convert<double, float>(r, g->f32a, g->n_total(), g->s);
     precond<float>(g, g->f32a, g->f32b, true, z, 0.0);
     ck(cudaGetLastError());
@@ -1639,6 +1674,7 @@ bool use_graph_path(rbfib_grid* g) { return g->use_graphs && g->timer_kind == 0;
 // -slip + J wall part, forces.  b is FP64 in the saddle layout.
 void build_rhs(rbfib_grid* g, const double* FT, const double* slip, const double* fluid, bool walls, double* b) {
   const i64 n = g->n_total();
+  need_solver(g);
   ck(cudaMemsetAsync(b, 0, sizeof(double) * n, g->s));
   if (fluid) ck(cudaMemcpyAsync(b, fluid, sizeof(double) * g->nf, cudaMemcpyDeviceToDevice, g->s));
   if (walls && g->walls_move) wall_rhs<double>(g->d, g->walls, g->desc.eta, b, g->s);
@@ -1811,6 +1847,7 @@ int rbfib_mobility_solve(rbfib_grid* g, const double* FT, const double* slip, co
 int rbfib_stokes_solve(rbfib_grid* g, const double* f, double* v, double* pi, rbfib_solve_info* info) {
   if (!g || !f || !v) return fail(g, RBFIB_EINVAL, "stokes_solve: null argument");
   try {
+    need_solver(g);
     ck(cudaMemsetAsync(g->bvec, 0, sizeof(double) * g->nfl, g->s));
     ck(cudaMemcpyAsync(g->bvec, f, sizeof(double) * g->nf, cudaMemcpyDeviceToDevice, g->s));
     int st = solve_system(g, g->bvec, g->xvec, false, info);
