@@ -446,9 +446,12 @@ cudaError_t dense_body_build(int nbl, int nb, const int* boff, const int* bob, c
 //   [U     ] = [E^T           N] [r_U],   E = P N,
 // so one product replaces the chain M^-1 s -> K^T -> N -> P U - t, whose four
 // dependent steps cost a cluster barrier or a run of FP64 latency each.
-// E: one thread per entry, FP64 sums.
-__global__ void k_body_e(int n3, int m, const float* __restrict__ P, const double* __restrict__ N,
-                         float* __restrict__ E) {
+// The rows of lambda are FP32 (B), as the chain's products with M^-1 and P
+// were; the rows of U, (E^T N), are held and summed in FP64 (G), as the chain's
+// K^T, N and U were.
+// E: one thread per entry, FP64 sums; its transpose goes to G, rows of ldg.
+__global__ void k_body_e(int n3, int m, int ldg, const float* __restrict__ P, const double* __restrict__ N,
+                         float* __restrict__ E, double* __restrict__ G) {
   pdl_entry();
   const i64 t = (i64)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= (i64)n3 * m) return;
@@ -461,12 +464,14 @@ __global__ void k_body_e(int n3, int m, const float* __restrict__ P, const doubl
   }
   if (k < m) a0 = fma((double)P[(i64)r * m + k], N[(i64)k * m + c], a0);
   E[t] = (float)(a0 + a1);
+  G[(i64)c * ldg + r] = a0 + a1;
+  if (r < m) G[(i64)c * ldg + n3 + r] = N[(i64)c * m + r];   // m <= n3: three blobs a body at least
 }
 
-// The matrix B (rows of ld floats), 32 x 32 tiles of 256 threads.
+// The rows of lambda, B (n3 rows of ld floats), 32 x 32 tiles of 256 threads.
 __global__ void __launch_bounds__(256) k_body_matrix(int n3, int m, int ld, const float* __restrict__ Mi,
                                                      const float* __restrict__ P, const float* __restrict__ E,
-                                                     const double* __restrict__ N, float* __restrict__ B) {
+                                                     float* __restrict__ B) {
   pdl_entry();
   __shared__ float Es[32][33], Ps[32][33];
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
@@ -489,22 +494,19 @@ __global__ void __launch_bounds__(256) k_body_matrix(int n3, int m, int ld, cons
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     const int r = r0 + ty + 8 * q;
-    if (r >= n || c >= ld) continue;
+    if (r >= n3 || c >= ld) continue;
     float v = 0.f;
-    if (c < n) {
-      if (r < n3) v = c < n3 ? acc[q] - Mi[(i64)r * n3 + c] : E[(i64)r * m + c - n3];
-      else v = c < n3 ? E[(i64)c * m + r - n3] : (float)N[(i64)(r - n3) * m + c - n3];
-    }
+    if (c < n) v = c < n3 ? acc[q] - Mi[(i64)r * n3 + c] : E[(i64)r * m + c - n3];
     B[(i64)r * ld + c] = v;
   }
 }
 
 void dense_body_matrix(int nbl, int nb, const float* Minv, const float* P, const double* N, float* E, float* B,
-                       cudaStream_t s) {
+                       double* G, cudaStream_t s) {
   const int n3 = 3 * nbl, m = 6 * nb, ld = body_ld(n3 + m);
-  launch_k(k_body_e, nblk((i64)n3 * m, 256), 256, 0, s, n3, m, P, N, E);
+  launch_k(k_body_e, nblk((i64)n3 * m, 256), 256, 0, s, n3, m, ld, P, N, E, G);
   note_launch();
-  launch_k(k_body_matrix, dim3((ld + 31) / 32, (n3 + m + 31) / 32), 256, 0, s, n3, m, ld, Minv, P, E, N, B);
+  launch_k(k_body_matrix, dim3((ld + 31) / 32, (n3 + 31) / 32), 256, 0, s, n3, m, ld, Minv, P, E, B);
   note_launch();
 }
 
@@ -533,23 +535,49 @@ RBFIB_DEVFN float body_row(const float* __restrict__ row, const float4 pre[kBody
   return t;
 }
 
-// Coupled block, z = B (r_lambda + J v, r_U).  Every cluster of 8 CTAs forms
+// One row of G (n doubles) times x (shared memory) by L lanes, lane l of them;
+// a lane's first kBodyPre64 entries come from registers, the others in batches
+// whose loads are in flight together.  Every lane gets the product.
+constexpr int kBodyPre64 = 4;
+template <int L>
+RBFIB_DEVFN void body_words64(const double* __restrict__ g, int c, int n, double w[kBodyPre64]) {
+#pragma unroll
+  for (int u = 0; u < kBodyPre64; ++u) w[u] = c + L * u < n ? __ldg(g + c + L * u) : 0.0;
+}
+template <int L, typename X>
+RBFIB_DEVFN double body_row64(const double* __restrict__ g, double w[kBodyPre64], const X* x, int n, int l) {
+  double a[kBodyPre64] = {0.0, 0.0, 0.0, 0.0};
+  for (int c = l; c < n; c += L * kBodyPre64) {
+    if (c != l) body_words64<L>(g, c, n, w);
+#pragma unroll
+    for (int u = 0; u < kBodyPre64; ++u)
+      if (c + L * u < n) a[u] = fma(w[u], (double)x[c + L * u], a[u]);
+  }
+  double t = (a[0] + a[1]) + (a[2] + a[3]);
+#pragma unroll
+  for (int o = L / 2; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  return t;
+}
+
+// Coupled block, z = (B; G) (r_lambda + J v, r_U).  Every cluster of 8 CTAs forms
 // the whole input, one warp per blob component over the cluster, each value
 // written to all eight CTAs through distributed shared memory; after the one
 // cluster barrier (the gather's latency hides the first rows' loads, issued
-// before it) the rows are split over the CTAs of all clusters.
+// before it) the rows of B, and from the last warps down those of G, are split
+// over the CTAs of all clusters.
 constexpr int kBodyCtas = 8, kBodyThreads = 512;
 __global__ void __cluster_dims__(kBodyCtas, 1, 1) __launch_bounds__(kBodyThreads)
-    k_dense_body_apply(int n3, int m, int ld, const float* __restrict__ B, const float* __restrict__ r,
-                       float* __restrict__ z, double* __restrict__ z64, Dims d, const BlobStencil<float>* __restrict__ tab,
-                       const float* __restrict__ v) {
+    k_dense_body_apply(int n3, int m, int ld, const float* __restrict__ B, const double* __restrict__ G,
+                       const float* __restrict__ r, float* __restrict__ z, double* __restrict__ z64, Dims d,
+                       const BlobStencil<float>* __restrict__ tab, const float* __restrict__ v) {
   pdl_entry();
   namespace cg = cooperative_groups;
   cg::cluster_group cl = cg::this_cluster();
-  extern __shared__ __align__(16) float sv[];   // ld
+  extern __shared__ __align__(16) double svd[];   // the input in FP64 (ld), then in FP32
+  float* sv = reinterpret_cast<float*>(svd + ld);
   const int n = n3 + m;
-  const int rpc = (n + gridDim.x - 1) / gridDim.x;
-  const int r0 = blockIdx.x * rpc, r1 = min(n, r0 + rpc);
+  const int rpc = (n3 + gridDim.x - 1) / gridDim.x;
+  const int r0 = blockIdx.x * rpc, r1 = min(n3, r0 + rpc);
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = kBodyThreads / 32;
   // every CTA of the cluster must have started before its memory is written
   auto started = cl.barrier_arrive();
@@ -557,13 +585,31 @@ __global__ void __cluster_dims__(kBodyCtas, 1, 1) __launch_bounds__(kBodyThreads
   if (r0 + wid < r1)
 #pragma unroll
     for (int q = 0; q < kBodyPre; ++q) pre[q] = body_word(B + (i64)(r0 + wid) * ld, ld, lane + 32 * q);
+  // rows of G, a warp each, dealt to the CTAs from their last warps down
+  const int u0 = (int)blockIdx.x + (int)gridDim.x * (nw - 1 - wid);
+  double gw[kBodyPre64];
+  if (u0 < m) body_words64<32>(G + (i64)u0 * ld, lane, n, gw);
   cl.barrier_wait(std::move(started));
   for (int c = (int)cl.block_rank() * nw + wid; c < n3; c += kBodyCtas * nw) {
     const float s = r[c] + warp_interp<float>(d, c % 3, tab + c, v, lane);
-    if (lane < kBodyCtas) cl.map_shared_rank(sv, lane)[c] = s;
+    if (lane < kBodyCtas) {
+      cl.map_shared_rank(sv, lane)[c] = s;
+      cl.map_shared_rank(svd, lane)[c] = (double)s;
+    }
   }
-  for (int i = n3 + threadIdx.x; i < ld; i += kBodyThreads) sv[i] = i < n ? r[i] : 0.f;
+  for (int i = n3 + threadIdx.x; i < ld; i += kBodyThreads) {
+    sv[i] = i < n ? r[i] : 0.f;
+    svd[i] = (double)sv[i];
+  }
   cl.sync();
+  for (int u = u0; u < m; u += (int)gridDim.x * nw) {
+    if (u != u0) body_words64<32>(G + (i64)u * ld, lane, n, gw);
+    const double t = body_row64<32>(G + (i64)u * ld, gw, svd, n, lane);
+    if (lane == 0) {
+      z[n3 + u] = (float)t;
+      if (z64) z64[n3 + u] = (double)(float)t;
+    }
+  }
   for (int row = r0 + wid; row < r1; row += nw) {
     if (row != r0 + wid)
 #pragma unroll
@@ -576,21 +622,25 @@ __global__ void __cluster_dims__(kBodyCtas, 1, 1) __launch_bounds__(kBodyThreads
   }
 }
 
-void dense_body_apply(int nbl, int nb, const float* B, const float* r, float* z, double* z64, const Dims& d,
-                      const BlobStencil<float>* tab, const float* v, cudaStream_t s) {
+void dense_body_apply(int nbl, int nb, const float* B, const double* G, const float* r, float* z, double* z64,
+                      const Dims& d, const BlobStencil<float>* tab, const float* v, cudaStream_t s) {
   const int n3 = 3 * nbl, m = 6 * nb, ld = body_ld(n3 + m);
-  // about four rows per warp at most
-  const int clusters = std::max(1, (n3 + m + 4 * kBodyCtas * (kBodyThreads / 32) - 1) / (4 * kBodyCtas * (kBodyThreads / 32)));
-  launch_k(k_dense_body_apply, kBodyCtas * clusters, kBodyThreads, sizeof(float) * ld, s, n3, m, ld, B, r, z, z64, d, tab, v);
+  // about four rows of B per warp and 4096 FP64 products (1 us of the pipe)
+  // per CTA at most
+  const int rows = 4 * kBodyCtas * (kBodyThreads / 32), products = 4096 * kBodyCtas;
+  const int clusters = std::min(152 / kBodyCtas, std::max((n3 + rows - 1) / rows, (m * (n3 + m) + products - 1) / products));
+  launch_k(k_dense_body_apply, kBodyCtas * clusters, kBodyThreads, (sizeof(double) + sizeof(float)) * ld, s, n3, m, ld, B, G,
+           r, z, z64, d, tab, v);
   note_launch();
 }
 
-// Per-body block: the matrix of each body's shape (B_s, in the body frame, of
-// n_s = 3 blobs + 6 rows; host-built, all shapes one after the other), one
+// Per-body block: the matrices of each body's shape in the body frame (B_s of
+// 3 blobs rows, G_s of 6; host-built, all shapes one after the other), one
 // CTA per body: input gathered, its three-vectors (blob velocities, force,
 // torque) turned into the body frame, product, turned back.
 __global__ void __launch_bounds__(512) k_body_apply(int nbl, const int* __restrict__ boff, const int* __restrict__ shape_of,
                                                     const i64* __restrict__ shape_off, const float* __restrict__ Bs,
+                                                    const i64* __restrict__ shape_offg, const double* __restrict__ Gs,
                                                     const double* __restrict__ quat, const float* __restrict__ r,
                                                     float* __restrict__ z, double* __restrict__ z64, Dims d,
                                                     const BlobStencil<float>* __restrict__ tab, const float* __restrict__ vel) {
@@ -598,13 +648,20 @@ __global__ void __launch_bounds__(512) k_body_apply(int nbl, const int* __restri
   extern __shared__ __align__(16) float sh[];
   const int p = blockIdx.x, b0 = boff[p], n3 = 3 * (boff[p + 1] - b0), n = n3 + 6, ld = body_ld(n);
   const float* B = Bs + shape_off[shape_of[p]];
-  float* x = sh;        // input in the lab, later the result in the body frame
-  float* y = sh + ld;   // input in the body frame
+  const double* G = Gs + shape_offg[shape_of[p]];
+  float* x = sh;            // input in the lab, later lambda in the body frame
+  float* y = sh + ld;       // input in the body frame
+  __shared__ double U[8];   // U in the body frame
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
   float4 pre[kBodyPre];
-  if (wid < n)
+  if (wid < n3)
 #pragma unroll
     for (int q = 0; q < kBodyPre; ++q) pre[q] = body_word(B + (i64)wid * ld, ld, lane + 32 * q);
+  // rows of U, eight lanes each (few lanes of the two-lane FP64 pipe go to the
+  // sums over lanes): four by the last warp, two by the one before
+  const int u = min(4 * (nw - 1 - wid) + (lane >> 3), 5);
+  double gw[kBodyPre64];
+  if (wid >= nw - 2) body_words64<8>(G + (i64)u * ld, lane & 7, n, gw);
   // FP64 costs a warp instruction whatever its lanes do: the rotation by one
   // warp, the turns by one thread per component
   __shared__ double R[9];
@@ -627,7 +684,11 @@ __global__ void __launch_bounds__(512) k_body_apply(int nbl, const int* __restri
     y[t] = (float)(R[a] * (double)x[3 * i] + R[3 + a] * (double)x[3 * i + 1] + R[6 + a] * (double)x[3 * i + 2]);
   }
   __syncthreads();
-  for (int row = wid; row < n; row += nw) {
+  if (wid >= nw - 2) {
+    const double t = body_row64<8>(G + (i64)u * ld, gw, y, n, lane & 7);
+    if ((lane & 7) == 0) U[4 * (nw - 1 - wid) + (lane >> 3)] = t;
+  }
+  for (int row = wid; row < n3; row += nw) {
     if (row != wid)
 #pragma unroll
       for (int q = 0; q < kBodyPre; ++q) pre[q] = body_word(B + (i64)row * ld, ld, lane + 32 * q);
@@ -637,7 +698,10 @@ __global__ void __launch_bounds__(512) k_body_apply(int nbl, const int* __restri
   __syncthreads();
   for (int t = threadIdx.x; t < n; t += blockDim.x) {
     const int i = t / 3, a = t - 3 * i;
-    const float v = (float)(R[3 * a] * (double)x[3 * i] + R[3 * a + 1] * (double)x[3 * i + 1] + R[3 * a + 2] * (double)x[3 * i + 2]);
+    double w[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) w[c] = t < n3 ? (double)x[3 * i + c] : U[3 * i + c - n3];
+    const float v = (float)(R[3 * a] * w[0] + R[3 * a + 1] * w[1] + R[3 * a + 2] * w[2]);
     const i64 o = t < n3 ? 3 * (i64)b0 + t : 3 * (i64)nbl + 6 * p + t - n3;
     z[o] = v;
     if (z64) z64[o] = (double)v;
@@ -652,7 +716,8 @@ void body_apply(const BodyView& b, const ShapeView& sv, const float* r, float* z
   // a body's gathers and rows are dealt to its warps one after another, so
   // larger bodies take more of them (one 42-blob sphere's mobility solve in a 32^3
   // box 2.99 -> 2.78 ms)
-  launch_k(k_body_apply, b.nb, sv.max_blobs > 20 ? 512 : 256, shm, s, b.nbl, b.boff, sv.shape_of, sv.off, sv.B, b.quat, r, z, z64, d, b.st32, v);
+  launch_k(k_body_apply, b.nb, sv.max_blobs > 20 ? 512 : 256, shm, s, b.nbl, b.boff, sv.shape_of, sv.off, sv.B,
+           sv.offg, sv.G, b.quat, r, z, z64, d, b.st32, v);
   note_launch();
 }
 

@@ -31,8 +31,10 @@ struct BodyView {
 struct ShapeView {
   int max_blobs = 0;
   const int* shape_of = nullptr;   // nb
-  const i64* off = nullptr;        // of each shape's matrix in B
+  const i64* off = nullptr;        // of each shape's rows of lambda in B
   const float* B = nullptr;
+  const i64* offg = nullptr;       // of each shape's rows of U in G
+  const double* G = nullptr;
 };
 
 struct Potentials {
@@ -165,10 +167,10 @@ void ns_decide(const double* ss, cudaGraphConditionalHandle h, long long* warm, 
 __host__ __device__ constexpr int body_ld(int n) { return (n + 3) & ~3; }
 constexpr int kBodyMaxSmem = 160 * 1024;   // the per-body form's input and output: up to 6824 blobs a body
 void dense_body_matrix(int nbl, int nb, const float* Minv, const float* P, const double* N, float* E, float* B,
-                       cudaStream_t);
+                       double* G, cudaStream_t);
 // z = block (r_lambda + J v, r_U); r and z: the lambda and U parts of a
 // saddle vector; z64: FP64 copy of the result (null: none)
-void dense_body_apply(int nbl, int nb, const float* B, const float* r, float* z, double* z64, const Dims& d,
+void dense_body_apply(int nbl, int nb, const float* B, const double* G, const float* r, float* z, double* z64, const Dims& d,
                       const BlobStencil<float>* tab, const float* v, cudaStream_t);
 void body_apply(const BodyView&, const ShapeView&, const float* r, float* z, double* z64, const Dims& d,
                 const float* v, cudaStream_t);

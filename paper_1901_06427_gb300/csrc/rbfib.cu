@@ -162,13 +162,14 @@ struct rbfib_grid {
   // body-block preconditioner
   int max_blobs = 0;
   DBuf<int> shape_of;
-  DBuf<i64> shape_off;
+  DBuf<i64> shape_off, shape_offg;
   DBuf<float> shape_B;
+  DBuf<double> shape_G;
   // coupled (all-blob) body block for small suspensions
   bool dense_body = false;
   PairMobility pair{};   // blob pair functions of the grid's kernel
   DBuf<float> dM, dP, dE, dB;
-  DBuf<double> dN, dNw;
+  DBuf<double> dN, dNw, dG;
   DBuf<int> dstatus;
   // Newton-Schulz update of dM from the previous configuration's inverse:
   // work matrices, the residual norm, whether dM holds a valid inverse, and
@@ -305,6 +306,8 @@ ShapeView shapes_of(rbfib_grid* g) {
   v.shape_of = g->shape_of;
   v.off = g->shape_off;
   v.B = g->shape_B;
+  v.offg = g->shape_offg;
+  v.G = g->shape_G;
   return v;
 }
 
@@ -507,7 +510,7 @@ void precond(rbfib_grid* g, const T* r, T* z, bool with_bodies, double* z64, dou
     if (with_bodies && g->nb > 0) {
       const BodyView bv = view_of(g, g->cur);
       double* zb64 = z64 ? z64 + g->nfl : nullptr;
-      if (g->dense_body) dense_body_apply(g->nbl, g->nb, g->dB, r + g->nfl, z + g->nfl, zb64, d, bv.st32, zv, g->s);
+      if (g->dense_body) dense_body_apply(g->nbl, g->nb, g->dB, g->dG, r + g->nfl, z + g->nfl, zb64, d, bv.st32, zv, g->s);
       else body_apply(bv, shapes_of(g), r + g->nfl, z + g->nfl, zb64, d, zv, g->s);
     }
   }
@@ -1072,7 +1075,7 @@ void build_body_block(rbfib_grid* g, const double* r, const double* arm, const d
       dense_body_gj(g->nbl, g->dM, g->dMw, g->dUw, g->dstatus, g->s);
     }
     dense_body_finish(g->nbl, g->nb, g->boff, arm, g->dM, g->dP, g->dN, g->dNw, g->dstatus, g->s);
-    dense_body_matrix(g->nbl, g->nb, g->dM, g->dP, g->dN, g->dE, g->dB, g->s);
+    dense_body_matrix(g->nbl, g->nb, g->dM, g->dP, g->dN, g->dE, g->dB, g->dG, g->s);
     ck(cudaMemcpyAsync(g->dinfo.p + 13, g->dstatus.p, sizeof(int), cudaMemcpyDeviceToDevice, g->s));
     if (quat) ck(cudaMemcpyAsync(g->dquat.p, quat, sizeof(double) * 4 * g->nb, cudaMemcpyDeviceToDevice, g->s));
     return;
@@ -1082,7 +1085,7 @@ void build_body_block(rbfib_grid* g, const double* r, const double* arm, const d
   g->dM_valid = false;
   ck(dense_body_build(g->nbl, g->nb, g->boff, g->bob, r, arm, quat, qold, g->pair, g->desc.h, g->desc.eta, g->dM, g->dP,
                       g->dN, g->dstatus, g->dMw, g->dTw, g->dUw, g->dNw, g->dss, g->h_pinned + 40, warm, g->s, &used));
-  dense_body_matrix(g->nbl, g->nb, g->dM, g->dP, g->dN, g->dE, g->dB, g->s);
+  dense_body_matrix(g->nbl, g->nb, g->dM, g->dP, g->dN, g->dE, g->dB, g->dG, g->s);
   int* hstat = (int*)(g->h_pinned + 42);
   ck(cudaMemcpyAsync(hstat, g->dstatus, sizeof(int), cudaMemcpyDeviceToHost, g->s));
   ck(cudaStreamSynchronize(g->s));
@@ -1132,9 +1135,9 @@ void alloc_solver(rbfib_grid* g) {
   g->bvec.ensure(n); g->xvec.ensure(n); g->xrfd.ensure(n);
 }
 
-// Appends the body-block matrix of a shape of n blobs x (body frame; k_body.cu)
-// to sB.  Returns why there is none, or null.
-const char* shape_matrix(const rbfib_grid* g, const double* x, int n, std::vector<float>& sB) {
+// Appends the body-block matrix of a shape of n blobs x (body frame; k_body.cu),
+// its rows of lambda to sB and of U to sG.  Returns why there is none, or null.
+const char* shape_matrix(const rbfib_grid* g, const double* x, int n, std::vector<float>& sB, std::vector<double>& sG) {
   const int n3 = 3 * n, ld = body_ld(n3 + 6);
   std::vector<double> M;
   if (!pair_inverse(x, n, g->pair, g->desc.h, g->desc.eta, M)) return "blob mobility of a shape is singular";
@@ -1158,19 +1161,19 @@ const char* shape_matrix(const rbfib_grid* g, const double* x, int n, std::vecto
   for (int r = 0; r < n3; ++r)
     for (int c = 0; c < 6; ++c)
       for (int k = 0; k < 6; ++k) E[(size_t)r * 6 + c] += P[(size_t)r * 6 + k] * N[6 * k + c];
-  for (int r = 0; r < n3 + 6; ++r)
+  for (int r = 0; r < n3; ++r)
     for (int c = 0; c < ld; ++c) {
       double v = 0.0;
-      if (c < n3 + 6) {
-        if (r < n3 && c < n3) {
-          v = -M[(size_t)r * n3 + c];
-          for (int k = 0; k < 6; ++k) v += E[(size_t)r * 6 + k] * P[(size_t)c * 6 + k];
-        } else if (r < n3) v = E[(size_t)r * 6 + c - n3];
-        else if (c < n3) v = E[(size_t)c * 6 + r - n3];
-        else v = N[6 * (r - n3) + c - n3];
+      if (c < n3) {
+        v = -M[(size_t)r * n3 + c];
+        for (int k = 0; k < 6; ++k) v += E[(size_t)r * 6 + k] * P[(size_t)c * 6 + k];
+      } else if (c < n3 + 6) {
+        v = E[(size_t)r * 6 + c - n3];
       }
       sB.push_back((float)v);
     }
+  for (int r = 0; r < 6; ++r)
+    for (int c = 0; c < ld; ++c) sG.push_back(c < n3 ? E[(size_t)c * 6 + r] : (c < n3 + 6 ? N[6 * r + c - n3] : 0.0));
   return nullptr;
 }
 
@@ -1560,12 +1563,14 @@ int rbfib_set_bodies(rbfib_grid* g, int32_t n_bodies, const int32_t* blob_offset
     // per-shape body-block matrices in the body frame (k_body.cu)
     const bool dense = nb >= 2 && 3 * nbl <= kDenseBodyMaxRows && 6 * nb <= kDenseBodyMaxBodyRows;
     const int ns = (int)shape_rep.size();
-    std::vector<i64> soff(std::max(ns, 1), 0);
+    std::vector<i64> soff(std::max(ns, 1), 0), soffg(std::max(ns, 1), 0);
     std::vector<float> sB;
+    std::vector<double> sG;
     for (int s = 0; s < ns && !dense; ++s) {
       const int p = shape_rep[s];
       soff[s] = (i64)sB.size();
-      if (const char* why = shape_matrix(g, ref.data() + 3 * (size_t)off[p], off[p + 1] - off[p], sB))
+      soffg[s] = (i64)sG.size();
+      if (const char* why = shape_matrix(g, ref.data() + 3 * (size_t)off[p], off[p + 1] - off[p], sB, sG))
         return fail(g, RBFIB_EINVAL, std::string("set_bodies: ") + why);
     }
 
@@ -1603,7 +1608,8 @@ int rbfib_set_bodies(rbfib_grid* g, int32_t n_bodies, const int32_t* blob_offset
       g->dquat.alloc(4 * (size_t)nb);
       g->dP.alloc((size_t)18 * nbl * nb);
       g->dE.alloc((size_t)18 * nbl * nb);
-      g->dB.alloc((size_t)(3 * nbl + 6 * nb) * body_ld(3 * nbl + 6 * nb));
+      g->dB.alloc((size_t)3 * nbl * body_ld(3 * nbl + 6 * nb));
+      g->dG.alloc((size_t)6 * nb * body_ld(3 * nbl + 6 * nb));
       g->dN.alloc((size_t)36 * nb * nb);
       g->dNw.alloc((size_t)72 * nb * nb);
       g->dstatus.alloc(1);
@@ -1617,6 +1623,11 @@ int rbfib_set_bodies(rbfib_grid* g, int32_t n_bodies, const int32_t* blob_offset
     g->shape_B.alloc(std::max<size_t>(sB.size(), 1));
     if (!sB.empty())
       ck(cudaMemcpyAsync(g->shape_B, sB.data(), sizeof(float) * sB.size(), cudaMemcpyHostToDevice, g->s));
+    g->shape_offg.alloc(std::max(ns, 1));
+    ck(cudaMemcpyAsync(g->shape_offg, soffg.data(), sizeof(i64) * std::max(ns, 1), cudaMemcpyHostToDevice, g->s));
+    g->shape_G.alloc(std::max<size_t>(sG.size(), 1));
+    if (!sG.empty())
+      ck(cudaMemcpyAsync(g->shape_G, sG.data(), sizeof(double) * sG.size(), cudaMemcpyHostToDevice, g->s));
     ck(cudaStreamSynchronize(g->s));
     // body-sized work arrays
     const size_t b6 = 6 * (size_t)std::max(nb, 1), l3 = 3 * (size_t)std::max(nbl, 1);
