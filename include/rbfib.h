@@ -287,7 +287,8 @@ int rbfib_krylov_stats(const rbfib_grid* g, int64_t* iterations, int64_t* second
  * kernels: out[0] FP64 Stokes operator, out[1] FP32 Stokes operator (0 on
  * uniform spacing, whose Stokes kernels have fixed tile shapes), out[2]
  * velocity smoothing sweep, out[3] pressure smoothing sweep (as 32 x n/32
- * blocks on uniform spacing). */
+ * blocks on uniform spacing; 256, untimed, where the finest level is solved
+ * exactly and not smoothed). */
 int rbfib_tuned_blocks(const rbfib_grid* g, int32_t out[4]);
 
 /* ---- building blocks of the hot path, exposed for parity checks ---------- */

@@ -1264,8 +1264,11 @@ void autotune(rbfib_grid* g) {
   t.stokes32 = uniform ? 0 : pick_block(g->s, [&](int bs) {
     stokes_apply<float>(d, (float)eta, x32, x32 + g->nf, y32, y32 + g->nf, g->s, bs);
   });
-  t.vrbgs = pick_block(g->s, [&](int bs) { vel_rbgs<float>(d, (float)eta, 0, x32, y32, g->s, bs); });
-  t.prbgs = pick_block(g->s, [&](int bs) { p_rbgs<float>(d, 0, x32 + g->nf, y32 + g->nf, g->s, bs); });
+  // the smoothing sweeps only where the finest level has any (build_fd)
+  if (g->fd_vel != 0)
+    t.vrbgs = pick_block(g->s, [&](int bs) { vel_rbgs<float>(d, (float)eta, 0, x32, y32, g->s, bs); });
+  if (g->fd_p != 0)
+    t.prbgs = pick_block(g->s, [&](int bs) { p_rbgs<float>(d, 0, x32 + g->nf, y32 + g->nf, g->s, bs); });
   g->tune = t;
   std::lock_guard<std::mutex> lk(g_tune_mu);
   g_tune_cache[key] = t;
