@@ -1179,14 +1179,4 @@ void refine_check(const double* rn2, double* rst, int* rsi, const int* inner, do
   note_launch();
 }
 
-// Condition of an IF node from a device int (nonzero -> 1).
-__global__ void k_cond_from(const int* flag, cudaGraphConditionalHandle h) {
-  pdl_entry();
-  if (threadIdx.x == 0 && blockIdx.x == 0) cudaGraphSetConditional(h, flag[0] ? 1u : 0u);
-}
-void cond_from(const int* flag, cudaGraphConditionalHandle h, cudaStream_t s) {
-  launch_k(k_cond_from, 1, 32, 0, s, flag, h);
-  note_launch();
-}
-
 }  // namespace rbfib

@@ -1227,8 +1227,9 @@ void add_grad(const Dims& d, T eta, T kappa, const T* phi, const T* q, T* z, dou
   note_launch();
 }
 
+template void stokes_apply<double>(const Dims&, double, const double*, const double*, double*, double*, cudaStream_t, int);
+template void stokes_apply<float>(const Dims&, float, const float*, const float*, float*, float*, cudaStream_t, int);
 #define INST(T)                                                                                  \
-  template void stokes_apply<T>(const Dims&, T, const T*, const T*, T*, T*, cudaStream_t, int);  \
   template void vel_rbgs<T>(const Dims&, T, int, T*, const T*, cudaStream_t, int);               \
   template void vel_first<T>(const Dims&, T, T*, const T*, cudaStream_t);                         \
   template bool vel_first2<T>(const Dims&, T, T*, const T*, cudaStream_t, int);                   \
@@ -1243,8 +1244,7 @@ void add_grad(const Dims& d, T eta, T kappa, const T* phi, const T* q, T* z, dou
   template void p_coarse<T>(const Dims&, T*, T*, int, cudaStream_t);                             \
   template void div_q<T>(const Dims&, const T*, const T*, T*, cudaStream_t);                     \
   template void add_grad<T>(const Dims&, T, T, const T*, const T*, T*, double*, cudaStream_t);
-INST(double)
-INST(float)
+INST(float)   // the preconditioner is FP32
 #undef INST
 
 }  // namespace rbfib

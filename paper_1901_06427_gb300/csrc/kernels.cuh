@@ -249,7 +249,6 @@ void refine_init(double* rst, int* rsi, cudaGraphConditionalHandle h, int* info,
 void refine_sweep(double* rst, int* rsi, double rtol, double inner_tol, int maxit, int m, cudaStream_t);
 void refine_check(const double* rn2, double* rst, int* rsi, const int* inner, double rtol, int maxit,
                   cudaGraphConditionalHandle h, int* info, double* rel, cudaStream_t);
-void cond_from(const int* flag, cudaGraphConditionalHandle h, cudaStream_t);
 template <typename T> void multi_axpy_dev(T* w, const T* V, i64 ldv, const int* ist, const double* coef,
                                           double sign, i64 n, int nparts, cudaStream_t);
 

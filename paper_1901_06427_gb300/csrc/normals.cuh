@@ -6,8 +6,7 @@
 // rounded once; the square root, conversions and products are left in FP64.
 // Against extended precision: mean 0.43, at most 2.3 units in the last place
 // (the library: 0.46, 2.8).  Forcing of a 128 x 128 x 64 grid, 9.4 million
-// normals: 698 -> 226 us.  The host branches let the functions be checked
-// without a GPU.
+// normals: 698 -> 226 us.
 #pragma once
 #include <cmath>
 
@@ -17,49 +16,27 @@ namespace rbfib {
 
 typedef unsigned long long u64;
 
-__host__ __device__ inline u64 mul_hi(u64 a, u64 b) {
-#ifdef __CUDA_ARCH__
+__device__ __forceinline__ u64 mul_hi(u64 a, u64 b) {
   return __umul64hi(a, b);
-#else
-  return (u64)(((unsigned __int128)a * b) >> 64);
-#endif
 }
-__host__ __device__ inline long long mul_hi_s(long long a, long long b) {
-#ifdef __CUDA_ARCH__
+__device__ __forceinline__ long long mul_hi_s(long long a, long long b) {
   return __mul64hi(a, b);
-#else
-  return (long long)(((__int128)a * b) >> 64);
-#endif
 }
-__host__ __device__ inline int lead_zeros(u64 a) {
-#ifdef __CUDA_ARCH__
+__device__ __forceinline__ int lead_zeros(u64 a) {
   return __clzll((long long)a);
-#else
-  return __builtin_clzll(a);
-#endif
 }
 
 // v / 2^63 for v in [2^62, 2^63], from its bits (rounded to 53)
-__host__ __device__ inline double unit_double(u64 v) {
+__device__ __forceinline__ double unit_double(u64 v) {
   const u64 m = (v + 512) >> 10;   // 53 bits, 2^53 for 1
   const u64 bits = (0x3FEULL << 52) + (m - (1ULL << 52));
-#ifdef __CUDA_ARCH__
   return __longlong_as_double((long long)bits);
-#else
-  double d;
-  __builtin_memcpy(&d, &bits, 8);
-  return d;
-#endif
 }
 
 // v 2^e, v > 0 (one rounding), -200 < e < 0
-__host__ __device__ inline double scaled_double(u64 v, int e) {
-#ifdef __CUDA_ARCH__
+__device__ __forceinline__ double scaled_double(u64 v, int e) {
   const double d = __ull2double_rn(v);
   return __hiloint2double(__double2hiint(d) + (e << 20), __double2loint(d));
-#else
-  return ldexp((double)v, e);
-#endif
 }
 
 // cos and sin of 2 pi k / 2^53 (k odd): the nearest quarter turn q and the
@@ -67,7 +44,7 @@ __host__ __device__ inline double scaled_double(u64 v, int e) {
 // z = t^2 the series of sin(x) / t and cos(x), x = (pi / 4) t, have terms
 // (pi / 4)^(2n + 1) / (2n + 1)! and (pi / 4)^2n / (2n)! in 2^64 fixed point,
 // falling, so the alternating Horner sums stay positive.
-__host__ __device__ inline void fixed_cossin(u64 k, double& c, double& s) {
+__device__ __forceinline__ void fixed_cossin(u64 k, double& c, double& s) {
   const u64 K = k << 11;
   const u64 q = (K + (1ULL << 61)) >> 62;
   const long long rest = (long long)(K - (q << 62));
@@ -80,13 +57,9 @@ __host__ __device__ inline void fixed_cossin(u64 k, double& c, double& s) {
       0x00000069B47CA881ULL, 0x000000007E74E28EULL, 0x00000000006DB894ULL, 0x0000000000004832ULL,
       0x0000000000000025ULL};
   u64 as = fs[8], ac = fc[8];
-#ifdef __CUDA_ARCH__
 #pragma unroll
-#endif
   for (int n = 7; n >= 0; --n) as = fs[n] - mul_hi(z, as);
-#ifdef __CUDA_ARCH__
 #pragma unroll
-#endif
   for (int n = 7; n >= 0; --n) ac = fc[n] - mul_hi(z, ac);
   const double cx = unit_double((1ULL << 63) - (mul_hi(z, ac) >> 1));
   // sin x = t times the sum, from the normalised t: one rounding
@@ -136,10 +109,7 @@ constexpr int kLogHalf = 53;
   {68618, 211931326892856672LL}, {68339, 193142040051111389LL}, {68062, 174411403425541569LL}, {67787, 155740446887414269LL}, \
   {67514, 137130207619826967LL}, {67243, 118581730052356888LL}, {66975, 100164923133719907LL}, {66709, 81812538408213418LL}, \
   {66444, 63456235382273711LL}, {66182, 45235625417602780LL}, {65922, 27082656347884782LL}, {65536, 0LL}
-#ifdef __CUDACC__
 static __device__ const LogEntry kLogDev[128] = {RBFIB_LOG_TABLE};
-#endif
-static const LogEntry kLogHost[128] = {RBFIB_LOG_TABLE};
 #undef RBFIB_LOG_TABLE
 
 // -log(k / 2^53), k odd: k = m 2^e, r = m c - 1 exactly (|r| < 2^-7, scale
@@ -147,25 +117,19 @@ static const LogEntry kLogHost[128] = {RBFIB_LOG_TABLE};
 // Added up in fixed point (scale 2^57 where a multiple of log 2 makes the
 // result at least 1 / 3, 2^62 below) and rounded once; next to 1 the
 // normalised product keeps the relative accuracy.
-__host__ __device__ inline double fixed_neglog(u64 k) {
+__device__ __forceinline__ double fixed_neglog(u64 k) {
   const u64 K = k << 11;
   const int n = lead_zeros(K);
   const u64 M = K << n;
   const int i = (int)(M >> 56) & 127;
-#ifdef __CUDA_ARCH__
   const LogEntry e = kLogDev[i];
-#else
-  const LogEntry e = kLogHost[i];
-#endif
   const bool half = i >= kLogHalf;
   const long long hi = (long long)mul_hi(M, (u64)e.c) - (half ? 65536 : 32768);
   const u64 lo = M * (u64)e.c;
   const long long R = half ? (long long)(((u64)hi << 54) | (lo >> 10)) : (long long)(((u64)hi << 55) | (lo >> 9));
   const long long one = 1LL << 62;
   long long a = one / 8;
-#ifdef __CUDA_ARCH__
 #pragma unroll
-#endif
   for (int j = 7; j >= 1; --j) a = one / j - (mul_hi_s(R, a) >> 6);
   const int n2 = half ? n : n + 1;
   const long long rp = mul_hi_s(R, a);              // r p, scale 2^68
@@ -177,7 +141,7 @@ __host__ __device__ inline double fixed_neglog(u64 k) {
 }
 
 // Two standard normals of two 64-bit words: u = (2 (word >> 12) + 1) 2^-53.
-__host__ __device__ inline void box_muller(u64 w0, u64 w1, double& z0, double& z1) {
+__device__ __forceinline__ void box_muller(u64 w0, u64 w1, double& z0, double& z1) {
   const double rad = sqrt(2.0 * fixed_neglog((w0 >> 12) * 2 + 1));
   double c, s;
   fixed_cossin((w1 >> 12) * 2 + 1, c, s);

@@ -184,7 +184,6 @@ struct rbfib_grid {
   double* h_pinned = nullptr;
   int nparts = 0;
   // precision-specific stores
-  MGStore<double> mg64;
   MGStore<float> mg32;
   KrylovStore<double> kr64;
   KrylovStore<float> kr32;
