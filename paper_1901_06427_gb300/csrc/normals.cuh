@@ -16,25 +16,25 @@ namespace rbfib {
 
 typedef unsigned long long u64;
 
-__device__ __forceinline__ u64 mul_hi(u64 a, u64 b) {
+__device__ inline u64 mul_hi(u64 a, u64 b) {
   return __umul64hi(a, b);
 }
-__device__ __forceinline__ long long mul_hi_s(long long a, long long b) {
+__device__ inline long long mul_hi_s(long long a, long long b) {
   return __mul64hi(a, b);
 }
-__device__ __forceinline__ int lead_zeros(u64 a) {
+__device__ inline int lead_zeros(u64 a) {
   return __clzll((long long)a);
 }
 
 // v / 2^63 for v in [2^62, 2^63], from its bits (rounded to 53)
-__device__ __forceinline__ double unit_double(u64 v) {
+__device__ inline double unit_double(u64 v) {
   const u64 m = (v + 512) >> 10;   // 53 bits, 2^53 for 1
   const u64 bits = (0x3FEULL << 52) + (m - (1ULL << 52));
   return __longlong_as_double((long long)bits);
 }
 
 // v 2^e, v > 0 (one rounding), -200 < e < 0
-__device__ __forceinline__ double scaled_double(u64 v, int e) {
+__device__ inline double scaled_double(u64 v, int e) {
   const double d = __ull2double_rn(v);
   return __hiloint2double(__double2hiint(d) + (e << 20), __double2loint(d));
 }
@@ -44,7 +44,7 @@ __device__ __forceinline__ double scaled_double(u64 v, int e) {
 // z = t^2 the series of sin(x) / t and cos(x), x = (pi / 4) t, have terms
 // (pi / 4)^(2n + 1) / (2n + 1)! and (pi / 4)^2n / (2n)! in 2^64 fixed point,
 // falling, so the alternating Horner sums stay positive.
-__device__ __forceinline__ void fixed_cossin(u64 k, double& c, double& s) {
+__device__ inline void fixed_cossin(u64 k, double& c, double& s) {
   const u64 K = k << 11;
   const u64 q = (K + (1ULL << 61)) >> 62;
   const long long rest = (long long)(K - (q << 62));
@@ -117,7 +117,7 @@ static __device__ const LogEntry kLogDev[128] = {RBFIB_LOG_TABLE};
 // Added up in fixed point (scale 2^57 where a multiple of log 2 makes the
 // result at least 1 / 3, 2^62 below) and rounded once; next to 1 the
 // normalised product keeps the relative accuracy.
-__device__ __forceinline__ double fixed_neglog(u64 k) {
+__device__ inline double fixed_neglog(u64 k) {
   const u64 K = k << 11;
   const int n = lead_zeros(K);
   const u64 M = K << n;
@@ -141,7 +141,7 @@ __device__ __forceinline__ double fixed_neglog(u64 k) {
 }
 
 // Two standard normals of two 64-bit words: u = (2 (word >> 12) + 1) 2^-53.
-__device__ __forceinline__ void box_muller(u64 w0, u64 w1, double& z0, double& z1) {
+__device__ inline void box_muller(u64 w0, u64 w1, double& z0, double& z1) {
   const double rad = sqrt(2.0 * fixed_neglog((w0 >> 12) * 2 + 1));
   double c, s;
   fixed_cossin((w1 >> 12) * 2 + 1, c, s);
