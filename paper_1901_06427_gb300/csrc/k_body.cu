@@ -563,8 +563,7 @@ RBFIB_DEVFN double body_row64(const double* __restrict__ g, double w[kBodyPre64]
 // the whole input, one warp per blob component over the cluster, each value
 // written to all eight CTAs through distributed shared memory; after the one
 // cluster barrier (the gather's latency hides the first rows' loads, issued
-// before it) the rows of B, and from the last warps down those of G, are split
-// over the CTAs of all clusters.
+// before it) the rows of B and G are split over the CTAs of all clusters.
 constexpr int kBodyCtas = 8, kBodyThreads = 512;
 __global__ void __cluster_dims__(kBodyCtas, 1, 1) __launch_bounds__(kBodyThreads)
     k_dense_body_apply(int n3, int m, int ld, const float* __restrict__ B, const double* __restrict__ G,
@@ -582,11 +581,12 @@ __global__ void __cluster_dims__(kBodyCtas, 1, 1) __launch_bounds__(kBodyThreads
   // every CTA of the cluster must have started before its memory is written
   auto started = cl.barrier_arrive();
   float4 pre[kBodyPre];
-  if (r0 + wid < r1)
+  // the last nu warps take the CTA's share of the rows of G, the others that of B
+  const int nu = min(nw / 2, (m + (int)gridDim.x - 1) / (int)gridDim.x), nr = nw - nu;
+  if (wid < nr && r0 + wid < r1)
 #pragma unroll
     for (int q = 0; q < kBodyPre; ++q) pre[q] = body_word(B + (i64)(r0 + wid) * ld, ld, lane + 32 * q);
-  // rows of G, a warp each, dealt to the CTAs from their last warps down
-  const int u0 = (int)blockIdx.x + (int)gridDim.x * (nw - 1 - wid);
+  const int u0 = wid < nr ? m : (int)blockIdx.x + (int)gridDim.x * (wid - nr);
   double gw[kBodyPre64];
   if (u0 < m) body_words64<32>(G + (i64)u0 * ld, lane, n, gw);
   cl.barrier_wait(std::move(started));
@@ -602,7 +602,7 @@ __global__ void __cluster_dims__(kBodyCtas, 1, 1) __launch_bounds__(kBodyThreads
     svd[i] = (double)sv[i];
   }
   cl.sync();
-  for (int u = u0; u < m; u += (int)gridDim.x * nw) {
+  for (int u = u0; u < m; u += (int)gridDim.x * nu) {
     if (u != u0) body_words64<32>(G + (i64)u * ld, lane, n, gw);
     const double t = body_row64<32>(G + (i64)u * ld, gw, svd, n, lane);
     if (lane == 0) {
@@ -610,7 +610,7 @@ __global__ void __cluster_dims__(kBodyCtas, 1, 1) __launch_bounds__(kBodyThreads
       if (z64) z64[n3 + u] = (double)(float)t;
     }
   }
-  for (int row = r0 + wid; row < r1; row += nw) {
+  for (int row = wid < nr ? r0 + wid : r1; row < r1; row += nr) {
     if (row != r0 + wid)
 #pragma unroll
       for (int q = 0; q < kBodyPre; ++q) pre[q] = body_word(B + (i64)row * ld, ld, lane + 32 * q);
@@ -654,11 +654,13 @@ __global__ void __launch_bounds__(512) k_body_apply(int nbl, const int* __restri
   __shared__ double U[8];   // U in the body frame
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
   float4 pre[kBodyPre];
-  if (wid < n3)
+  if (wid < min(n3, nw - 2))
 #pragma unroll
     for (int q = 0; q < kBodyPre; ++q) pre[q] = body_word(B + (i64)wid * ld, ld, lane + 32 * q);
   // rows of U, eight lanes each (few lanes of the two-lane FP64 pipe go to the
-  // sums over lanes): four by the last warp, two by the one before
+  // sums over lanes): four by the last warp, two by the one before, which take
+  // no rows of B (with some of them one sphere's solve in a 32^3 box took 2.72 ms,
+  // now 2.68)
   const int u = min(4 * (nw - 1 - wid) + (lane >> 3), 5);
   double gw[kBodyPre64];
   if (wid >= nw - 2) body_words64<8>(G + (i64)u * ld, lane & 7, n, gw);
@@ -688,7 +690,7 @@ __global__ void __launch_bounds__(512) k_body_apply(int nbl, const int* __restri
     const double t = body_row64<8>(G + (i64)u * ld, gw, y, n, lane & 7);
     if ((lane & 7) == 0) U[4 * (nw - 1 - wid) + (lane >> 3)] = t;
   }
-  for (int row = wid; row < n3; row += nw) {
+  for (int row = wid < nw - 2 ? wid : n3; row < n3; row += nw - 2) {
     if (row != wid)
 #pragma unroll
       for (int q = 0; q < kBodyPre; ++q) pre[q] = body_word(B + (i64)row * ld, ld, lane + 32 * q);
