@@ -314,14 +314,16 @@ RBFIB_DEVFN void quat_rot(const double* qt, double R[9]) {
   R[6] = 2 * (x * z - w * y); R[7] = 2 * (y * z + w * x); R[8] = 1 - 2 * (x * x + y * y);
 }
 
-// Programmatic dependent launch.  Every kernel of the library begins with
-// pdl_entry(), before it touches global memory: griddepcontrol.wait returns
+// Programmatic dependent launch.  Every kernel of the library calls
+// pdl_entry() before it touches global memory that another kernel writes (the
+// level solves stage their constant tables first, uploaded before any of
+// them is launched): griddepcontrol.wait returns
 // once the kernels this grid depends on have completed and their memory
 // operations are visible (at once for a normal launch).  A kernel launched
 // by launch_k carries the programmatic-serialization attribute, so it may be
 // launched as soon as every block of its predecessor has exited, without
-// waiting for the predecessor's completion to be processed; since its own
-// first instruction is the wait, neither read-after-write nor
+// waiting for the predecessor's completion to be processed; since all
+// it reads and writes of theirs follows the wait, neither read-after-write nor
 // write-after-read order between the two kernels changes.  No kernel
 // releases its dependents early (griddepcontrol.launch_dependents): on
 // GB300 that placed the blocks of the next short grid while the current one

@@ -355,6 +355,9 @@ constexpr int kNSIters = 4;   // even: the result lands in Minv
 // Up to this size the warm start's eight products take about as long as the
 // blocked inversion (40 us each at n = 252); above it they grow with n^3
 // while the inversion's launches grow with n.
+// With this M the start is close after small moves only: two 42-blob spheres'
+// Brownian steps (0.05 h, 0.016 rad) leave ||R0||_F at 2 to 4 and are inverted
+// anew, a hundredth of them 0.02 to 0.04.
 constexpr int kNSMaxRows = 256;
 bool dense_body_warm(int nbl) { return 3 * nbl <= kNSMaxRows; }
 // The pieces of the set-up, also used one by one by the device-driven SEM

@@ -465,10 +465,13 @@ void vcycle_p(rbfib_grid* g, T* u0, T* rhs0) {
 
 // kappa of the pressure block: per axis the walls' share of the viscous drag
 // on a flow across it, 12 / H^2 between two no-slip walls, 3 / H^2 (half a
-// channel of height 2 H) with one of them free-slip; the smallest sum over
-// the two axes across a direction, which is that of the longest waves.
-// Krylov iterations of a fluid-driven and a sphere's solve to 1e-8: two-sphere
-// box 33 -> 27 (rigid), slit of 384 x 48 x 12 57 -> 35 (fluid).
+// channel of height 2 H) with one of them free-slip; the smallest of the three
+// directions' sums over the two axes across them, so that no wave's drag is
+// overstated.  It is that of waves across the narrowest gap, the shortest
+// ones: nothing in a slit that is periodic along it, and a small part of what
+// waves along a thin channel feel (12 / 96^2 for 12 / 12^2 + 12 / 96^2 in 384 x 96 x
+// 12).  Krylov iterations of a fluid-driven and a sphere's solve to 1e-8:
+// two-sphere box 33 -> 27 (rigid), channel of 384 x 48 x 12 57 -> 35 (fluid).
 double pressure_kappa(const Dims& d) {
   double drag[3];
   for (int b = 0; b < 3; ++b) {
