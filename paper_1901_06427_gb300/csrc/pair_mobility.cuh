@@ -23,12 +23,17 @@
 // the point dipole's, is taken off the average: the two meet at 6 without a
 // step, at most 0.8% (0.4%) below the average, and only ripples of that
 // density's transform at short waves are left below zero (pair_raise).
-// The six-point table then adds 1.5e-5 (1 - r/6)^4 (4 r/6 + 1) to f and g (also
-// positive definite): a closed shell's uniform normal force, against which
-// the enclosed fluid hardly yields, has mobility 2e-6 on average but several
-// times that and less as the shell sits on the grid, and FP32 sweeps stall
-// when M takes it that small (22 shells of 42 blobs refined to 1e-10: 528
-// iterations without, 192 with; the sampled averages 190).
+// A closed shell's uniform normal force, against which the enclosed fluid
+// hardly yields, has the smallest mobility, and how small depends on how the
+// shell sits on the grid:
+// - the three-point table takes half of the average's part along k,
+//   compressible motions that the kernel's aliases let through: a shell of 12
+//   blobs then has 1.3e-4 (1.9e-4 with all of it; 1.0e-4 on the grid at a sample
+//   place); with all of it an ensemble took 2% longer, with none a monolayer 3%;
+// - the six-point table adds 1.5e-5 (1 - r/6)^4 (4 r/6 + 1), also positive
+//   definite, to f and g: FP32 sweeps stall when M takes a shell of 42 blobs at
+//   2e-6 (22 of them refined to 1e-10: 528 iterations without, 192 with; the
+//   sampled averages 190).
 // Near r = 0 f and g are flat, where the Rotne-Prager-Yamakawa tensor has a
 // corner, so the smallest eigenvalues of M, which set the solver's
 // iterations, are up to 50 times smaller than the tensor's.  Both constrained
@@ -61,14 +66,14 @@ inline void pair_tail(double a, double r, double& f, double& g) {
 // r = 6.
 inline PairMobility pair_mobility(int kw) {
   static const double three[2][kPairKnots] = {
-    {0.058383518, 0.057064867, 0.053407145, 0.048098018, 0.041981828, 0.035881263, 0.030397332, 0.025812839,
-     0.022161247, 0.019321799, 0.017112281, 0.015364997, 0.013952640, 0.012786548, 0.011806782, 0.010971495,
+    {0.058368451, 0.057051804, 0.053397584, 0.048091051, 0.041976915, 0.035878361, 0.030395895, 0.025812222,
+     0.022161058, 0.019321777, 0.017112285, 0.015364995, 0.013952638, 0.012786547, 0.011806782, 0.010971495,
      0.010250170, 0.009620144, 0.009064496, 0.008570304, 0.008127448, 0.007727941, 0.007365507, 0.007035210,
      0.006733151},
-    {0.058383518, 0.057710540, 0.055814263, 0.052950333, 0.049426834, 0.045585682, 0.041733503, 0.038081219,
-     0.034752018, 0.031795009, 0.029204034, 0.026945855, 0.024977816, 0.023256849, 0.021744350, 0.020407711,
-     0.019219880, 0.018158527, 0.017205261, 0.016344867, 0.015564698, 0.014854215, 0.014204612, 0.013608474,
-     0.013059525}};
+    {0.058368451, 0.057700866, 0.055811053, 0.052949791, 0.049430216, 0.045591886, 0.041738681, 0.038084725,
+     0.034754085, 0.031795648, 0.029204022, 0.026945810, 0.024977833, 0.023256868, 0.021744354, 0.020407704,
+     0.019219873, 0.018158529, 0.017205266, 0.016344867, 0.015564695, 0.014854215, 0.014204614, 0.013608474,
+     0.013059524}};
   static const double six[2][kPairKnots] = {
     {0.035868804, 0.035554658, 0.034637362, 0.033188571, 0.031316283, 0.029150271, 0.026825876, 0.024469031,
      0.022184819, 0.020050849, 0.018115583, 0.016400845, 0.014907102, 0.013619957, 0.012516480, 0.011570452,
@@ -129,13 +134,13 @@ __host__ __device__ inline void pair_functions(const PairMobility& P, double r, 
 
 // What the diagonal is raised by.  The smallest eigenvalues are those of
 // motions that the kernel averages away, next to zero; splines, the step of
-// the digits and the correction above move them by less than 8e-6 (cubes of
-// up to 11^3 blobs at 0.9 to 1.5 h, plates, slabs, rods, 1200 blobs at random in
-// boxes of 6 to 20 h, packed shells), a quarter of the shift.  A blob with more
-// than 32 others (itself included) within 2 h is raised by that much more:
-// such a cluster's largest eigenvalue grows with its blobs, and with it the
-// rounding of the FP32 inverse (512 blobs at random within h / 20: largest
-// eigenvalue 30, smallest pivot 3e-3; 4.8e-4 with the six-point kernel).
+// the digits and the changes above move them by less than 1e-5, over cubes of up
+// to 11^3 blobs at 0.9 to 1.5 h, plates, slabs, rods, 1200 blobs at random in boxes
+// of 6 to 20 h, packed shells: a third of the six-point kernel's shift, a
+// twentieth of the other's.  A blob with more than 32 others (itself included)
+// within 2 h is raised by that much more: both that and the rounding of the FP32
+// inverse grow with the blobs of a cluster (400 at random within h / 5: 2e-5 below
+// zero at most, raised by 2.5e-3).
 constexpr double kPairNear = 2.0;
 __host__ __device__ inline double pair_raise(const PairMobility& P, int near) {
   return P.shift * (near > 32 ? near / 32.0 : 1.0);
