@@ -132,7 +132,8 @@ const char* rbfib_last_error(const rbfib_grid* g);   /* g may be NULL */
  * no blob, or whose blobs lie on one line (its rotation about that line
  * would be undetermined: fewer than three non-collinear blobs).  Two blobs at
  * one place, whose forces cannot be told apart: EINVAL, or EINTERNAL from the
- * coupled body block. */
+ * coupled body block.  After EINVAL the grid is as it was, after another
+ * failure it may be left without bodies (rbfib_saddle_layout tells). */
 int rbfib_set_bodies(rbfib_grid* g, int32_t n_bodies, const int32_t* blob_offsets,
                      const double* ref_blobs, const double* q, const double* quat);
 
@@ -153,7 +154,7 @@ int rbfib_apply_saddle(rbfib_grid* g, const void* x, void* y, int32_t dtype);
  * multiple of the projection's potential, for the drag of no-slip walls)
  * and, for the bodies, the Schur complement with the blob mobility replaced
  * by the kernel's free-space blob mobility.  r, z: device FP64 saddle
- * vectors; computed in FP32 internally. */
+ * vectors; computed in FP32 internally but for the rows of U. */
 int rbfib_apply_preconditioner(rbfib_grid* g, const double* r, double* z);
 
 /* Solve the constrained system (Eqs. LangevinD1-D4) with forces/torques FT
